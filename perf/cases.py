@@ -155,7 +155,8 @@ def _stable_dt(p, U, xyz):
     ub = math.sqrt(6.0) * U[..., 0]
     u = torch.linalg.norm(ub[:, 1:4], dim=1) / ub[:, 0]
     c = torch.sqrt(GAMMA * (GAMMA - 1) * (ub[:, 4] - 0.5 * ub[:, 0] * u * u) / ub[:, 0])
-    vol = torch.linalg.det(xyz[:, 1:] - xyz[:, :1]).abs() / 6
+    a, b, d = (xyz[:, 1:] - xyz[:, :1]).unbind(1)
+    vol = (torch.linalg.cross(a, b) * d).sum(1).abs() / 6
     area = torch.stack([torch.linalg.norm(torch.linalg.cross(xyz[:, v[1]] - xyz[:, v[0]], xyz[:, v[2]] - xyz[:, v[0]]), dim=1) / 2
                         for v in FV]).amax(0)
     return CFL * float((3 * vol / area / ((2 * p + 1) * (u + c))).min())
