@@ -81,7 +81,6 @@ void free_mesh(dg_mesh* m) {
     cudaFree(m->d_ncan);
     cudaFree(m->d_flist);
     cudaFree(m->d_T);
-    cudaFree(m->d_Hs);
     if (m->rk_exec) cudaGraphExecDestroy(m->rk_exec);
     if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
     cudaFree(m->d_red);

@@ -93,8 +93,8 @@ struct dg_mesh {
     double* d_farea = nullptr;
     // one evaluation per face (FP64): per slot the owner flag and the owner's outward normal
     // (host copies kept for partitions), the list of slots whose face flux this mesh evaluates,
-    // the number of elements with traces (own + halo on a partition's mesh), and the trace and
-    // face-flux buffers [n_trace][4][Nqf][5] (lazy)
+    // (boundary faces last), the number of elements with traces (own + halo on a partition's mesh),
+    // and the face buffer [n_trace][4][5][Nqf] (traces, then the fluxes in their place)
     bool face_once = false;
     std::vector<uint8_t> h_fown;
     std::vector<double> h_ncan;
@@ -103,7 +103,6 @@ struct dg_mesh {
     int32_t* d_flist = nullptr;
     int64_t n_flist = 0, n_trace = 0;
     void* d_T = nullptr;
-    void* d_Hs = nullptr;
     // small meshes: a CUDA graph of several captured RK3 steps at one dt (dg_rk3_step)
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t rk_exec = nullptr;

@@ -159,7 +159,6 @@ void free_sub(dg_mesh* s) {
     cudaFree(s->d_ncan);
     cudaFree(s->d_flist);
     cudaFree(s->d_T);
-    cudaFree(s->d_Hs);
     delete s;
 }
 
