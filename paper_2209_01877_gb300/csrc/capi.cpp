@@ -1,5 +1,6 @@
 // C ABI entry points (include/dg.h): argument checks, device buffers, and
 // the sequencing of kernel launches on the caller's stream.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -77,9 +78,12 @@ void free_mesh(dg_mesh* m) {
     cudaFree(m->d_hs);
     cudaFree(m->d_wslot);
     cudaFree(m->d_farea);
-    cudaFree(m->d_fown);
-    cudaFree(m->d_ncan);
-    cudaFree(m->d_flist);
+    cudaFree(m->d_frec);
+    cudaFree(m->d_fnorm);
+    if (m->d_TW != m->d_T) cudaFree(m->d_TW);
+    if (m->d_TA != m->d_T) cudaFree(m->d_TA);
+    cudaFree(m->d_TL);
+    cudaFree(m->d_fscale);
     cudaFree(m->d_T);
     if (m->rk_exec) cudaGraphExecDestroy(m->rk_exec);
     if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
@@ -98,12 +102,32 @@ dg_status ensure_work_buffers(dg_mesh* m) {
     return DG_OK;
 }
 
+// a buffer of the face-once form, allocated on first use; left null on an FP32 mesh without room for
+// it, which then runs the kernels that need none
+dg_status ensure_face_buffer(dg_mesh* m, void*& buf, size_t bytes) {
+    if (!m->face_once || buf) return DG_OK;
+    const cudaError_t e = cudaMalloc(&buf, bytes);
+    if (e == cudaSuccess) return DG_OK;
+    buf = nullptr;
+    if (m->precision == DG_FP64 || e != cudaErrorMemoryAllocation) return cuda_fail(e, "cudaMalloc(face buffer)");
+    (void)cudaGetLastError();
+    return DG_OK;
+}
+
+// the buffers of the calls that leave a residual in d_W
+dg_status ensure_residual_buffers(dg_mesh* m) {
+    const dg_status st = ensure_work_buffers(m);
+    if (st != DG_OK || m->precision == DG_FP64) return st;
+    return ensure_face_buffer(m, m->d_TW, m->face_bytes());
+}
+
 }  // namespace
 
 namespace dg {
 dg_status set_error(dg_status code, const char* msg) { return fail(code, msg); }
 }  // namespace dg
 
+size_t dg_mesh::face_bytes() const { return (size_t)n_trace * 20 * nqf * (precision == DG_FP64 ? 8 : 4); }
 size_t dg_mesh::state_bytes() const { return (size_t)host.ne * 5 * nb * real_size(precision); }
 
 extern "C" {
@@ -198,11 +222,25 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
         DG_TRY(upload(&m->d_mhdr, cnt.data(), cnt.size(), s));
         DG_TRY(upload(&m->d_mxnbr, xnbr.data(), xnbr.size(), s));
     }
-    if (m->precision == DG_FP64) {
-        // every face's traces and flux once (owner flags, canonical normals, trace and flux buffers)
-        dg::build_face_owners(m->host, m->h_fown, m->h_ncan);
-        cudaError_t e = dg::setup_face_once(m, m->h_fown, m->h_ncan, m->host.ne, s);
-        if (e != cudaSuccess) { free_mesh(m); return cuda_fail(e, "face buffers"); }
+    if (!is_mixed(m)) {
+        // every face's traces and flux once; an FP32 mesh without room for the face buffer runs the
+        // kernel that needs none
+        std::vector<dg::FaceRec> rec;
+        std::vector<int32_t> owner;
+        dg::build_face_list(m->host, m->host, 0, rec, owner);
+        cudaError_t e = dg::setup_face_once(m, rec, owner, m->d_jinv64, m->host.ne, s);
+        if (e == cudaErrorMemoryAllocation && m->precision == DG_FP32) {
+            (void)cudaGetLastError();
+            cudaFree(m->d_frec);
+            cudaFree(m->d_fnorm);
+            m->d_frec = nullptr;
+            m->d_fnorm = nullptr;
+            m->d_T = nullptr;
+        } else if (e != cudaSuccess) {
+            free_mesh(m);
+            return cuda_fail(e, "face buffers");
+        }
+        if (m->precision == DG_FP64) m->d_TW = m->d_TA = m->d_T;
     }
     if (m->precision == DG_FP64) {
         m->d_tab = m->d_tab64;   // shared; freed once below
@@ -359,7 +397,7 @@ dg_status dg_get_state(const dg_mesh* mc, double* U, int on_device, void* stream
 dg_status dg_residual(dg_mesh* m, const double* U, double* R, void* stream) {
     if (!m || !R) return fail(DG_ERR_ARG, "mesh and R must be non-NULL");
     if (!U && !m->has_state) return fail(DG_ERR_NOSTATE, "no state set and U is NULL");
-    dg_status st = ensure_work_buffers(m);
+    dg_status st = ensure_residual_buffers(m);
     if (st != DG_OK) return st;
     cudaStream_t s = as_stream(stream);
     const void* in = m->d_B[0];
@@ -374,7 +412,7 @@ dg_status dg_residual(dg_mesh* m, const double* U, double* R, void* stream) {
         DG_CUDA(dg::launch_scatter_f32(m, out, R, s));
         return DG_OK;
     }
-    DG_CUDA(dg::launch_residual(m, in, nullptr, m->d_W[1], 0, 0.0, 0.0, 0.0, s));
+    DG_CUDA(dg::launch_residual(m, in, nullptr, m->d_W[1], 0, 0.0, 0.0, 0.0, m->d_TW, s));
     DG_CUDA(dg::launch_scatter(m, m->d_W[1], R, s));
     return DG_OK;
 }
@@ -386,7 +424,7 @@ cudaError_t euler_residual_internal(dg_mesh* m, const void* in, void* R, cudaStr
     if (is_mixed(m))
         return dg::launch_residual_mixed(m, static_cast<const float*>(in), nullptr, nullptr, nullptr,
                                          static_cast<float*>(R), nullptr, 0, 0.0, 0.0, 0.0, s);
-    return dg::launch_residual(m, in, nullptr, R, 0, 0.0, 0.0, 0.0, s);
+    return dg::launch_residual(m, in, nullptr, R, 0, 0.0, 0.0, 0.0, m->d_TW, s);
 }
 
 dg_status ensure_ns_buffers(dg_mesh* m) {
@@ -401,7 +439,7 @@ dg_status dg_ns_residual(dg_mesh* m, const double* U, double* R, double mu, doub
     if (!m || !R) return fail(DG_ERR_ARG, "mesh and R must be non-NULL");
     if (!(mu >= 0.0) || !(prandtl > 0.0)) return fail(DG_ERR_ARG, "mu must be >= 0 and prandtl > 0");
     if (!U && !m->has_state) return fail(DG_ERR_NOSTATE, "no state set and U is NULL");
-    dg_status st = ensure_work_buffers(m);
+    dg_status st = ensure_residual_buffers(m);
     if (st != DG_OK) return st;
     cudaStream_t s = as_stream(stream);
     const void* in = m->d_B[0];
@@ -480,7 +518,7 @@ dg_status dg_set_conservative(dg_mesh* m, int enable) {
 namespace {
 // one fused residual + RK stage: out = a U0 + b (U + dt R(U))
 cudaError_t stage_launch(dg_mesh* m, void* U, void* U0, void* out, double dt, double a, double b, cudaStream_t s) {
-    if (!is_mixed(m)) return dg::launch_residual(m, U, U0, out, 1, dt, a, b, s);
+    if (!is_mixed(m)) return dg::launch_residual(m, U, U0, out, 1, dt, a, b, m->d_T, s);
     const size_t n = (size_t)m->host.ne * 5 * m->nb;
     float* u = static_cast<float*>(U);
     float* u0 = static_cast<float*>(U0);
@@ -575,7 +613,7 @@ dg_status dg_ns_rk3_step(dg_mesh* m, double dt, int nsteps, double mu, double pr
     if (nsteps == 0) return DG_OK;
     if (!m->has_state) return fail(DG_ERR_NOSTATE, "no state set");
     if (!(dt >= 0.0)) return fail(DG_ERR_ARG, "dt must be >= 0");
-    dg_status st = ensure_work_buffers(m);
+    dg_status st = ensure_residual_buffers(m);
     if (st != DG_OK) return st;
     if (mu > 0.0) {
         st = ensure_ns_buffers(m);
@@ -670,10 +708,18 @@ dg_status dg_applied_boundary_flux(dg_mesh* m, double out[5], void* stream) {
 }
 
 namespace {
-dg_status ensure_adjoint_buffers(dg_mesh* m) {
+dg_status ensure_adjoint_buffers(dg_mesh* m, cudaStream_t s) {
     for (auto& b : m->d_V)
         if (!b) DG_CUDA(cudaMalloc(&b, m->state_bytes() + 256));
-    return DG_OK;
+    dg_status st = m->precision == DG_FP64 ? DG_OK : ensure_face_buffer(m, m->d_TA, m->face_bytes());
+    if (st == DG_OK) st = ensure_face_buffer(m, m->d_TL, m->face_bytes());
+    if (st != DG_OK || !m->face_once || m->d_fscale) return st;
+    st = ensure_face_buffer(m, m->d_fscale, (size_t)std::max<int64_t>(m->n_flist, 1) * 2 * (m->precision == DG_FP64 ? 8 : 4));
+    if (st == DG_OK && m->d_fscale) {
+        DG_CUDA(dg::launch_face_scales(m, m->d_fscale, s));
+        DG_CUDA(cudaStreamSynchronize(s));   // once per mesh: later calls may come on other streams
+    }
+    return st;
 }
 }  // namespace
 
@@ -681,7 +727,7 @@ dg_status dg_residual_vjp(dg_mesh* m, const double* U, const double* lambda, dou
     if (!m || !U || !lambda || !out) return fail(DG_ERR_ARG, "mesh, U, lambda and out must be non-NULL");
     if (is_mixed(m)) return fail(DG_ERR_UNSUPPORTED, "the adjoint runs in FP64 or FP32 meshes");
     cudaStream_t s = as_stream(stream);
-    dg_status st = ensure_adjoint_buffers(m);
+    dg_status st = ensure_adjoint_buffers(m, s);
     if (st != DG_OK) return st;
     void** V = m->d_V;
     const double c[4] = {0.0, 0.0, 0.0, 1.0};
@@ -697,13 +743,13 @@ dg_status dg_rk3_step_vjp(dg_mesh* m, const double* U0, double dt, const double*
     if (is_mixed(m)) return fail(DG_ERR_UNSUPPORTED, "the adjoint runs in FP64 or FP32 meshes");
     if (!(dt >= 0.0)) return fail(DG_ERR_ARG, "dt must be >= 0");
     cudaStream_t s = as_stream(stream);
-    dg_status st = ensure_adjoint_buffers(m);
+    dg_status st = ensure_adjoint_buffers(m, s);
     if (st != DG_OK) return st;
     void** V = m->d_V;   // V0 = U0, V1 = lambda, V2 = U1, V3 = U2 (then result), V4 = m2, V5 = m1
     DG_CUDA(dg::launch_gather(m, U0, V[0], s));
     DG_CUDA(dg::launch_gather(m, lambda, V[1], s));
-    DG_CUDA(dg::launch_residual(m, V[0], nullptr, V[2], 1, dt, 0.0, 1.0, s));
-    DG_CUDA(dg::launch_residual(m, V[2], V[0], V[3], 1, dt, 0.75, 0.25, s));
+    DG_CUDA(dg::launch_residual(m, V[0], nullptr, V[2], 1, dt, 0.0, 1.0, m->d_TA, s));
+    DG_CUDA(dg::launch_residual(m, V[2], V[0], V[3], 1, dt, 0.75, 0.25, m->d_TA, s));
     const double c2[4] = {2.0 / 3.0, 0.0, 0.0, 2.0 / 3.0 * dt};   // m2 = 2/3 (lambda + dt J(U2)^T lambda)
     DG_CUDA(dg::launch_residual_vjp(m, V[3], V[1], V[1], nullptr, nullptr, c2, V[4], s));
     const double c1[4] = {0.25, 0.0, 0.0, 0.25 * dt};             // m1 = 1/4 (m2 + dt J(U1)^T m2)

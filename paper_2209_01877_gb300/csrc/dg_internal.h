@@ -43,7 +43,21 @@ struct MeshHost {
 
 bool build_mesh(const int32_t* tet_vid, const double* tet_xyz, const int8_t* bc_tag, int64_t ne,
                 int renumber, MeshHost& out, int& code, std::string& err);
-void build_face_owners(const MeshHost& h, std::vector<uint8_t>& fown, std::vector<double>& ncan);
+
+// A face that a mesh evaluates, from one of its slots 4 e + f (on its owner's side, unless the owner
+// is a halo element of a partition).
+struct FaceRec {
+    int32_t slot;
+    int32_t other;      // the matching slot, or -1 - bc_type
+    int32_t code;       // bits 0-2 the orientation (face-point permutation), bit 3 set if slot owns the face
+    int32_t pad;
+};
+
+// The faces of the elements [first, first + local.ne) of `whole`, whose connectivity in local numbers
+// (own elements, then halo) is `local`; boundary faces last.  owner: each face's owning slot in
+// whole's numbers.
+void build_face_list(const MeshHost& whole, const MeshHost& local, int64_t first, std::vector<FaceRec>& rec,
+                     std::vector<int32_t>& owner);
 
 }  // namespace dg
 
@@ -91,18 +105,19 @@ struct dg_mesh {
     float* d_hs = nullptr;
     double* d_wslot = nullptr;
     double* d_farea = nullptr;
-    // one evaluation per face (FP64): per slot the owner flag and the owner's outward normal
-    // (host copies kept for partitions), the list of slots whose face flux this mesh evaluates,
-    // (boundary faces last), the number of elements with traces (own + halo on a partition's mesh),
-    // and the face buffer [n_trace][4][5][Nqf] (traces, then the fluxes in their place)
+    // one evaluation per face (FP64, FP32): the faces this mesh evaluates (boundary faces last) with
+    // their owners' outward normals, the number of elements with traces (own + halo on a
+    // partition's mesh), and the face buffers [n_trace][4][5][Nqf] (traces, then the fluxes in their
+    // place): d_T of the RK stages; FP32 (lazy): d_TW of the calls that leave a residual in d_W and
+    // d_TA of the adjoint, which stay independent of a step in progress (FP64: both are d_T); d_TL
+    // the adjoint direction's traces, d_fscale Real [n_flist][2] the two sides' |grad lambda| (lazy)
     bool face_once = false;
-    std::vector<uint8_t> h_fown;
-    std::vector<double> h_ncan;
-    uint8_t* d_fown = nullptr;
-    void* d_ncan = nullptr;        // Real [ne][4][3]
-    int32_t* d_flist = nullptr;
-    int64_t n_flist = 0, n_trace = 0;
+    dg::FaceRec* d_frec = nullptr;
+    void* d_fnorm = nullptr;       // Real [n_flist][3]
+    int64_t n_flist = 0, n_interior = 0, n_trace = 0;   // listed faces, interior ones among them
     void* d_T = nullptr;
+    void *d_TW = nullptr, *d_TA = nullptr, *d_TL = nullptr, *d_fscale = nullptr;
+    size_t face_bytes() const;
     // small meshes: a CUDA graph of several captured RK3 steps at one dt (dg_rk3_step)
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t rk_exec = nullptr;
@@ -112,12 +127,17 @@ struct dg_mesh {
 
 // Launchers (kernels.cu).  All return a cudaError_t of the launch.
 namespace dg {
+// T: the face buffer to use (null: the FP32 kernel that needs none)
 cudaError_t launch_residual(dg_mesh* m, const void* U, const void* U0, void* out, int mode,
-                            double dt, double a, double b, cudaStream_t s);
-// the face-once path's device data from per-slot owner flags and normals of the mesh's own
-// elements (n_trace - ne halo elements follow them in the state)
-cudaError_t setup_face_once(dg_mesh* m, const std::vector<uint8_t>& fown, const std::vector<double>& ncan,
-                            int64_t n_trace, cudaStream_t s);
+                            double dt, double a, double b, void* T, cudaStream_t s);
+// the face-once path's device data: the face list, the owners' normals from the whole mesh's J^-1,
+// the face buffer of n_trace elements
+cudaError_t setup_face_once(dg_mesh* m, const std::vector<FaceRec>& rec, const std::vector<int32_t>& owner,
+                            const double* d_jinv64_whole, int64_t n_trace, cudaStream_t s);
+// face traces of two states of the mesh's precision, into the face buffers T and T1
+cudaError_t launch_traces2(dg_mesh* m, const void* U, void* T, const void* U1, void* T1, cudaStream_t s);
+// per listed face |grad lambda| of its slot and of the matching one, Real [n_flist][2]
+cudaError_t launch_face_scales(dg_mesh* m, void* out, cudaStream_t s);
 cudaError_t launch_gather(dg_mesh* m, const double* user, void* internal, cudaStream_t s);   // caller -> internal
 // Navier-Stokes lines: the BR1 gradient into Z, then the viscous volume and face terms added to
 // the residual R (internal order), in the mesh's arithmetic (FP64 meshes FP64; FP32 and mixed

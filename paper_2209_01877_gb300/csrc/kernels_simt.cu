@@ -19,19 +19,26 @@
 // buffer (written and read twice per stage, 4 Nqf 5 values per element) and of the states.
 // Measured, one SSP-RK3 step between set and get of the state, dense operators and one thread per
 // point before -> factored operators: FP64 P3 Roe, 196,608 elements 27.7 -> 17.1 ms; FP64 P1 Rusanov,
-// 1,296 elements 85 -> 62 us.
+// 1,296 elements 85 -> 62 us; FP32 P2 Rusanov, 663,552 elements, per stage 980 us (one kernel, each face
+// from both sides) -> 65 + 151 + 126 us.
 #include <algorithm>
 
 #include "dg_internal.h"
 #include "euler_device.cuh"
 #include "face_flux.cuh"
 #include "modal_ops.cuh"
+#include "tc_ops.cuh"
 
 namespace dg {
 
 namespace {
 
 constexpr int NT = 256;
+
+// ---- FP32 without a face buffer ------------------------------------------------------------------
+// One persistent kernel per residual that evaluates every face from both sides; used only where the
+// face buffer (80 Nqf bytes per element) cannot be allocated: a P2 stage takes twice the time of the
+// face-once form below.
 
 template <int P> struct Tile;
 template <> struct Tile<1> { static constexpr int EPB = 32; };
@@ -253,87 +260,59 @@ cudaError_t dispatch_flux(const ResArgs<Real>& args, int flux, bool rk, cudaStre
 
 // ---- face-once form -----------------------------------------------------------------------------
 
-// the values of one contiguous row, in the widest accesses its alignment allows
-template <int N, typename Real>
-__device__ __forceinline__ void load_row(const Real* __restrict__ p, Real* x) {
-    constexpr int B = N * (int)sizeof(Real);
-    if constexpr (B % 16 == 0) {
-        constexpr int V = 16 / sizeof(Real);
-#pragma unroll
-        for (int i = 0; i < N / V; ++i) {
-            const float4 t = reinterpret_cast<const float4*>(p)[i];
-            const Real* r = reinterpret_cast<const Real*>(&t);
-#pragma unroll
-            for (int k = 0; k < V; ++k) x[i * V + k] = r[k];
-        }
-    } else if constexpr (B % 8 == 0) {
-        constexpr int V = 8 / sizeof(Real);
-#pragma unroll
-        for (int i = 0; i < N / V; ++i) {
-            const float2 t = reinterpret_cast<const float2*>(p)[i];
-            const Real* r = reinterpret_cast<const Real*>(&t);
-#pragma unroll
-            for (int k = 0; k < V; ++k) x[i * V + k] = r[k];
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < N; ++i) x[i] = p[i];
-    }
-}
-template <int N, typename Real>
-__device__ __forceinline__ void store_row(Real* p, const Real* x) {
-    constexpr int B = N * (int)sizeof(Real);
-    if constexpr (B % 16 == 0) {
-        constexpr int V = 16 / sizeof(Real);
-#pragma unroll
-        for (int i = 0; i < N / V; ++i) {
-            float4 t;
-            Real* r = reinterpret_cast<Real*>(&t);
-#pragma unroll
-            for (int k = 0; k < V; ++k) r[k] = x[i * V + k];
-            reinterpret_cast<float4*>(p)[i] = t;
-        }
-    } else if constexpr (B % 8 == 0) {
-        constexpr int V = 8 / sizeof(Real);
-#pragma unroll
-        for (int i = 0; i < N / V; ++i) {
-            float2 t;
-            Real* r = reinterpret_cast<Real*>(&t);
-#pragma unroll
-            for (int k = 0; k < V; ++k) r[k] = x[i * V + k];
-            reinterpret_cast<float2*>(p)[i] = t;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < N; ++i) p[i] = x[i];
-    }
-}
+constexpr int FT = 128;       // threads of k_faces
 
-constexpr int TT = 128;   // threads of k_traces
-constexpr int FT = 128;   // threads of k_faces
-
-// the trace of every (element, face, point): thread per (element, variable) row
+// The trace of every (element, face, point) of one or (gridDim.y = 2) two states: thread per (element,
+// variable) row.  In FP32 the tile's
+// coefficients and traces pass through shared memory, so that the global accesses are whole lines:
+// rows written directly (24 to 48 bytes each) kept the load-store unit busy (P2, 663,552 elements:
+// 127 us at 39 % of the DRAM rate).  FP64 is bound by its pipe and writes its rows directly.
 template <typename Real, int P>
-__global__ void __launch_bounds__(TT) k_traces(const Real* __restrict__ U, Real* __restrict__ T, int64_t nrow) {
+__global__ void __launch_bounds__(ER, sizeof(Real) == 8 ? (P == 3 ? 3 : P == 2 ? 6 : 10) : (P == 3 ? 5 : 10))
+    k_traces(const Real* U0, Real* T0, const Real* U1, Real* T1, int64_t ne) {
     constexpr int NB = nb_of(P), NQF = nqf_of(P);
-    const int64_t row = blockIdx.x * (int64_t)TT + threadIdx.x;
-    if (row >= nrow) return;
-    const int64_t e = row / 5;
-    const int v = (int)(row - 5 * e);
-    Real c[NB];
-    load_row<NB>(U + row * NB, c);
-    Real* t = T + (e * 20 + v) * NQF;
-    modal::traces<Real, P>(c, [&](int f, const Real* u) { store_row<NQF>(t + f * 5 * NQF, u); });
+    const Real* __restrict__ U = blockIdx.y == 0 ? U0 : U1;
+    Real* __restrict__ T = blockIdx.y == 0 ? T0 : T1;
+    const int t = threadIdx.x;
+    const int64_t e0 = blockIdx.x * (int64_t)EE;
+    const int nel = (ne - e0) < (int64_t)EE ? (int)(ne - e0) : EE;
+    const int e = t / 5, v = t - 5 * e;
+    if constexpr (sizeof(Real) == 8) {
+        if (t >= 5 * nel) return;
+        Real c[NB];
+        load_row<NB>(U + (e0 * 5 + t) * NB, c);
+        Real* o = T + ((e0 + e) * 20 + v) * NQF;
+        modal::traces<Real, P>(c, [&](int f, const Real* u) { store_row<NQF>(o + f * 5 * NQF, u); });
+    } else {
+        __shared__ __align__(16) Real sU[ER * NB], sT[EE * 20 * NQF];
+        copy_tile(sU, U + e0 * 5 * NB, nel * 5 * NB * (int)sizeof(Real));
+        tc::cp_async_wait_all();
+        __syncthreads();
+        if (t < 5 * nel) {
+            Real c[NB];
+            load_row<NB>(sU + t * NB, c);
+            Real* o = sT + (e * 20 + v) * NQF;
+            modal::traces<Real, P>(c, [&](int f, const Real* u) { store_row<NQF>(o + f * 5 * NQF, u); });
+        }
+        __syncthreads();
+        float4* g = reinterpret_cast<float4*>(T + e0 * 20 * NQF);
+        for (int i = t; i < nel * 5 * NQF; i += ER) g[i] = reinterpret_cast<const float4*>(sT)[i];
+    }
+}
+
+template <typename Real, int P>
+cudaError_t traces(const void* U, void* T, const void* U1, void* T1, int64_t ne, cudaStream_t s) {
+    const dim3 grid((unsigned)((ne + EE - 1) / EE), U1 ? 2 : 1);
+    k_traces<Real, P><<<grid, ER, 0, s>>>(static_cast<const Real*>(U), static_cast<Real*>(T), static_cast<const Real*>(U1),
+                                          static_cast<Real*>(T1), ne);
+    return cudaGetLastError();
 }
 
 template <typename Real>
 struct FaceArgs {
     Real* T;                // face buffer [n_trace][4][5][Nqf]: traces in, fluxes out
-    const Real* ncan;       // [ne][4][3] the owner's outward normal
-    const uint8_t* fown;    // [ne][4] 1 where the slot's element owns the face
-    const int32_t* flist;   // slots 4 e + f whose face this mesh evaluates, boundary faces last
-    const int32_t* nbr;
-    const uint8_t* fcode;
+    const FaceRec* rec;
+    const Real* normal;     // [faces][3] the owner's outward normal
     const int8_t* fperm;
     int64_t n;              // listed faces x Nqf
     Real gamma, roe_eps;
@@ -350,17 +329,17 @@ __global__ void __launch_bounds__(FT) k_faces(FaceArgs<Real> a) {
     if (i >= a.n) return;
     const int64_t li = i / NQF;
     const int q = (int)(i - li * NQF);
-    const int64_t slot = a.flist[li];
-    const Real* nc = a.ncan + slot * 3;
+    const int4 f = *reinterpret_cast<const int4*>(a.rec + li);   // slot, other, code
+    const Real* nc = a.normal + li * 3;
     const Real nv[3] = {nc[0], nc[1], nc[2]};
+    const int64_t slot = f.x;
     Real* te = a.T + slot * 5 * NQF + q;
     Real Ue[5], Un[5], H[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) Ue[v] = te[v * NQF];
-    const int32_t n = a.nbr[slot];
     bool okL, okR;
-    if (n < 0) {
-        if (n == -1 - DG_BC_WALL) wall_ghost(Ue, nv, Un);
+    if (f.y < 0) {
+        if (f.y == -1 - DG_BC_WALL) wall_ghost(Ue, nv, Un);
         else farfield_ghost(Ue, nv, a.finf, a.gamma, Un);
         face_flux<Real, FLUX>(Ue, Un, nv, a.gamma, a.roe_eps, H, okL, okR);
         if (!okL) atomicOr(a.status, 1u);
@@ -368,12 +347,11 @@ __global__ void __launch_bounds__(FT) k_faces(FaceArgs<Real> a) {
         for (int v = 0; v < 5; ++v) te[v * NQF] = H[v];
         return;
     }
-    const int code = a.fcode[slot];
-    const int qn = a.fperm[(code >> 2) * NQF + q];
-    Real* tn = a.T + ((int64_t)n * 4 + (code & 3)) * 5 * NQF + qn;
+    const int qn = a.fperm[(f.z & 7) * NQF + q];
+    Real* tn = a.T + (int64_t)f.y * 5 * NQF + qn;
 #pragma unroll
     for (int v = 0; v < 5; ++v) Un[v] = tn[v * NQF];
-    const bool own = a.fown[slot] != 0;   // false only for a face shared with a halo element that owns it
+    const bool own = (f.z & 8) != 0;   // false only for a face shared with a halo element that owns it
     Real sg = Real(1);
     if (!own) {
         sg = Real(-1);
@@ -394,15 +372,19 @@ __global__ void __launch_bounds__(FT) k_faces(FaceArgs<Real> a) {
     }
 }
 
-constexpr int EE = 32;        // elements per tile of k_element
-constexpr int ER = 5 * EE;    // rows (element, variable) = threads
-
 template <typename Real, int P>
 struct ElemPlan {
-    static constexpr int NQ = nq_of(P);
-    // shared memory (Reals): point states [NQ][ER], (W_0, W_1, W_2, p) [NQ][EE][4], J^-1 [EE][9],
-    // |grad lambda_f| [EE][4]
-    static constexpr int W = NQ * ER, J = W + NQ * EE * 4, G = J + EE * 9, REALS = G + EE * 4;
+    // FP32 projects the deviation from the flux of the element's mean state, which is point NQ, and
+    // passes its rows through shared memory
+    static constexpr bool F32 = sizeof(Real) == 4;
+    static constexpr int NB = nb_of(P), NQ = nq_of(P), NP = NQ + (F32 ? 1 : 0);
+    // shared memory (Reals): point states [NP][ER], (W_0, W_1, W_2, p) [NP][EE][4], then J^-1 [EE][9],
+    // |grad lambda_f| [EE][4]; FP32: the tile's coefficients [ER][NB] (the new ones at the end) and
+    // its face fluxes, which take the place of the point values once those are projected (P3: 5
+    // tiles per SM instead of 2)
+    static constexpr int W = NP * ER, POINTS = W + NP * EE * 4, FACES = F32 ? EE * 20 * nqf_of(P) : 0;
+    static constexpr int J = POINTS > FACES ? POINTS : FACES;
+    static constexpr int G = J + EE * 9, C = G + EE * 4, REALS = C + (F32 ? ER * NB : 0);
     static constexpr size_t BYTES = REALS * sizeof(Real);
 };
 
@@ -415,22 +397,28 @@ __global__ void __launch_bounds__(ER) k_element(ResArgs<Real> a) {
     Real* sW = sU + S::W;
     Real* sJ = sU + S::J;
     Real* sG = sU + S::G;
+    Real* sC = sU + S::C;
     const int t = threadIdx.x;
     const int64_t e0 = blockIdx.x * (int64_t)EE;
     const int nel = (a.ne - e0) < (int64_t)EE ? (int)(a.ne - e0) : EE;
     const bool live = t < 5 * nel;
     const int64_t row = e0 * 5 + t;
+    if (S::F32) {
+        copy_tile(sC, a.U + e0 * 5 * NB, nel * 5 * NB * (int)sizeof(Real));
+    }
     for (int i = t; i < nel * 9; i += ER) sJ[i] = a.jinv[e0 * 9 + i];
+    if (S::F32) {
+        tc::cp_async_wait_all();
+        __syncthreads();
+    }
     if (live) {
-        Real c[NB], u[NQ];
-        load_row<NB>(a.U + row * NB, c);
-        modal::interpolate<Real, P>(c, u);
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) sU[q * ER + t] = u[q];
+        Real c[NB];
+        load_row<NB>(S::F32 ? sC + t * NB : a.U + row * NB, c);
+        modal::interpolate<Real, P, NB>(c, 0, NQ, [&](int q, Real u) { sU[q * ER + t] = u; });
+        if (S::F32) sU[NQ * ER + t] = Real(2.449489742783178) * c[0];
     }
     __syncthreads();
-    // |grad lambda_f| = 2 |S_f| / |det J|, by the threads that the point loop below leaves idle last
-    if (t < nel * 4) {
+    if (t < nel * 4) {   // |grad lambda_f| = 2 |S_f| / |det J|
         const Real* I = sJ + (t >> 2) * 9;
         const int f = t & 3;
         Real g[3];
@@ -439,69 +427,105 @@ __global__ void __launch_bounds__(ER) k_element(ResArgs<Real> a) {
         sG[t] = EulerOps<Real>::sqrt_(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
     }
     // contravariant velocity W_k = sum_d (J^-1)_kd u_d and pressure at every (element, point)
-    for (int i = t; i < NQ * EE; i += ER) {
+    for (int i = t; i < S::NP * EE; i += ER) {
         const int e = i % EE, q = i / EE;
         if (e >= nel) continue;
         const Real* u = sU + q * ER + 5 * e;
         const Real rho = u[0], ri = recip(rho);
         const Real x = u[1] * ri, y = u[2] * ri, z = u[3] * ri;
         const Real p = (a.gamma - Real(1)) * (u[4] - Real(0.5) * (u[1] * x + u[2] * y + u[3] * z));
-        if (!(positive(rho) && positive(p))) atomicOr(a.status, 1u);
+        if (q < NQ && !(positive(rho) && positive(p))) atomicOr(a.status, 1u);
         const Real* I = sJ + e * 9;
-        Real* w = sW + (q * EE + e) * 4;
         Real o[4] = {I[0] * x + I[1] * y + I[2] * z, I[3] * x + I[4] * y + I[5] * z, I[6] * x + I[7] * y + I[8] * z, p};
-        store_row<4>(w, o);
+        store_row<4>(sW + (q * EE + e) * 4, o);
     }
     __syncthreads();
-    if (!live) return;
     const int e = t / 5, v = t - 5 * e;
-    // G_k of variable v: W_k a + p J_k, a = U_v (+ p for the energy), J_k = (J^-1)_k,v-1 for a momentum
+    // G_k of variable v: W_k b + p J_k, b = U_v (+ p for the energy), J_k = (J^-1)_k,v-1 for a momentum
     const Real s4 = v == 4 ? Real(1) : Real(0);
-    Real Jk[3];
+    Real Jk[3], M[3][NM], G0[3] = {0, 0, 0};
 #pragma unroll
-    for (int k = 0; k < 3; ++k) Jk[k] = v >= 1 && v <= 3 ? sJ[e * 9 + 3 * k + v - 1] : Real(0);
-    Real M[3][NM];
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < 3; ++k) {
+        Jk[k] = live && v >= 1 && v <= 3 ? sJ[e * 9 + 3 * k + v - 1] : Real(0);
 #pragma unroll
         for (int m = 0; m < NM; ++m) M[k][m] = 0;
+    }
     auto flux = [&](int q, Real* g) {
         Real w[4];
         load_row<4>(sW + (q * EE + e) * 4, w);
         const Real b = sU[q * ER + t] + s4 * w[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) g[k] = w[k] * b + w[3] * Jk[k];
+        for (int k = 0; k < 3; ++k) g[k] = w[k] * b + (w[3] * Jk[k] - G0[k]);
     };
+    if (live) {
+        if (S::F32) flux(NQ, G0);
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int m = modal::kT<P>.vmir[q];
-        if (m < q) continue;
-        Real g[3], gm[3] = {0, 0, 0};
-        flux(q, g);
-        if (m != q) flux(m, gm);
+        for (int q = 0; q < NQ; ++q) {
+            const int m = modal::kT<P>.vmir[q];
+            if (m < q) continue;
+            Real g[3], gm[3] = {0, 0, 0};
+            flux(q, g);
+            if (m != q) flux(m, gm);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) modal::moments<Real, P, NM>(q, g[k], gm[k], M[k]);
-    }
-    Real r[NB];
-#pragma unroll
-    for (int j = 0; j < NB; ++j) r[j] = 0;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) modal::grad_transposed<Real, P>(k, M[k], r);
-    const Real s[4] = {-sG[4 * e], -sG[4 * e + 1], -sG[4 * e + 2], -sG[4 * e + 3]};
-    const Real* h = a.Hs + ((e0 + e) * 20 + v) * NQF;
-    modal::lift<Real, P>([&](int f, Real* x) { load_row<NQF>(h + f * 5 * NQF, x); }, s, r);
-    if (RK) {
-        Real c[NB];
-        load_row<NB>(a.U + row * NB, c);
-#pragma unroll
-        for (int j = 0; j < NB; ++j) r[j] = a.b * (c[j] + a.dt * r[j]);
-        if (a.a != Real(0)) {
-            load_row<NB>(a.U0 + row * NB, c);
-#pragma unroll
-            for (int j = 0; j < NB; ++j) r[j] += a.a * c[j];
+            for (int k = 0; k < 3; ++k) modal::moments<Real, P, NM>(q, g[k], gm[k], M[k]);
         }
     }
-    store_row<NB>(a.out + row * NB, r);
+    if (S::F32) {
+        __syncthreads();
+        copy_tile(sU, a.Hs + e0 * 20 * NQF, nel * 20 * NQF * (int)sizeof(Real));
+        tc::cp_async_wait_all();
+        __syncthreads();
+    }
+    if (live) {
+        Real r[NB];
+#pragma unroll
+        for (int j = 0; j < NB; ++j) r[j] = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) modal::grad_transposed<Real, P>(k, M[k], r);
+        // the lift of -s_f H; a constant flux F has s_f F.n_f = -grad lambda_f . F = -G_f-1 (f = 0:
+        // the sum of the three), so its part cancels that of the volume term
+        const Real* h = (S::F32 ? sU + e * 20 * NQF : a.Hs + (e0 + e) * 20 * NQF) + v * NQF;
+        modal::lift<Real, P>(
+            [&](int f, Real* x) {
+                load_row<NQF>(h + f * 5 * NQF, x);
+                const Real s = -sG[4 * e + f];
+                if (!S::F32) return s;
+                const Real g = f == 0 ? G0[0] + G0[1] + G0[2] : -G0[f - 1];
+#pragma unroll
+                for (int q = 0; q < NQF; ++q) x[q] = s * x[q] + g;
+                return Real(1);
+            },
+            r);
+        if (RK) {
+            Real c[NB];
+            load_row<NB>(S::F32 ? sC + t * NB : a.U + row * NB, c);
+#pragma unroll
+            for (int j = 0; j < NB; ++j) r[j] = a.b * (c[j] + a.dt * r[j]);
+            if (!S::F32 && a.a != Real(0)) {
+                load_row<NB>(a.U0 + row * NB, c);
+#pragma unroll
+                for (int j = 0; j < NB; ++j) r[j] += a.a * c[j];
+            }
+        }
+        store_row<NB>(S::F32 ? sC + t * NB : a.out + row * NB, r);
+    }
+    if constexpr (S::F32) {   // whole lines: out = the tile (+ a U0)
+        __syncthreads();
+        const int n = nel * 5 * NB;
+        for (int i = 4 * t; i < n; i += 4 * ER) {
+            float4 x = *reinterpret_cast<const float4*>(sC + i);
+            const int64_t g = e0 * 5 * NB + i;
+            if (i + 4 <= n) {
+                if (RK && a.a != 0.f) {
+                    const float4 y = *reinterpret_cast<const float4*>(a.U0 + g);
+                    x = make_float4(x.x + a.a * y.x, x.y + a.a * y.y, x.z + a.a * y.z, x.w + a.a * y.w);
+                }
+                *reinterpret_cast<float4*>(a.out + g) = x;
+            } else {   // P2: an odd number of elements leaves two values
+                for (int k = 0; i + k < n; ++k) a.out[g + k] = sC[i + k] + (RK && a.a != 0.f ? a.a * a.U0[g + k] : 0.f);
+            }
+        }
+    }
 }
 
 template <typename Real, int P, bool RK>
@@ -519,23 +543,18 @@ cudaError_t launch_element(const ResArgs<Real>& r, cudaStream_t s) {
 }
 
 template <typename Real, int P>
-cudaError_t launch_face_once(dg_mesh* m, ResArgs<Real>& r, bool rk, cudaStream_t s) {
+cudaError_t launch_face_once(dg_mesh* m, ResArgs<Real>& r, bool rk, void* T, cudaStream_t s) {
     FaceArgs<Real> f;
-    f.T = static_cast<Real*>(m->d_T);
-    f.ncan = static_cast<const Real*>(m->d_ncan);
-    f.fown = m->d_fown;
-    f.flist = m->d_flist;
-    f.nbr = m->d_nbr;
-    f.fcode = m->d_fcode;
+    f.T = static_cast<Real*>(T);
+    f.rec = m->d_frec;
+    f.normal = static_cast<const Real*>(m->d_fnorm);
     f.fperm = m->d_fperm;
     f.n = m->n_flist * nqf_of(P);
     f.gamma = r.gamma;
     f.roe_eps = r.roe_eps;
     for (int v = 0; v < 5; ++v) f.finf[v] = r.finf[v];
     f.status = m->d_status;
-    const int64_t nrow = 5 * m->n_trace;
-    k_traces<Real, P><<<(unsigned)((nrow + TT - 1) / TT), TT, 0, s>>>(r.U, f.T, nrow);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = traces<Real, P>(r.U, f.T, nullptr, nullptr, m->n_trace, s);
     if (e != cudaSuccess) return e;
     if (f.n > 0) {
         const unsigned grid = (unsigned)((f.n + FT - 1) / FT);
@@ -550,7 +569,7 @@ cudaError_t launch_face_once(dg_mesh* m, ResArgs<Real>& r, bool rk, cudaStream_t
 
 template <typename Real>
 cudaError_t dispatch(dg_mesh* m, const void* U, const void* U0, void* out, int mode, double dt, double ca,
-                     double cb, cudaStream_t s) {
+                     double cb, void* T, cudaStream_t s) {
     ResArgs<Real> r;
     r.U = static_cast<const Real*>(U);
     r.U0 = static_cast<const Real*>(U0);
@@ -570,15 +589,15 @@ cudaError_t dispatch(dg_mesh* m, const void* U, const void* U0, void* out, int m
     r.status = m->d_status;
     r.Hs = nullptr;
     const bool rk = mode != 0;
-    if (m->face_once) {
+    if (T) {
         switch (m->p) {
-            case 1: return launch_face_once<Real, 1>(m, r, rk, s);
-            case 2: return launch_face_once<Real, 2>(m, r, rk, s);
-            default: return launch_face_once<Real, 3>(m, r, rk, s);
+            case 1: return launch_face_once<Real, 1>(m, r, rk, T, s);
+            case 2: return launch_face_once<Real, 2>(m, r, rk, T, s);
+            default: return launch_face_once<Real, 3>(m, r, rk, T, s);
         }
     }
     if constexpr (sizeof(Real) == 8) {
-        return cudaErrorInvalidValue;   // FP64 meshes always hold a face buffer
+        return cudaErrorInvalidValue;   // FP64 has no other form
     } else {
         int nsm = 0;
         cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
@@ -593,42 +612,91 @@ cudaError_t dispatch(dg_mesh* m, const void* U, const void* U0, void* out, int m
 
 }  // namespace
 
-cudaError_t setup_face_once(dg_mesh* m, const std::vector<uint8_t>& fown, const std::vector<double>& ncan,
-                            int64_t n_trace, cudaStream_t s) {
-    const int64_t ne = m->host.ne;
-    std::vector<int32_t> list;
-    // owned, or shared with a halo; boundary faces last, so that warps mostly run one kind
-    for (int kind = 0; kind < 2; ++kind)
-        for (int64_t sl = 0; sl < 4 * ne; ++sl)
-            if ((fown[sl] || m->host.nbr[sl] >= ne) && (m->host.nbr[sl] < 0) == (kind == 1)) list.push_back((int32_t)sl);
-    const size_t rbytes = m->precision == DG_FP64 ? sizeof(double) : sizeof(float);
-    std::vector<float> n32;
-    const void* nsrc = ncan.data();
-    if (rbytes == sizeof(float)) {
-        n32.assign(ncan.begin(), ncan.end());
-        nsrc = n32.data();
+namespace {
+// outward unit normals -grad lambda_f / |grad lambda_f| of the listed slots
+template <typename Real>
+__global__ void k_face_normals(const double* __restrict__ jinv, const int32_t* __restrict__ slot, int64_t n, Real* out) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double* I = jinv + (int64_t)(slot[i] >> 2) * 9;
+    const int f = slot[i] & 3;
+    double g[3];
+    for (int d = 0; d < 3; ++d) g[d] = f == 0 ? -(I[d] + I[3 + d] + I[6 + d]) : I[3 * (f - 1) + d];
+    const double gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+    for (int d = 0; d < 3; ++d) out[3 * i + d] = (Real)(-g[d] / gn);
+}
+
+template <typename Real>
+__global__ void k_face_scales(const double* __restrict__ jinv, const FaceRec* __restrict__ rec, int64_t n, Real* out) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    for (int side = 0; side < 2; ++side) {
+        const int32_t sl = side == 0 ? rec[i].slot : rec[i].other;
+        double g[3] = {0, 0, 0};
+        if (sl >= 0) {
+            const double* I = jinv + (int64_t)(sl >> 2) * 9;
+            const int f = sl & 3;
+            for (int d = 0; d < 3; ++d) g[d] = f == 0 ? -(I[d] + I[3 + d] + I[6 + d]) : I[3 * (f - 1) + d];
+        }
+        out[2 * i + side] = (Real)sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
     }
-    cudaError_t e = cudaMalloc(&m->d_fown, fown.size());
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_ncan, ncan.size() * rbytes);
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_flist, std::max<size_t>(list.size(), 1) * sizeof(int32_t));
-    const size_t buf = (size_t)n_trace * 4 * m->nqf * 5 * rbytes;
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_T, buf);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(m->d_fown, fown.data(), fown.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(m->d_ncan, nsrc, ncan.size() * rbytes, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && !list.empty())
-        e = cudaMemcpyAsync(m->d_flist, list.data(), list.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the host vectors go out of scope
-    if (e != cudaSuccess) return e;
-    m->n_flist = (int64_t)list.size();
+}
+}  // namespace
+
+cudaError_t launch_face_scales(dg_mesh* m, void* out, cudaStream_t s) {
+    if (m->n_flist == 0) return cudaSuccess;
+    const unsigned grid = (unsigned)((m->n_flist + 255) / 256);
+    if (m->precision == DG_FP64) k_face_scales<double><<<grid, 256, 0, s>>>(m->d_jinv64, m->d_frec, m->n_flist, static_cast<double*>(out));
+    else k_face_scales<float><<<grid, 256, 0, s>>>(m->d_jinv64, m->d_frec, m->n_flist, static_cast<float*>(out));
+    return cudaGetLastError();
+}
+
+cudaError_t setup_face_once(dg_mesh* m, const std::vector<FaceRec>& rec, const std::vector<int32_t>& owner,
+                            const double* d_jinv64_whole, int64_t n_trace, cudaStream_t s) {
+    const int64_t n = (int64_t)rec.size();
+    m->n_flist = n;
+    m->n_interior = 0;
+    while (m->n_interior < n && rec[m->n_interior].other >= 0) ++m->n_interior;
     m->n_trace = n_trace;
-    m->face_once = true;
-    return cudaSuccess;
+    const size_t nn = std::max<size_t>(rec.size(), 1);
+    int32_t* d_owner = nullptr;
+    cudaError_t e = cudaMalloc(&m->d_frec, nn * sizeof(FaceRec));
+    if (e == cudaSuccess) e = cudaMalloc(&m->d_fnorm, nn * 3 * (m->precision == DG_FP64 ? 8 : 4));
+    if (e == cudaSuccess) e = cudaMalloc(&m->d_T, m->face_bytes());
+    if (e == cudaSuccess) e = cudaMalloc(&d_owner, nn * sizeof(int32_t));
+    if (e == cudaSuccess && n > 0) {
+        e = cudaMemcpyAsync(m->d_frec, rec.data(), rec.size() * sizeof(FaceRec), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d_owner, owner.data(), owner.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
+        const unsigned grid = (unsigned)((n + 255) / 256);
+        if (e == cudaSuccess) {
+            if (m->precision == DG_FP64)
+                k_face_normals<double><<<grid, 256, 0, s>>>(d_jinv64_whole, d_owner, n, static_cast<double*>(m->d_fnorm));
+            else
+                k_face_normals<float><<<grid, 256, 0, s>>>(d_jinv64_whole, d_owner, n, static_cast<float*>(m->d_fnorm));
+            e = cudaGetLastError();
+        }
+        const cudaError_t es = cudaStreamSynchronize(s);   // the host vectors go out of scope
+        if (e == cudaSuccess) e = es;
+    }
+    cudaFree(d_owner);
+    if (e == cudaSuccess) m->face_once = true;
+    return e;
+}
+
+cudaError_t launch_traces2(dg_mesh* m, const void* U, void* T, const void* U1, void* T1, cudaStream_t s) {
+    const int64_t n = m->host.ne;
+    const bool f64 = m->precision == DG_FP64;
+    switch (m->p) {
+        case 1: return f64 ? traces<double, 1>(U, T, U1, T1, n, s) : traces<float, 1>(U, T, U1, T1, n, s);
+        case 2: return f64 ? traces<double, 2>(U, T, U1, T1, n, s) : traces<float, 2>(U, T, U1, T1, n, s);
+        default: return f64 ? traces<double, 3>(U, T, U1, T1, n, s) : traces<float, 3>(U, T, U1, T1, n, s);
+    }
 }
 
 cudaError_t launch_residual(dg_mesh* m, const void* U, const void* U0, void* out, int mode, double dt, double a,
-                            double b, cudaStream_t s) {
-    if (m->precision == DG_FP64) return dispatch<double>(m, U, U0, out, mode, dt, a, b, s);
-    return dispatch<float>(m, U, U0, out, mode, dt, a, b, s);
+                            double b, void* T, cudaStream_t s) {
+    if (m->precision == DG_FP64) return dispatch<double>(m, U, U0, out, mode, dt, a, b, T, s);
+    return dispatch<float>(m, U, U0, out, mode, dt, a, b, T, s);
 }
 
 }  // namespace dg

@@ -21,11 +21,14 @@
 //     swap symmetry); the E_f are sparse, and E_0[m][j] = (-1)^i E_1[m][j] by the swap, so faces 0
 //     and 1 share their sums.
 //
+// Sums over modes start from the highest, so that the mean, the largest term, is added last.
+//
 // D and E are moments taken with the rules themselves (both integrands have degree <= 2p, which
 // the rules integrate exactly); entries that vanish identically are exact zeros and cost nothing.
 #pragma once
 
 #include "dg_device.h"
+#include "tc_ops.cuh"
 
 namespace dg {
 namespace modal {
@@ -235,25 +238,26 @@ __device__ __forceinline__ void axpy(Real& r, double c, Real x) {
     if (c != 0.0) r += (Real)c * x;
 }
 
-// u[q] = sum_j c[j] phi_j(x_q)
-template <typename Real, int P>
-__device__ __forceinline__ void interpolate(const Real* c, Real* u) {
+// values at the volume points q0 .. q1 - 1 (a range closed under the mirror) of a field of the first N
+// modes, store(q, sum_j c[j] phi_j(x_q))
+template <typename Real, int P, int N, typename Store>
+__device__ __forceinline__ void interpolate(const Real* c, int q0, int q1, Store store) {
     constexpr auto& T = kT<P>;
 #pragma unroll
-    for (int q = 0; q < T.NQ; ++q) {
+    for (int q = q0; q < q1; ++q) {
         const int m = T.vmir[q];
         if (m < q) continue;
         Real e = 0, o = 0;
 #pragma unroll
-        for (int j = 0; j < T.NB; ++j) {
+        for (int j = N - 1; j >= 0; --j) {
             if (!T.odd[j]) axpy(e, T.phi[q][j], c[j]);
             else if (m != q) axpy(o, T.phi[q][j], c[j]);
         }
         if (m == q) {
-            u[q] = e;
+            store(q, e);
         } else {
-            u[q] = e + o;
-            u[m] = e - o;
+            store(q, e + o);
+            store(m, e - o);
         }
     }
 }
@@ -304,7 +308,7 @@ __device__ __forceinline__ void face_values(const Real* a, Real* u) {
         if (n < q) continue;
         Real e = 0, o = 0;
 #pragma unroll
-        for (int m = 0; m < T.NF; ++m) {
+        for (int m = T.NF - 1; m >= 0; --m) {
             if (!T.fodd[m]) axpy(e, T.psi[q][m], a[m]);
             else if (n != q) axpy(o, T.psi[q][m], a[m]);
         }
@@ -347,7 +351,7 @@ __device__ __forceinline__ void traces(const Real* c, Store store) {
         for (int m = 0; m < T.NF; ++m) {
             Real e = 0, o = 0;
 #pragma unroll
-            for (int j = 0; j < T.NB; ++j) axpy(T.odd[j] ? o : e, T.E[1][m][j], c[j]);
+            for (int j = T.NB - 1; j >= 0; --j) axpy(T.odd[j] ? o : e, T.E[1][m][j], c[j]);
             a[m] = e - o;
             b[m] = e + o;
         }
@@ -363,27 +367,28 @@ __device__ __forceinline__ void traces(const Real* c, Store store) {
         for (int m = 0; m < T.NF; ++m) {
             a[m] = 0;
 #pragma unroll
-            for (int j = 0; j < T.NB; ++j) axpy(a[m], T.E[f][m][j], c[j]);
+            for (int j = T.NB - 1; j >= 0; --j) axpy(a[m], T.E[f][m][j], c[j]);
         }
         face_values<Real, P>(a, u);
         store(f, u);
     }
 }
 
-// r[j] += sum_f s_f sum_q wf_q h_f(q) phi_j on face f; load(f, h) fills a face's NQF values
+// r[j] += sum_f sum_q wf_q h_f(q) phi_j on face f; load(f, h) fills a face's NQF values and returns
+// a factor of the face, which multiplies its moments
 template <typename Real, int P, typename Load>
-__device__ __forceinline__ void lift(Load load, const Real* s, Real* r) {
+__device__ __forceinline__ void lift(Load load, Real* r) {
     constexpr auto& T = kT<P>;
     Real h[T.NQF];
     {
         Real a[T.NF], b[T.NF];
-        load(0, h);
+        const Real s0 = load(0, h);
         face_moments<Real, P>(h, a);
-        load(1, h);
+        const Real s1 = load(1, h);
         face_moments<Real, P>(h, b);
 #pragma unroll
         for (int m = 0; m < T.NF; ++m) {
-            const Real x = s[0] * a[m], e = s[1] * b[m] + x, o = s[1] * b[m] - x;
+            const Real x = s0 * a[m], e = s1 * b[m] + x, o = s1 * b[m] - x;
 #pragma unroll
             for (int j = 0; j < T.NB; ++j) axpy(r[j], T.E[1][m][j], T.odd[j] ? o : e);
         }
@@ -391,11 +396,11 @@ __device__ __forceinline__ void lift(Load load, const Real* s, Real* r) {
 #pragma unroll
     for (int f = 2; f < 4; ++f) {
         Real a[T.NF];
-        load(f, h);
+        const Real s = load(f, h);
         face_moments<Real, P>(h, a);
 #pragma unroll
         for (int m = 0; m < T.NF; ++m) {
-            const Real x = s[f] * a[m];
+            const Real x = s * a[m];
 #pragma unroll
             for (int j = 0; j < T.NB; ++j) axpy(r[j], T.E[f][m][j], x);
         }
@@ -403,4 +408,74 @@ __device__ __forceinline__ void lift(Load load, const Real* s, Real* r) {
 }
 
 }  // namespace modal
+
+// ---- rows and tiles -------------------------------------------------------------------------------
+
+constexpr int EE = 32;        // elements per tile of the CUDA-core kernels
+constexpr int ER = 5 * EE;    // rows (element, variable) = threads
+
+// n bytes of a tile, global -> shared, by all ER threads (asynchronous, 16 bytes each; n rounded up:
+// the buffers end in slack)
+__device__ __forceinline__ void copy_tile(void* dst, const void* src, int n) {
+    for (int i = threadIdx.x * 16; i < n; i += ER * 16)
+        tc::cp_async16(static_cast<char*>(dst) + i, static_cast<const char*>(src) + i);
+    tc::cp_async_commit();
+}
+
+// the values of one contiguous row, in the widest accesses its alignment allows
+template <int N, typename Real>
+__device__ __forceinline__ void load_row(const Real* __restrict__ p, Real* x) {
+    constexpr int B = N * (int)sizeof(Real);
+    if constexpr (B % 16 == 0) {
+        constexpr int V = 16 / sizeof(Real);
+#pragma unroll
+        for (int i = 0; i < N / V; ++i) {
+            const float4 t = reinterpret_cast<const float4*>(p)[i];
+            const Real* r = reinterpret_cast<const Real*>(&t);
+#pragma unroll
+            for (int k = 0; k < V; ++k) x[i * V + k] = r[k];
+        }
+    } else if constexpr (B % 8 == 0) {
+        constexpr int V = 8 / sizeof(Real);
+#pragma unroll
+        for (int i = 0; i < N / V; ++i) {
+            const float2 t = reinterpret_cast<const float2*>(p)[i];
+            const Real* r = reinterpret_cast<const Real*>(&t);
+#pragma unroll
+            for (int k = 0; k < V; ++k) x[i * V + k] = r[k];
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) x[i] = p[i];
+    }
+}
+template <int N, typename Real>
+__device__ __forceinline__ void store_row(Real* p, const Real* x) {
+    constexpr int B = N * (int)sizeof(Real);
+    if constexpr (B % 16 == 0) {
+        constexpr int V = 16 / sizeof(Real);
+#pragma unroll
+        for (int i = 0; i < N / V; ++i) {
+            float4 t;
+            Real* r = reinterpret_cast<Real*>(&t);
+#pragma unroll
+            for (int k = 0; k < V; ++k) r[k] = x[i * V + k];
+            reinterpret_cast<float4*>(p)[i] = t;
+        }
+    } else if constexpr (B % 8 == 0) {
+        constexpr int V = 8 / sizeof(Real);
+#pragma unroll
+        for (int i = 0; i < N / V; ++i) {
+            float2 t;
+            Real* r = reinterpret_cast<Real*>(&t);
+#pragma unroll
+            for (int k = 0; k < V; ++k) r[k] = x[i * V + k];
+            reinterpret_cast<float2*>(p)[i] = t;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) p[i] = x[i];
+    }
+}
+
 }  // namespace dg

@@ -155,9 +155,8 @@ void free_sub(dg_mesh* s) {
     cudaFree(s->d_jinv);
     cudaFree(s->d_jinv64);
     cudaFree(s->d_red);
-    cudaFree(s->d_fown);
-    cudaFree(s->d_ncan);
-    cudaFree(s->d_flist);
+    cudaFree(s->d_frec);
+    cudaFree(s->d_fnorm);
     cudaFree(s->d_T);
     delete s;
 }
@@ -256,14 +255,14 @@ dg_status dg_partition_create(dg_mesh* m, int k, void* stream, dg_partition** ou
             PTRY(upload_vec(&sm->d_mhdr, hdr, s));
             PTRY(upload_vec(&sm->d_mxnbr, xnbr, s));
         }
-        // face-once form: the parent's owner flags and normals of the own slots; the faces shared
-        // with halo elements are evaluated here too, in their owner's orientation, so every own
-        // element receives the flux the whole mesh would give it
+        // face-once form, with the whole mesh's owners and normals; the faces shared with halo elements
+        // are evaluated here too, in their owner's orientation, so every own element receives the
+        // flux the whole mesh would give it
         if (m->face_once) {
-            const int64_t c = pl.count;
-            std::vector<uint8_t> fo(m->h_fown.begin() + 4 * pl.first, m->h_fown.begin() + 4 * (pl.first + c));
-            std::vector<double> nc(m->h_ncan.begin() + 12 * pl.first, m->h_ncan.begin() + 12 * (pl.first + c));
-            PTRY(dg::setup_face_once(sm, fo, nc, c + (int64_t)pl.halo.size(), s));
+            std::vector<dg::FaceRec> rec;
+            std::vector<int32_t> owner;
+            dg::build_face_list(m->host, sm->host, pl.first, rec, owner);
+            PTRY(dg::setup_face_once(sm, rec, owner, m->d_jinv64, pl.count + (int64_t)pl.halo.size(), s));
         }
         // local state: own then halo blocks (mixed: hi plane of own + halo, then the lo plane)
         const size_t nloc = (size_t)(pl.count + pl.halo.size()) * nv_of(m);
@@ -404,7 +403,7 @@ dg_status dg_partition_residual(dg_partition* P, const double* U, double* R, voi
             e = dg::launch_residual_mixed(sm, static_cast<const float*>(sm->d_B[0]), nullptr, nullptr, nullptr,
                                           static_cast<float*>(sm->d_W[1]), nullptr, 0, 0.0, 0.0, 0.0, s);
         else
-            e = dg::launch_residual(sm, sm->d_B[0], nullptr, sm->d_W[1], 0, 0.0, 0.0, 0.0, s);
+            e = dg::launch_residual(sm, sm->d_B[0], nullptr, sm->d_W[1], 0, 0.0, 0.0, 0.0, sm->d_T, s);
         // the partition's residual into the parent's internal-order residual buffer
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(static_cast<char*>(m->d_W[1]) + P->plan[r].first * nv * es, sm->d_W[1],
