@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(ER) k_element(ResArgs<Real> a) {
     if (live) {
         Real c[NB];
         load_row<NB>(S::F32 ? sC + t * NB : a.U + row * NB, c);
-        modal::interpolate<Real, P, NB>(c, 0, NQ, [&](int q, Real u) { sU[q * ER + t] = u; });
+        modal::interpolate<Real, P, NB, 0, NQ>(c, [&](int q, Real u) { sU[q * ER + t] = u; });
         if (S::F32) sU[NQ * ER + t] = Real(2.449489742783178) * c[0];
     }
     __syncthreads();

@@ -1,33 +1,38 @@
 // Adjoint of the residual: out = (dR/dU)^T lambda (FP64 / FP32, CUDA cores).
-// The paper has no adjoint; this is the reverse of the forward kernel's steps.
-//
-// Element-centric over output elements e.  R_e depends on U_e (volume term,
-// own side of its 4 face fluxes) and on the 4 neighbours (the other side of
-// those fluxes); U_e also enters each neighbour's residual through the shared
-// face.  Per tile, with the basis tables in shared memory:
-//   faces   thread per (element, face, point): the own face flux
-//           H(U-, U+, n_e) differentiated w.r.t. U- (dual numbers, 5
-//           directions; through the ghost state on boundary faces), and the
-//           neighbour's flux H(U+, U-, n_n) at the same physical point
-//           differentiated w.r.t. its second argument; each Jacobian is
-//           applied transposed to that residual's weighted lambda
-//           (-s wf sum_j lambda_j phi_j);
-//   volume  thread per (element, point): lambda mapped to the contravariant
-//           flux, through J^-1 to the Cartesian flux, through the transposed
-//           Euler-flux Jacobian (dual numbers) to the point state;
-//   project thread per (element, variable, mode): the transposed
-//           interpolations back to the modes, then the fused epilogue
-//           out = c0 X + c1 Y + c2 Z + c3 (dR/dU)^T lambda.
+// The paper has no adjoint; this is the reverse of the forward kernels' steps, in the same three
+// launches with every face once:
+//   k_traces       (kernels_simt.cu) the traces of U and of lambda at the points of every face, to
+//                  two face buffers;
+//   k_faces_vjp    thread per (interior face, point): the flux H(U_owner, U_other, n_owner) enters the
+//                  owner's residual with -s wf and the other's with +s' wf, so its cotangent is
+//                  s' lambda_other - s lambda_owner (wf is applied by the lift below); one reverse
+//                  sweep gives both states' adjoints, written over the traces of U.  At a kink, where
+//                  the two residuals take different branches, a sweep for each;
+//   k_bfaces_vjp   the same on boundary faces, through the ghost state (dual numbers: few faces);
+//   k_element_vjp  tiles of 32 elements, thread per (element, variable) row: U and the three
+//                  derivatives of lambda at the volume points; thread per (element, point): the
+//                  reverse of the contravariant Euler flux; rows again: the transposed interpolation,
+//                  the lift of the face adjoints, and the epilogue
+//                  out = c0 X + c1 Y + c2 Z + c3 (dR/dU)^T lambda.
+// FP64 is bound by the FP64 pipe.  Before, each side of each face differentiated two fluxes in forward
+// mode (5 tangents each) between dense contractions: one P2 Rusanov VJP of 196,608 elements took
+// 13.4 ms.
 #include <algorithm>
+#include <type_traits>
 
 #include "dg_internal.h"
 #include "dual.cuh"
+#include "face_flux.cuh"
+#include "modal_ops.cuh"
 
 namespace dg {
 
 namespace {
 
 constexpr int NT = 256;
+
+// ---- FP32 without face buffers: each element differentiates its faces from both sides in forward
+// mode; used only where the face buffers cannot be allocated
 
 template <int P> struct VTile;
 template <> struct VTile<1> { static constexpr int EPB = 16; };
@@ -327,6 +332,253 @@ cudaError_t vlaunch(const VjpArgs<Real>& args, cudaStream_t s, int nsm) {
     return cudaGetLastError();
 }
 
+// ---- face-once form -------------------------------------------------------------------------------
+
+constexpr int VF = 128;   // threads of the face kernels
+
+template <typename Real>
+struct FaceVjpArgs {
+    Real* T;                // traces of U in, face adjoints out [ne][4][5][Nqf]
+    const Real* TL;         // traces of lambda
+    const FaceRec* rec;
+    const Real* normal;     // [faces][3]
+    const Real* scale;      // [faces][2] |grad lambda_f| of the slot and of the matching one
+    const int8_t* fperm;
+    int64_t n;              // faces x Nqf
+    Real gamma, roe_eps;
+    Real finf[5];
+};
+
+template <typename Real, int P, int FLUX>
+__global__ void __launch_bounds__(VF) k_faces_vjp(FaceVjpArgs<Real> a) {
+    constexpr int NQF = nqf_of(P);
+    const int64_t i = blockIdx.x * (int64_t)VF + threadIdx.x;
+    if (i >= a.n) return;
+    const int64_t li = i / NQF;
+    const int q = (int)(i - li * NQF);
+    const int4 f = *reinterpret_cast<const int4*>(a.rec + li);   // slot (the owner's), other, code
+    const Real n[3] = {a.normal[3 * li], a.normal[3 * li + 1], a.normal[3 * li + 2]};
+    const Real so = a.scale[2 * li], sn = a.scale[2 * li + 1];
+    const int64_t oe = (int64_t)f.x * 5 * NQF + q, on = (int64_t)f.y * 5 * NQF + a.fperm[(f.z & 7) * NQF + q];
+    Real L[5], R[5], Ho[5], Hn[5], Hb[5], Lb[5], Rb[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+        L[v] = a.T[oe + v * NQF];
+        R[v] = a.T[on + v * NQF];
+        Ho[v] = -so * a.TL[oe + v * NQF];
+        Hn[v] = sn * a.TL[on + v * NQF];
+        Hb[v] = Ho[v] + Hn[v];
+    }
+    if (face_reverse<Real, FLUX>(L, R, n, a.gamma, a.roe_eps, Hb, Real(1), Lb, Rb)) {
+        Real x[5], y[5];
+        face_reverse<Real, FLUX>(L, R, n, a.gamma, a.roe_eps, Ho, Real(1), Lb, Rb);
+        face_reverse<Real, FLUX>(L, R, n, a.gamma, a.roe_eps, Hn, Real(-1), x, y);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+            Lb[v] += x[v];
+            Rb[v] += y[v];
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+        a.T[oe + v * NQF] = Lb[v];
+        a.T[on + v * NQF] = Rb[v];
+    }
+}
+
+template <typename Real, int P, int FLUX>
+__global__ void __launch_bounds__(VF) k_bfaces_vjp(FaceVjpArgs<Real> a) {
+    using D5 = Dual<Real, 5>;
+    constexpr int NQF = nqf_of(P);
+    const int64_t i = blockIdx.x * (int64_t)VF + threadIdx.x;
+    if (i >= a.n) return;
+    const int64_t li = i / NQF;
+    const int q = (int)(i - li * NQF);
+    const int4 f = *reinterpret_cast<const int4*>(a.rec + li);
+    const Real s = a.scale[2 * li];
+    const int64_t oe = (int64_t)f.x * 5 * NQF + q;
+    D5 U[5], G[5], n[3], Fi[5], H[5];
+    const D5 g = D5(a.gamma), eps = D5(a.roe_eps);
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+        U[v] = D5(a.T[oe + v * NQF]);
+        U[v].d[v] = Real(1);
+        Fi[v] = D5(a.finf[v]);
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) n[d] = D5(a.normal[3 * li + d]);
+    if (f.y == -1 - DG_BC_WALL) wall_ghost(U, n, G);
+    else farfield_ghost(U, n, Fi, g, G);
+    riemann<FLUX>(U, G, n, g, eps, H);
+    Real ub[5] = {0, 0, 0, 0, 0};
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+        const Real hb = -s * a.TL[oe + v * NQF];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) ub[k] += H[v].d[k] * hb;
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) a.T[oe + v * NQF] = ub[v];
+}
+
+template <typename Real, int P>
+struct VElemPlan {
+    // the volume points go in NC chunks of consecutive points, closed under the mirror, so that
+    // several tiles fit an SM
+    static constexpr int NQ = nq_of(P), NC = P == 1 ? 1 : 2;
+    static constexpr int first(int c) { return c == 0 ? 0 : c == NC ? NQ : P == 2 ? 8 : 12; }
+    static constexpr int MAXQ = P == 1 ? 4 : P == 2 ? 8 : 12;
+    // shared memory (Reals): point states, then their adjoints [MAXQ][ER]; d_k lambda [MAXQ][3][ER];
+    // J^-1 [EE][9]
+    static constexpr int D = MAXQ * ER, J = D + 3 * MAXQ * ER, REALS = J + EE * 9;
+    static constexpr size_t BYTES = REALS * sizeof(Real);
+};
+
+template <typename Real, int P>
+__global__ void __launch_bounds__(ER) k_element_vjp(VjpArgs<Real> a, const Real* __restrict__ UB) {
+    using S = VElemPlan<Real, P>;
+    constexpr int NB = nb_of(P), NQF = nqf_of(P), NM = modal::Tables<P>::NM;
+    extern __shared__ __align__(16) unsigned char smem[];
+    Real* sU = reinterpret_cast<Real*>(smem);
+    Real* sD = sU + S::D;
+    Real* sJ = sU + S::J;
+    const int t = threadIdx.x;
+    const int64_t e0 = blockIdx.x * (int64_t)EE;
+    const int nel = (a.ne - e0) < (int64_t)EE ? (int)(a.ne - e0) : EE;
+    const bool live = t < 5 * nel;
+    const int64_t row = e0 * 5 + t;
+    const Real g1 = a.gamma - Real(1);
+    for (int i = t; i < nel * 9; i += ER) sJ[i] = a.jinv[e0 * 9 + i];
+    Real r[NB];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) r[j] = 0;
+    // one chunk of points; its bounds are compile-time constants, as the operators' loops need
+    auto chunk = [&](auto ch) {
+        constexpr int q0 = S::first(ch.value), q1 = S::first(ch.value + 1);
+        if (live) {
+            Real c[NB];
+            load_row<NB>(a.U + row * NB, c);
+            modal::interpolate<Real, P, NB, q0, q1>(c, [&](int q, Real u) { sU[(q - q0) * ER + t] = u; });
+            load_row<NB>(a.lam + row * NB, c);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                Real d[NM];
+                modal::grad_modes<Real, P>(k, c, d);
+                modal::interpolate<Real, P, NM, q0, q1>(d, [&](int q, Real x) { sD[((q - q0) * 3 + k) * ER + t] = x; });
+            }
+        }
+        __syncthreads();
+        // reverse of G_k = W_k (m_.. , E + p) + p J^-1_k, W = J^-1 u, against the derivatives of lambda
+        for (int i = t; i < (q1 - q0) * EE; i += ER) {
+            const int e = i % EE, q = i / EE;
+            if (e >= nel) continue;
+            Real* u = sU + q * ER + 5 * e;
+            const Real* g = sD + q * 3 * ER + 5 * e;
+            const Real* I = sJ + e * 9;
+            const Real ri = recip(u[0]);
+            const Real x[3] = {u[1] * ri, u[2] * ri, u[3] * ri};
+            const Real k2 = Real(0.5) * (x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
+            const Real p = g1 * (u[4] - u[0] * k2), ep = u[4] + p;
+            Real ub[5] = {0, 0, 0, 0, 0}, vb[3] = {0, 0, 0}, pb = 0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const Real* gk = g + k * ER;
+                const Real W = I[3 * k] * x[0] + I[3 * k + 1] * x[1] + I[3 * k + 2] * x[2];
+                const Real Wb = gk[0] * u[0] + gk[1] * u[1] + gk[2] * u[2] + gk[3] * u[3] + gk[4] * ep;
+#pragma unroll
+                for (int v = 0; v < 5; ++v) ub[v] += gk[v] * W;
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    vb[d] += I[3 * k + d] * Wb;
+                    pb += I[3 * k + d] * gk[1 + d];
+                }
+            }
+            pb = g1 * (pb + ub[4]);
+            ub[0] += pb * k2 - ri * (vb[0] * x[0] + vb[1] * x[1] + vb[2] * x[2]);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) ub[1 + d] += vb[d] * ri - pb * x[d];
+            ub[4] += pb;
+#pragma unroll
+            for (int v = 0; v < 5; ++v) u[v] = ub[v];
+        }
+        __syncthreads();
+        if (live) {
+#pragma unroll
+            for (int q = q0; q < q1; ++q) {
+                const int m = modal::kT<P>.vmir[q];
+                if (m < q) continue;
+                modal::moments<Real, P, NB>(q, sU[(q - q0) * ER + t], m != q ? sU[(m - q0) * ER + t] : Real(0), r);
+            }
+        }
+    };
+    chunk(std::integral_constant<int, 0>());
+    if constexpr (S::NC > 1) {
+        __syncthreads();
+        chunk(std::integral_constant<int, 1>());
+    }
+    if (!live) return;
+    const int e = t / 5, v = t - 5 * e;
+    const Real* h = UB + ((e0 + e) * 20 + v) * NQF;
+    modal::lift<Real, P>(
+        [&](int f, Real* x) {
+            load_row<NQF>(h + f * 5 * NQF, x);
+            return Real(1);
+        },
+        r);
+#pragma unroll
+    for (int j = 0; j < NB; ++j) r[j] *= a.c3;
+    auto add = [&](const Real* X, Real c) {
+        if (!X) return;
+        Real x[NB];
+        load_row<NB>(X + row * NB, x);
+#pragma unroll
+        for (int j = 0; j < NB; ++j) r[j] += c * x[j];
+    };
+    add(a.X, a.c0);
+    add(a.Y, a.c1);
+    add(a.Z, a.c2);
+    store_row<NB>(a.out + row * NB, r);
+}
+
+template <typename Real, int P, int FLUX>
+cudaError_t vlaunch_faces(dg_mesh* m, const VjpArgs<Real>& r, cudaStream_t s) {
+    constexpr int NQF = nqf_of(P);
+    cudaError_t e = launch_traces2(m, r.U, m->d_TA, r.lam, m->d_TL, s);
+    if (e != cudaSuccess) return e;
+    FaceVjpArgs<Real> f;
+    f.T = static_cast<Real*>(m->d_TA);
+    f.TL = static_cast<const Real*>(m->d_TL);
+    f.rec = m->d_frec;
+    f.normal = static_cast<const Real*>(m->d_fnorm);
+    f.scale = static_cast<const Real*>(m->d_fscale);
+    f.fperm = m->d_fperm;
+    f.n = m->n_interior * NQF;
+    f.gamma = r.gamma;
+    f.roe_eps = r.roe_eps;
+    for (int v = 0; v < 5; ++v) f.finf[v] = r.finf[v];
+    if (f.n > 0) k_faces_vjp<Real, P, FLUX><<<(unsigned)((f.n + VF - 1) / VF), VF, 0, s>>>(f);
+    const int64_t nb = m->n_flist - m->n_interior;
+    if (nb > 0) {
+        f.rec += m->n_interior;
+        f.normal += 3 * m->n_interior;
+        f.scale += 2 * m->n_interior;
+        f.n = nb * NQF;
+        k_bfaces_vjp<Real, P, FLUX><<<(unsigned)((f.n + VF - 1) / VF), VF, 0, s>>>(f);
+    }
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    auto kern = k_element_vjp<Real, P>;
+    constexpr size_t bytes = VElemPlan<Real, P>::BYTES;
+    static bool init = false;
+    if (!init) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+        init = true;
+    }
+    kern<<<(unsigned)((r.ne + EE - 1) / EE), ER, bytes, s>>>(r, f.T);
+    return cudaGetLastError();
+}
+
 template <typename Real>
 cudaError_t vdispatch(dg_mesh* m, const void* U, const void* lam, const void* X, const void* Y, const void* Z,
                       const double c[4], void* out, cudaStream_t s) {
@@ -350,14 +602,25 @@ cudaError_t vdispatch(dg_mesh* m, const void* U, const void* lam, const void* X,
     r.gamma = (Real)m->gamma;
     r.roe_eps = (Real)m->roe_eps;
     for (int v = 0; v < 5; ++v) r.finf[v] = (Real)m->finf[v];
-    int nsm = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
-    if (e != cudaSuccess) return e;
     const bool roe = m->flux == DG_ROE;
-    switch (m->p) {
-        case 1: return roe ? vlaunch<Real, 1, DG_ROE>(r, s, nsm) : vlaunch<Real, 1, DG_RUSANOV>(r, s, nsm);
-        case 2: return roe ? vlaunch<Real, 2, DG_ROE>(r, s, nsm) : vlaunch<Real, 2, DG_RUSANOV>(r, s, nsm);
-        default: return roe ? vlaunch<Real, 3, DG_ROE>(r, s, nsm) : vlaunch<Real, 3, DG_RUSANOV>(r, s, nsm);
+    if (m->face_once && m->d_TA && m->d_TL && m->d_fscale) {
+        switch (m->p) {
+            case 1: return roe ? vlaunch_faces<Real, 1, DG_ROE>(m, r, s) : vlaunch_faces<Real, 1, DG_RUSANOV>(m, r, s);
+            case 2: return roe ? vlaunch_faces<Real, 2, DG_ROE>(m, r, s) : vlaunch_faces<Real, 2, DG_RUSANOV>(m, r, s);
+            default: return roe ? vlaunch_faces<Real, 3, DG_ROE>(m, r, s) : vlaunch_faces<Real, 3, DG_RUSANOV>(m, r, s);
+        }
+    }
+    if constexpr (sizeof(Real) == 8) {
+        return cudaErrorInvalidValue;   // FP64 has no other form
+    } else {
+        int nsm = 0;
+        cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
+        if (e != cudaSuccess) return e;
+        switch (m->p) {
+            case 1: return roe ? vlaunch<Real, 1, DG_ROE>(r, s, nsm) : vlaunch<Real, 1, DG_RUSANOV>(r, s, nsm);
+            case 2: return roe ? vlaunch<Real, 2, DG_ROE>(r, s, nsm) : vlaunch<Real, 2, DG_RUSANOV>(r, s, nsm);
+            default: return roe ? vlaunch<Real, 3, DG_ROE>(r, s, nsm) : vlaunch<Real, 3, DG_RUSANOV>(r, s, nsm);
+        }
     }
 }
 

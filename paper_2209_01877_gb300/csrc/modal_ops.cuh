@@ -238,13 +238,13 @@ __device__ __forceinline__ void axpy(Real& r, double c, Real x) {
     if (c != 0.0) r += (Real)c * x;
 }
 
-// values at the volume points q0 .. q1 - 1 (a range closed under the mirror) of a field of the first N
+// values at the volume points Q0 .. Q1 - 1 (a range closed under the mirror) of a field of the first N
 // modes, store(q, sum_j c[j] phi_j(x_q))
-template <typename Real, int P, int N, typename Store>
-__device__ __forceinline__ void interpolate(const Real* c, int q0, int q1, Store store) {
+template <typename Real, int P, int N, int Q0, int Q1, typename Store>
+__device__ __forceinline__ void interpolate(const Real* c, Store store) {
     constexpr auto& T = kT<P>;
 #pragma unroll
-    for (int q = q0; q < q1; ++q) {
+    for (int q = Q0; q < Q1; ++q) {
         const int m = T.vmir[q];
         if (m < q) continue;
         Real e = 0, o = 0;
