@@ -260,17 +260,18 @@ cudaError_t dispatch_flux(const ResArgs<Real>& args, int flux, bool rk, cudaStre
 
 // ---- face-once form -----------------------------------------------------------------------------
 
-constexpr int FT = 128;       // threads of k_faces
+constexpr int FT = 128;       // threads of k_faces; 32 where that would leave SMs without a block
+inline unsigned face_block(int64_t n) { return n < (int64_t)FT * 4 * 152 ? 32 : FT; }
 
 // The trace of every (element, face, point) of one or (gridDim.y = 2) two states: thread per (element,
 // variable) row.  In FP32 the tile's
 // coefficients and traces pass through shared memory, so that the global accesses are whole lines:
 // rows written directly (24 to 48 bytes each) kept the load-store unit busy (P2, 663,552 elements:
 // 127 us at 39 % of the DRAM rate).  FP64 is bound by its pipe and writes its rows directly.
-template <typename Real, int P>
-__global__ void __launch_bounds__(ER, sizeof(Real) == 8 ? (P == 3 ? 3 : P == 2 ? 6 : 10) : (P == 3 ? 5 : 10))
+template <typename Real, int P, int EE>
+__global__ void __launch_bounds__(threads_of(EE), EE == 32 ? (sizeof(Real) == 8 ? (P == 3 ? 3 : P == 2 ? 6 : 10) : (P == 3 ? 5 : 10)) : 14)
     k_traces(const Real* U0, Real* T0, const Real* U1, Real* T1, int64_t ne) {
-    constexpr int NB = nb_of(P), NQF = nqf_of(P);
+    constexpr int NB = nb_of(P), NQF = nqf_of(P), NT = threads_of(EE);
     const Real* __restrict__ U = blockIdx.y == 0 ? U0 : U1;
     Real* __restrict__ T = blockIdx.y == 0 ? T0 : T1;
     const int t = threadIdx.x;
@@ -284,8 +285,8 @@ __global__ void __launch_bounds__(ER, sizeof(Real) == 8 ? (P == 3 ? 3 : P == 2 ?
         Real* o = T + ((e0 + e) * 20 + v) * NQF;
         modal::traces<Real, P>(c, [&](int f, const Real* u) { store_row<NQF>(o + f * 5 * NQF, u); });
     } else {
-        __shared__ __align__(16) Real sU[ER * NB], sT[EE * 20 * NQF];
-        copy_tile(sU, U + e0 * 5 * NB, nel * 5 * NB * (int)sizeof(Real));
+        __shared__ __align__(16) Real sU[rows_of(EE) * NB + 4], sT[EE * 20 * NQF];
+        copy_tile<NT>(sU, U + e0 * 5 * NB, nel * 5 * NB * (int)sizeof(Real));
         tc::cp_async_wait_all();
         __syncthreads();
         if (t < 5 * nel) {
@@ -296,15 +297,18 @@ __global__ void __launch_bounds__(ER, sizeof(Real) == 8 ? (P == 3 ? 3 : P == 2 ?
         }
         __syncthreads();
         float4* g = reinterpret_cast<float4*>(T + e0 * 20 * NQF);
-        for (int i = t; i < nel * 5 * NQF; i += ER) g[i] = reinterpret_cast<const float4*>(sT)[i];
+        for (int i = t; i < nel * 5 * NQF; i += NT) g[i] = reinterpret_cast<const float4*>(sT)[i];
     }
 }
 
 template <typename Real, int P>
 cudaError_t traces(const void* U, void* T, const void* U1, void* T1, int64_t ne, cudaStream_t s) {
-    const dim3 grid((unsigned)((ne + EE - 1) / EE), U1 ? 2 : 1);
-    k_traces<Real, P><<<grid, ER, 0, s>>>(static_cast<const Real*>(U), static_cast<Real*>(T), static_cast<const Real*>(U1),
-                                          static_cast<Real*>(T1), ne);
+    const Real *u = static_cast<const Real*>(U), *u1 = static_cast<const Real*>(U1);
+    Real *t = static_cast<Real*>(T), *t1 = static_cast<Real*>(T1);
+    if (small_tiles(ne))
+        k_traces<Real, P, 6><<<dim3((unsigned)((ne + 5) / 6), U1 ? 2 : 1), threads_of(6), 0, s>>>(u, t, u1, t1, ne);
+    else
+        k_traces<Real, P, 32><<<dim3((unsigned)((ne + 31) / 32), U1 ? 2 : 1), threads_of(32), 0, s>>>(u, t, u1, t1, ne);
     return cudaGetLastError();
 }
 
@@ -325,7 +329,7 @@ struct FaceArgs {
 template <typename Real, int P, int FLUX>
 __global__ void __launch_bounds__(FT) k_faces(FaceArgs<Real> a) {
     constexpr int NQF = nqf_of(P);
-    const int64_t i = blockIdx.x * (int64_t)FT + threadIdx.x;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     const int64_t li = i / NQF;
     const int q = (int)(i - li * NQF);
@@ -372,25 +376,28 @@ __global__ void __launch_bounds__(FT) k_faces(FaceArgs<Real> a) {
     }
 }
 
-template <typename Real, int P>
+template <typename Real, int P, int EE>
 struct ElemPlan {
     // FP32 projects the deviation from the flux of the element's mean state, which is point NQ, and
     // passes its rows through shared memory
     static constexpr bool F32 = sizeof(Real) == 4;
+    static constexpr int ER = rows_of(EE);
     static constexpr int NB = nb_of(P), NQ = nq_of(P), NP = NQ + (F32 ? 1 : 0);
     // shared memory (Reals): point states [NP][ER], (W_0, W_1, W_2, p) [NP][EE][4], then J^-1 [EE][9],
     // |grad lambda_f| [EE][4]; FP32: the tile's coefficients [ER][NB] (the new ones at the end) and
     // its face fluxes, which take the place of the point values once those are projected (P3: 5
     // tiles per SM instead of 2)
-    static constexpr int W = NP * ER, POINTS = W + NP * EE * 4, FACES = F32 ? EE * 20 * nqf_of(P) : 0;
+    static constexpr int r4(int n) { return (n + 3) / 4 * 4; }   // regions start on 16-byte boundaries
+    static constexpr int W = r4(NP * ER), POINTS = W + NP * EE * 4, FACES = F32 ? EE * 20 * nqf_of(P) : 0;
     static constexpr int J = POINTS > FACES ? POINTS : FACES;
-    static constexpr int G = J + EE * 9, C = G + EE * 4, REALS = C + (F32 ? ER * NB : 0);
+    static constexpr int G = J + EE * 9, C = r4(G + EE * 4), REALS = C + (F32 ? ER * NB + 4 : 0);
     static constexpr size_t BYTES = REALS * sizeof(Real);
 };
 
-template <typename Real, int P, bool RK>
-__global__ void __launch_bounds__(ER) k_element(ResArgs<Real> a) {
-    using S = ElemPlan<Real, P>;
+template <typename Real, int P, bool RK, int EE>
+__global__ void __launch_bounds__(threads_of(EE)) k_element(ResArgs<Real> a) {
+    using S = ElemPlan<Real, P, EE>;
+    constexpr int ER = S::ER, NT = threads_of(EE);
     constexpr int NB = nb_of(P), NQ = nq_of(P), NQF = nqf_of(P), NM = modal::Tables<P>::NM;
     extern __shared__ __align__(16) unsigned char smem[];
     Real* sU = reinterpret_cast<Real*>(smem);
@@ -404,9 +411,9 @@ __global__ void __launch_bounds__(ER) k_element(ResArgs<Real> a) {
     const bool live = t < 5 * nel;
     const int64_t row = e0 * 5 + t;
     if (S::F32) {
-        copy_tile(sC, a.U + e0 * 5 * NB, nel * 5 * NB * (int)sizeof(Real));
+        copy_tile<NT>(sC, a.U + e0 * 5 * NB, nel * 5 * NB * (int)sizeof(Real));
     }
-    for (int i = t; i < nel * 9; i += ER) sJ[i] = a.jinv[e0 * 9 + i];
+    for (int i = t; i < nel * 9; i += NT) sJ[i] = a.jinv[e0 * 9 + i];
     if (S::F32) {
         tc::cp_async_wait_all();
         __syncthreads();
@@ -427,7 +434,7 @@ __global__ void __launch_bounds__(ER) k_element(ResArgs<Real> a) {
         sG[t] = EulerOps<Real>::sqrt_(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
     }
     // contravariant velocity W_k = sum_d (J^-1)_kd u_d and pressure at every (element, point)
-    for (int i = t; i < S::NP * EE; i += ER) {
+    for (int i = t; i < S::NP * EE; i += NT) {
         const int e = i % EE, q = i / EE;
         if (e >= nel) continue;
         const Real* u = sU + q * ER + 5 * e;
@@ -472,7 +479,7 @@ __global__ void __launch_bounds__(ER) k_element(ResArgs<Real> a) {
     }
     if (S::F32) {
         __syncthreads();
-        copy_tile(sU, a.Hs + e0 * 20 * NQF, nel * 20 * NQF * (int)sizeof(Real));
+        copy_tile<NT>(sU, a.Hs + e0 * 20 * NQF, nel * 20 * NQF * (int)sizeof(Real));
         tc::cp_async_wait_all();
         __syncthreads();
     }
@@ -512,7 +519,7 @@ __global__ void __launch_bounds__(ER) k_element(ResArgs<Real> a) {
     if constexpr (S::F32) {   // whole lines: out = the tile (+ a U0)
         __syncthreads();
         const int n = nel * 5 * NB;
-        for (int i = 4 * t; i < n; i += 4 * ER) {
+        for (int i = 4 * t; i < n; i += 4 * NT) {
             float4 x = *reinterpret_cast<const float4*>(sC + i);
             const int64_t g = e0 * 5 * NB + i;
             if (i + 4 <= n) {
@@ -528,18 +535,23 @@ __global__ void __launch_bounds__(ER) k_element(ResArgs<Real> a) {
     }
 }
 
-template <typename Real, int P, bool RK>
-cudaError_t launch_element(const ResArgs<Real>& r, cudaStream_t s) {
-    constexpr size_t bytes = ElemPlan<Real, P>::BYTES;
-    auto kern = k_element<Real, P, RK>;
+template <typename Real, int P, bool RK, int EE>
+cudaError_t launch_tiles(const ResArgs<Real>& r, cudaStream_t s) {
+    constexpr size_t bytes = ElemPlan<Real, P, EE>::BYTES;
+    auto kern = k_element<Real, P, RK, EE>;
     static bool init = false;
     if (!init) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e != cudaSuccess) return e;
         init = true;
     }
-    kern<<<(unsigned)((r.ne + EE - 1) / EE), ER, bytes, s>>>(r);
+    kern<<<(unsigned)((r.ne + EE - 1) / EE), threads_of(EE), bytes, s>>>(r);
     return cudaGetLastError();
+}
+
+template <typename Real, int P, bool RK>
+cudaError_t launch_element(const ResArgs<Real>& r, cudaStream_t s) {
+    return small_tiles(r.ne) ? launch_tiles<Real, P, RK, 6>(r, s) : launch_tiles<Real, P, RK, 32>(r, s);
 }
 
 template <typename Real, int P>
@@ -557,9 +569,9 @@ cudaError_t launch_face_once(dg_mesh* m, ResArgs<Real>& r, bool rk, void* T, cud
     cudaError_t e = traces<Real, P>(r.U, f.T, nullptr, nullptr, m->n_trace, s);
     if (e != cudaSuccess) return e;
     if (f.n > 0) {
-        const unsigned grid = (unsigned)((f.n + FT - 1) / FT);
-        if (m->flux == DG_ROE) k_faces<Real, P, DG_ROE><<<grid, FT, 0, s>>>(f);
-        else k_faces<Real, P, DG_RUSANOV><<<grid, FT, 0, s>>>(f);
+        const unsigned nt = face_block(f.n), grid = (unsigned)((f.n + nt - 1) / nt);
+        if (m->flux == DG_ROE) k_faces<Real, P, DG_ROE><<<grid, nt, 0, s>>>(f);
+        else k_faces<Real, P, DG_RUSANOV><<<grid, nt, 0, s>>>(f);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

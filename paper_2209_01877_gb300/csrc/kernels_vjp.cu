@@ -334,7 +334,8 @@ cudaError_t vlaunch(const VjpArgs<Real>& args, cudaStream_t s, int nsm) {
 
 // ---- face-once form -------------------------------------------------------------------------------
 
-constexpr int VF = 128;   // threads of the face kernels
+constexpr int VF = 128;   // threads of the face kernels; 32 where that would leave SMs without a block
+inline unsigned vface_block(int64_t n) { return n < (int64_t)VF * 4 * 152 ? 32 : VF; }
 
 template <typename Real>
 struct FaceVjpArgs {
@@ -352,7 +353,7 @@ struct FaceVjpArgs {
 template <typename Real, int P, int FLUX>
 __global__ void __launch_bounds__(VF) k_faces_vjp(FaceVjpArgs<Real> a) {
     constexpr int NQF = nqf_of(P);
-    const int64_t i = blockIdx.x * (int64_t)VF + threadIdx.x;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     const int64_t li = i / NQF;
     const int q = (int)(i - li * NQF);
@@ -390,7 +391,7 @@ template <typename Real, int P, int FLUX>
 __global__ void __launch_bounds__(VF) k_bfaces_vjp(FaceVjpArgs<Real> a) {
     using D5 = Dual<Real, 5>;
     constexpr int NQF = nqf_of(P);
-    const int64_t i = blockIdx.x * (int64_t)VF + threadIdx.x;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     const int64_t li = i / NQF;
     const int q = (int)(i - li * NQF);
@@ -421,8 +422,9 @@ __global__ void __launch_bounds__(VF) k_bfaces_vjp(FaceVjpArgs<Real> a) {
     for (int v = 0; v < 5; ++v) a.T[oe + v * NQF] = ub[v];
 }
 
-template <typename Real, int P>
+template <typename Real, int P, int EE>
 struct VElemPlan {
+    static constexpr int ER = rows_of(EE);
     // the volume points go in NC chunks of consecutive points, closed under the mirror, so that
     // several tiles fit an SM
     static constexpr int NQ = nq_of(P), NC = P == 1 ? 1 : 2;
@@ -434,9 +436,10 @@ struct VElemPlan {
     static constexpr size_t BYTES = REALS * sizeof(Real);
 };
 
-template <typename Real, int P>
-__global__ void __launch_bounds__(ER) k_element_vjp(VjpArgs<Real> a, const Real* __restrict__ UB) {
-    using S = VElemPlan<Real, P>;
+template <typename Real, int P, int EE>
+__global__ void __launch_bounds__(threads_of(EE)) k_element_vjp(VjpArgs<Real> a, const Real* __restrict__ UB) {
+    using S = VElemPlan<Real, P, EE>;
+    constexpr int ER = S::ER, NT = threads_of(EE);
     constexpr int NB = nb_of(P), NQF = nqf_of(P), NM = modal::Tables<P>::NM;
     extern __shared__ __align__(16) unsigned char smem[];
     Real* sU = reinterpret_cast<Real*>(smem);
@@ -448,7 +451,7 @@ __global__ void __launch_bounds__(ER) k_element_vjp(VjpArgs<Real> a, const Real*
     const bool live = t < 5 * nel;
     const int64_t row = e0 * 5 + t;
     const Real g1 = a.gamma - Real(1);
-    for (int i = t; i < nel * 9; i += ER) sJ[i] = a.jinv[e0 * 9 + i];
+    for (int i = t; i < nel * 9; i += NT) sJ[i] = a.jinv[e0 * 9 + i];
     Real r[NB];
 #pragma unroll
     for (int j = 0; j < NB; ++j) r[j] = 0;
@@ -469,7 +472,7 @@ __global__ void __launch_bounds__(ER) k_element_vjp(VjpArgs<Real> a, const Real*
         }
         __syncthreads();
         // reverse of G_k = W_k (m_.. , E + p) + p J^-1_k, W = J^-1 u, against the derivatives of lambda
-        for (int i = t; i < (q1 - q0) * EE; i += ER) {
+        for (int i = t; i < (q1 - q0) * EE; i += NT) {
             const int e = i % EE, q = i / EE;
             if (e >= nel) continue;
             Real* u = sU + q * ER + 5 * e;
@@ -540,6 +543,20 @@ __global__ void __launch_bounds__(ER) k_element_vjp(VjpArgs<Real> a, const Real*
     store_row<NB>(a.out + row * NB, r);
 }
 
+template <typename Real, int P, int EE>
+cudaError_t vlaunch_tiles(const VjpArgs<Real>& r, const Real* UB, cudaStream_t s) {
+    auto kern = k_element_vjp<Real, P, EE>;
+    constexpr size_t bytes = VElemPlan<Real, P, EE>::BYTES;
+    static bool init = false;
+    if (!init) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+        init = true;
+    }
+    kern<<<(unsigned)((r.ne + EE - 1) / EE), threads_of(EE), bytes, s>>>(r, UB);
+    return cudaGetLastError();
+}
+
 template <typename Real, int P, int FLUX>
 cudaError_t vlaunch_faces(dg_mesh* m, const VjpArgs<Real>& r, cudaStream_t s) {
     constexpr int NQF = nqf_of(P);
@@ -556,27 +573,20 @@ cudaError_t vlaunch_faces(dg_mesh* m, const VjpArgs<Real>& r, cudaStream_t s) {
     f.gamma = r.gamma;
     f.roe_eps = r.roe_eps;
     for (int v = 0; v < 5; ++v) f.finf[v] = r.finf[v];
-    if (f.n > 0) k_faces_vjp<Real, P, FLUX><<<(unsigned)((f.n + VF - 1) / VF), VF, 0, s>>>(f);
+    unsigned nt = vface_block(f.n);
+    if (f.n > 0) k_faces_vjp<Real, P, FLUX><<<(unsigned)((f.n + nt - 1) / nt), nt, 0, s>>>(f);
     const int64_t nb = m->n_flist - m->n_interior;
     if (nb > 0) {
         f.rec += m->n_interior;
         f.normal += 3 * m->n_interior;
         f.scale += 2 * m->n_interior;
         f.n = nb * NQF;
-        k_bfaces_vjp<Real, P, FLUX><<<(unsigned)((f.n + VF - 1) / VF), VF, 0, s>>>(f);
+        nt = vface_block(f.n);
+        k_bfaces_vjp<Real, P, FLUX><<<(unsigned)((f.n + nt - 1) / nt), nt, 0, s>>>(f);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    auto kern = k_element_vjp<Real, P>;
-    constexpr size_t bytes = VElemPlan<Real, P>::BYTES;
-    static bool init = false;
-    if (!init) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        init = true;
-    }
-    kern<<<(unsigned)((r.ne + EE - 1) / EE), ER, bytes, s>>>(r, f.T);
-    return cudaGetLastError();
+    return small_tiles(r.ne) ? vlaunch_tiles<Real, P, 6>(r, f.T, s) : vlaunch_tiles<Real, P, 32>(r, f.T, s);
 }
 
 template <typename Real>

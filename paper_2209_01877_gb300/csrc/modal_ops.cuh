@@ -411,13 +411,19 @@ __device__ __forceinline__ void lift(Load load, Real* r) {
 
 // ---- rows and tiles -------------------------------------------------------------------------------
 
-constexpr int EE = 32;        // elements per tile of the CUDA-core kernels
-constexpr int ER = 5 * EE;    // rows (element, variable) = threads
+// The CUDA-core kernels work on tiles of EE consecutive elements, thread per (element, variable) row:
+// 32 elements (five full warps), or 6 (30 rows of one warp) on a mesh whose tiles of 32 would not
+// give every SM two: 10 SSP-RK3 steps of 1,296 P1 elements in FP64 617 -> 542 us; on 196,608 P3
+// elements 6 would cost 4% (17.4 -> 18.1 ms per step).  An element's arithmetic does not depend on EE.
+constexpr int rows_of(int ee) { return 5 * ee; }
+constexpr int threads_of(int ee) { return (5 * ee + 31) / 32 * 32; }
+inline bool small_tiles(int64_t ne) { return ne < 32 * 2 * 152; }
 
-// n bytes of a tile, global -> shared, by all ER threads (asynchronous, 16 bytes each; n rounded up:
+// n bytes of a tile, global -> shared, by all NT threads (asynchronous, 16 bytes each; n rounded up:
 // the buffers end in slack)
+template <int NT>
 __device__ __forceinline__ void copy_tile(void* dst, const void* src, int n) {
-    for (int i = threadIdx.x * 16; i < n; i += ER * 16)
+    for (int i = threadIdx.x * 16; i < n; i += NT * 16)
         tc::cp_async16(static_cast<char*>(dst) + i, static_cast<const char*>(src) + i);
     tc::cp_async_commit();
 }
