@@ -21,9 +21,9 @@ constexpr int nqf_of(int p) { return p == 1 ? 3 : (p == 2 ? 6 : 12); }
 //   PHIFW [4][Nqf][Nb]  wf_q * phi_j at point q of local face f
 //   WQ    [Nq]          volume weights (sum 1/6)
 struct TabLayout {
-    int nb, nq, nqf;
-    int phiq, dphiw, phif, phifw, wq, total;
-    explicit TabLayout(int p) {
+    int nb = 0, nq = 0, nqf = 0;
+    int phiq = 0, dphiw = 0, phif = 0, phifw = 0, wq = 0, total = 0;
+    constexpr explicit TabLayout(int p) {
         nb = nb_of(p); nq = nq_of(p); nqf = nqf_of(p);
         phiq = 0;
         dphiw = phiq + nb * nq;
