@@ -71,11 +71,9 @@ namespace dg {
 
 namespace {
 
-constexpr int MT = 512;      // threads per CTA
 constexpr int CT = 256;      // threads per context
 constexpr int ET = 12;       // elements per tile
 constexpr int SLOTS = 4 * ET;
-constexpr int TMEM_COLS = 512, CTX_COLS = 256;
 constexpr long WAIT_ITERS = 20000000;
 
 constexpr int r8(int x) { return (x + 7) / 8 * 8; }
@@ -117,7 +115,13 @@ struct SPlan {
     // over independent accumulators, so consecutive MMAs do not wait on one another
     static constexpr int NCH = 3;
     static constexpr int C_D1 = 0, C_D2 = r16(N1);
-    static_assert(C_D2 + NCH * 2 * N2 <= CTX_COLS, "tensor memory");
+    // contexts of the CTA: three where shared memory and the 512 tensor-memory columns hold them (80
+    // registers a thread then; P3 holds two).  A context's tile is a chain of phases of about 4 us
+    // whatever the order, so more chains per SM hide more of it: P1, 48,000 elements, 54 -> 42 us per
+    // stage; P2, 663,552 elements, 883 -> 740 us
+    static constexpr int NCTX = P < 3 ? 3 : 2, MT = NCTX * CT;
+    static constexpr int CTX_COLS = P == 1 ? 64 : P == 2 ? 160 : 256, TMEM_COLS = P == 1 ? 256 : 512;
+    static_assert(C_D2 + NCH * 2 * N2 <= CTX_COLS && NCTX * CTX_COLS <= TMEM_COLS, "tensor memory");
     static_assert(K2 / 16 >= NCH, "every accumulator receives a K step");
     // point-state staging [ET][5][VSTR]: VSTR = 8 (mod 32) and >= the staged columns, so USTR =
     // 5 VSTR = 8 (mod 32) too; then row 5e + v starts at bank 8 (e + v) (mod 32), any 4
@@ -153,7 +157,7 @@ struct SPlan {
     static constexpr int X_C = a128(X_XN + (SLOTS + 1) * 4);                // float [SLOTS][5 Nb] neighbour blocks
     static constexpr int X_MB = a128(X_C + SZ_C);                          // mbarrier, then the drain mbarrier
     static constexpr int CTX_BYTES = a128(X_MB + 16);
-    static constexpr int O_PERM = O_CTX + 2 * CTX_BYTES;                   // int8 [6][NQF]
+    static constexpr int O_PERM = O_CTX + NCTX * CTX_BYTES;                   // int8 [6][NQF]
     static constexpr int O_SLOT = a128(O_PERM + 6 * NQF);                  // tmem slot
     static constexpr int BYTES = O_SLOT + 16;
     static_assert(BYTES <= 227 * 1024, "shared memory");
@@ -306,8 +310,9 @@ __device__ __forceinline__ void elem_setup(const StageArgs& a, int64_t ge, int e
 }
 
 template <int P, int FLUX, bool BF, bool CONS>
-__global__ void __launch_bounds__(MT, 1) k_stage_mixed(StageArgs a) {
+__global__ void __launch_bounds__(SPlan<P>::MT, 1) k_stage_mixed(StageArgs a) {
     using S = SPlan<P>;
+    constexpr int MT = S::MT;
     constexpr int NB = S::NB, NQ = S::NQ, NQF = S::NQF, NQF4 = S::NQF4, FPAD = S::FPAD;
     constexpr int K1 = S::K1, K2 = S::K2, N1 = S::N1, N2 = S::N2, VSTR = S::VSTR, USTR = S::USTR, NV5 = S::NV5;
     constexpr int ELW = S::ELW;
@@ -346,9 +351,12 @@ __global__ void __launch_bounds__(MT, 1) k_stage_mixed(StageArgs a) {
         dst = reinterpret_cast<uint4*>(smem + S::O_T2);
         src = reinterpret_cast<const uint4*>(a.tab16 + S::G_T2);
         for (int i = tid; i < S::SZ_T2 / 16; i += MT) dst[i] = src[i];
-        // every byte an MMA may read is finite
+        // every byte an MMA may read is finite (a context without a tile issues none)
         uint4* z = reinterpret_cast<uint4*>(smem + S::O_CTX);
-        for (int i = tid; i < 2 * S::CTX_BYTES / 16; i += MT) z[i] = make_uint4(0, 0, 0, 0);
+        const int64_t nt = (a.ne + ET - 1) / ET;
+        int nact = 0;
+        while (nact < S::NCTX && (int64_t)blockIdx.x + nact * (int64_t)gridDim.x < nt) ++nact;
+        for (int i = tid; i < nact * S::CTX_BYTES / 16; i += MT) z[i] = make_uint4(0, 0, 0, 0);
         int8_t* pm = reinterpret_cast<int8_t*>(smem + S::O_PERM);
         for (int i = tid; i < 6 * NQF; i += MT) pm[i] = a.fperm[i];
         // face-point basis, transposed to [f][p][j] so a point's row is contiguous
@@ -363,20 +371,21 @@ __global__ void __launch_bounds__(MT, 1) k_stage_mixed(StageArgs a) {
         tc::mbar_init(mbar);
         tc::mbar_init(mbar + 1);   // drain: one commit after the last MMA of the context
     }
-    if (warp == 0) tc::tmem_alloc(tslot, TMEM_COLS);
+    if (warp == 0) tc::tmem_alloc(tslot, S::TMEM_COLS);
     tc::fence_async_smem();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    const uint32_t tmem = *tslot + ctx * CTX_COLS;
+    const uint32_t tmem = *tslot + ctx * S::CTX_COLS;
     uint32_t phase = 0;
     const int wc = ct >> 5;                          // warp within the context
     const int qq = wc & 3, part = wc >> 2;           // TMEM lane quarter (warp % 4), column part (0, 1)
     const uint32_t lane_base = (uint32_t)(qq * 32) << 16;
 
     const int64_t ntiles = (a.ne + ET - 1) / ET;
-    const int64_t tstride = 2 * (int64_t)gridDim.x;
-    const int64_t tfirst = 2 * (int64_t)blockIdx.x + ctx;
+    // tiles go round the CTAs first, so that a mesh of few tiles uses every SM
+    const int64_t tstride = S::NCTX * (int64_t)gridDim.x;
+    const int64_t tfirst = (int64_t)blockIdx.x + ctx * (int64_t)gridDim.x;
     // prologue: the first tile's operand rows, metadata and neighbour blocks.  Later tiles' are
     // prepared during the previous tile: neighbour ids while MMA 1 runs, the block copies after
     // the traces, the operand rows and metadata while MMA 2 runs
@@ -808,7 +817,7 @@ __global__ void __launch_bounds__(MT, 1) k_stage_mixed(StageArgs a) {
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    if (warp == 0) tc::tmem_dealloc(*tslot, TMEM_COLS);
+    if (warp == 0) tc::tmem_dealloc(*tslot, S::TMEM_COLS);
 }
 
 namespace {
@@ -824,7 +833,7 @@ cudaError_t slaunch1(const StageArgs& sa, cudaStream_t s, int nsm) {
         init = true;
     }
     const int64_t ntiles = (sa.ne + ET - 1) / ET;
-    k<<<(int)std::min<int64_t>((ntiles + 1) / 2, (int64_t)nsm), MT, S::BYTES, s>>>(sa);
+    k<<<(int)std::min<int64_t>(ntiles, (int64_t)nsm), S::MT, S::BYTES, s>>>(sa);
     return cudaGetLastError();
 }
 
