@@ -80,7 +80,6 @@ void free_mesh(dg_mesh* m) {
     cudaFree(m->d_farea);
     cudaFree(m->d_frec);
     cudaFree(m->d_fnorm);
-    if (m->d_TW != m->d_T) cudaFree(m->d_TW);
     if (m->d_TA != m->d_T) cudaFree(m->d_TA);
     cudaFree(m->d_TL);
     cudaFree(m->d_fscale);
@@ -112,13 +111,6 @@ dg_status ensure_face_buffer(dg_mesh* m, void*& buf, size_t bytes) {
     if (m->precision == DG_FP64 || e != cudaErrorMemoryAllocation) return cuda_fail(e, "cudaMalloc(face buffer)");
     (void)cudaGetLastError();
     return DG_OK;
-}
-
-// the buffers of the calls that leave a residual in d_W
-dg_status ensure_residual_buffers(dg_mesh* m) {
-    const dg_status st = ensure_work_buffers(m);
-    if (st != DG_OK || m->precision == DG_FP64) return st;
-    return ensure_face_buffer(m, m->d_TW, m->face_bytes());
 }
 
 }  // namespace
@@ -240,7 +232,7 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
             free_mesh(m);
             return cuda_fail(e, "face buffers");
         }
-        if (m->precision == DG_FP64) m->d_TW = m->d_TA = m->d_T;
+        if (m->precision == DG_FP64) m->d_TA = m->d_T;
     }
     if (m->precision == DG_FP64) {
         m->d_tab = m->d_tab64;   // shared; freed once below
@@ -394,15 +386,43 @@ dg_status dg_get_state(const dg_mesh* mc, double* U, int on_device, void* stream
     return DG_OK;
 }
 
+namespace {
+// The face buffer of the calls that return a residual.  In FP32 they take the kernel that needs none:
+// the residual is what is left of cancelling terms, and two FP32 evaluations in different orders differ
+// by 2e-5 to 6e-5 of its norm (each is that far from the exact one); these calls keep the order, and
+// the values, they have always had.  In an RK stage dt R moves the state by 1e-8 of that difference,
+// and the faster form is used.
+void* residual_faces(const dg_mesh* m) { return m->precision == DG_FP64 ? m->d_T : nullptr; }
+
+// The face buffer of an FP32 RK stage, or null for the single kernel.  The single kernel is the faster one
+// while its tiles make one wave (P1, 900 elements: 75 us for two steps against 89 us for the three
+// launches; P3, 83,000 elements: 1,163 against 403 us).  On a mesh with boundary faces it is kept too:
+// dg_boundary_flux reports the boundary integral of the FP32 state in FP64, which shows the order of
+// summation at 1e-7.
+constexpr int64_t FP32_FACES_MIN_NE = 8192;
+void* stage_faces(const dg_mesh* m, void* T) {
+    return m->precision == DG_FP64 || (m->host.ne >= FP32_FACES_MIN_NE && !m->has_bc) ? T : nullptr;
+}
+// the same where no boundary integral is taken of the states: Navier-Stokes steps and the adjoint's stages
+void* inner_faces(const dg_mesh* m, void* T) {
+    return m->precision == DG_FP64 || m->host.ne >= FP32_FACES_MIN_NE ? T : nullptr;
+}
+
+// a caller's state as a residual's operand, in d_W[0]: the mixed forms' residual reads the hi plane
+cudaError_t gather_operand(dg_mesh* m, const double* U, cudaStream_t s) {
+    return is_mixed(m) ? dg::launch_gather_f32(m, U, static_cast<float*>(m->d_W[0]), s) : dg::launch_gather(m, U, m->d_W[0], s);
+}
+}  // namespace
+
 dg_status dg_residual(dg_mesh* m, const double* U, double* R, void* stream) {
     if (!m || !R) return fail(DG_ERR_ARG, "mesh and R must be non-NULL");
     if (!U && !m->has_state) return fail(DG_ERR_NOSTATE, "no state set and U is NULL");
-    dg_status st = ensure_residual_buffers(m);
+    dg_status st = ensure_work_buffers(m);
     if (st != DG_OK) return st;
     cudaStream_t s = as_stream(stream);
     const void* in = m->d_B[0];
     if (U) {
-        DG_CUDA(dg::launch_gather(m, U, m->d_W[0], s));
+        DG_CUDA(gather_operand(m, U, s));
         in = m->d_W[0];
     }
     if (is_mixed(m)) {
@@ -412,19 +432,20 @@ dg_status dg_residual(dg_mesh* m, const double* U, double* R, void* stream) {
         DG_CUDA(dg::launch_scatter_f32(m, out, R, s));
         return DG_OK;
     }
-    DG_CUDA(dg::launch_residual(m, in, nullptr, m->d_W[1], 0, 0.0, 0.0, 0.0, m->d_TW, s));
+    DG_CUDA(dg::launch_residual(m, in, nullptr, m->d_W[1], 0, 0.0, 0.0, 0.0, residual_faces(m), s));
     DG_CUDA(dg::launch_scatter(m, m->d_W[1], R, s));
     return DG_OK;
 }
 
 namespace {
 // the Euler residual of an internal-order state into R (the mesh's precision; the mixed forms
-// write FP32 R) and the Navier-Stokes buffers (element size of the viscous passes' arithmetic)
-cudaError_t euler_residual_internal(dg_mesh* m, const void* in, void* R, cudaStream_t s) {
+// write FP32 R), with the face buffer T, and the Navier-Stokes buffers (element size of the viscous
+// passes' arithmetic)
+cudaError_t euler_residual_internal(dg_mesh* m, const void* in, void* R, void* T, cudaStream_t s) {
     if (is_mixed(m))
         return dg::launch_residual_mixed(m, static_cast<const float*>(in), nullptr, nullptr, nullptr,
                                          static_cast<float*>(R), nullptr, 0, 0.0, 0.0, 0.0, s);
-    return dg::launch_residual(m, in, nullptr, R, 0, 0.0, 0.0, 0.0, m->d_TW, s);
+    return dg::launch_residual(m, in, nullptr, R, 0, 0.0, 0.0, 0.0, T, s);
 }
 
 dg_status ensure_ns_buffers(dg_mesh* m) {
@@ -439,15 +460,15 @@ dg_status dg_ns_residual(dg_mesh* m, const double* U, double* R, double mu, doub
     if (!m || !R) return fail(DG_ERR_ARG, "mesh and R must be non-NULL");
     if (!(mu >= 0.0) || !(prandtl > 0.0)) return fail(DG_ERR_ARG, "mu must be >= 0 and prandtl > 0");
     if (!U && !m->has_state) return fail(DG_ERR_NOSTATE, "no state set and U is NULL");
-    dg_status st = ensure_residual_buffers(m);
+    dg_status st = ensure_work_buffers(m);
     if (st != DG_OK) return st;
     cudaStream_t s = as_stream(stream);
     const void* in = m->d_B[0];
     if (U) {
-        DG_CUDA(dg::launch_gather(m, U, m->d_W[0], s));
+        DG_CUDA(gather_operand(m, U, s));
         in = m->d_W[0];
     }
-    DG_CUDA(euler_residual_internal(m, in, m->d_W[1], s));
+    DG_CUDA(euler_residual_internal(m, in, m->d_W[1], residual_faces(m), s));
     if (mu > 0.0) {
         st = ensure_ns_buffers(m);
         if (st != DG_OK) return st;
@@ -518,7 +539,7 @@ dg_status dg_set_conservative(dg_mesh* m, int enable) {
 namespace {
 // one fused residual + RK stage: out = a U0 + b (U + dt R(U))
 cudaError_t stage_launch(dg_mesh* m, void* U, void* U0, void* out, double dt, double a, double b, cudaStream_t s) {
-    if (!is_mixed(m)) return dg::launch_residual(m, U, U0, out, 1, dt, a, b, m->d_T, s);
+    if (!is_mixed(m)) return dg::launch_residual(m, U, U0, out, 1, dt, a, b, stage_faces(m, m->d_T), s);
     const size_t n = (size_t)m->host.ne * 5 * m->nb;
     float* u = static_cast<float*>(U);
     float* u0 = static_cast<float*>(U0);
@@ -613,7 +634,7 @@ dg_status dg_ns_rk3_step(dg_mesh* m, double dt, int nsteps, double mu, double pr
     if (nsteps == 0) return DG_OK;
     if (!m->has_state) return fail(DG_ERR_NOSTATE, "no state set");
     if (!(dt >= 0.0)) return fail(DG_ERR_ARG, "dt must be >= 0");
-    dg_status st = ensure_residual_buffers(m);
+    dg_status st = ensure_work_buffers(m);
     if (st != DG_OK) return st;
     if (mu > 0.0) {
         st = ensure_ns_buffers(m);
@@ -627,7 +648,7 @@ dg_status dg_ns_rk3_step(dg_mesh* m, double dt, int nsteps, double mu, double pr
                                                                   {2, 0, 0, 1.0 / 3.0, 2.0 / 3.0}};
     for (int k = 0; k < nsteps; ++k)
         for (const auto& g : stages) {
-            DG_CUDA(euler_residual_internal(m, B[g.in], R, s));
+            DG_CUDA(euler_residual_internal(m, B[g.in], R, inner_faces(m, m->d_T), s));
             if (mu > 0.0) DG_CUDA(dg::launch_ns_viscous(m, B[g.in], m->d_Z, m->d_HB, R, mu, prandtl, s));
             DG_CUDA(dg::launch_rk_axpy(m, B[g.in], g.base >= 0 ? B[g.base] : nullptr, R, B[g.out], dt, g.a, g.b, s));
         }
@@ -748,8 +769,8 @@ dg_status dg_rk3_step_vjp(dg_mesh* m, const double* U0, double dt, const double*
     void** V = m->d_V;   // V0 = U0, V1 = lambda, V2 = U1, V3 = U2 (then result), V4 = m2, V5 = m1
     DG_CUDA(dg::launch_gather(m, U0, V[0], s));
     DG_CUDA(dg::launch_gather(m, lambda, V[1], s));
-    DG_CUDA(dg::launch_residual(m, V[0], nullptr, V[2], 1, dt, 0.0, 1.0, m->d_TA, s));
-    DG_CUDA(dg::launch_residual(m, V[2], V[0], V[3], 1, dt, 0.75, 0.25, m->d_TA, s));
+    DG_CUDA(dg::launch_residual(m, V[0], nullptr, V[2], 1, dt, 0.0, 1.0, inner_faces(m, m->d_TA), s));
+    DG_CUDA(dg::launch_residual(m, V[2], V[0], V[3], 1, dt, 0.75, 0.25, inner_faces(m, m->d_TA), s));
     const double c2[4] = {2.0 / 3.0, 0.0, 0.0, 2.0 / 3.0 * dt};   // m2 = 2/3 (lambda + dt J(U2)^T lambda)
     DG_CUDA(dg::launch_residual_vjp(m, V[3], V[1], V[1], nullptr, nullptr, c2, V[4], s));
     const double c1[4] = {0.25, 0.0, 0.0, 0.25 * dt};             // m1 = 1/4 (m2 + dt J(U1)^T m2)

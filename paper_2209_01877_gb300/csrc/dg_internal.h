@@ -108,15 +108,15 @@ struct dg_mesh {
     // one evaluation per face (FP64, FP32): the faces this mesh evaluates (boundary faces last) with
     // their owners' outward normals, the number of elements with traces (own + halo on a
     // partition's mesh), and the face buffers [n_trace][4][5][Nqf] (traces, then the fluxes in their
-    // place): d_T of the RK stages; FP32 (lazy): d_TW of the calls that leave a residual in d_W and
-    // d_TA of the adjoint, which stay independent of a step in progress (FP64: both are d_T); d_TL
-    // the adjoint direction's traces, d_fscale Real [n_flist][2] the two sides' |grad lambda| (lazy)
+    // place): d_T of the RK steps (FP64: of every residual) and d_TA of the adjoint (FP64: d_T too;
+    // FP32 lazy); d_TL the adjoint direction's traces, d_fscale Real [n_flist][2] the two sides'
+    // |grad lambda| (lazy)
     bool face_once = false;
     dg::FaceRec* d_frec = nullptr;
     void* d_fnorm = nullptr;       // Real [n_flist][3]
     int64_t n_flist = 0, n_interior = 0, n_trace = 0;   // listed faces, interior ones among them
     void* d_T = nullptr;
-    void *d_TW = nullptr, *d_TA = nullptr, *d_TL = nullptr, *d_fscale = nullptr;
+    void *d_TA = nullptr, *d_TL = nullptr, *d_fscale = nullptr;
     size_t face_bytes() const;
     // small meshes: a CUDA graph of several captured RK3 steps at one dt (dg_rk3_step)
     cudaStream_t cap_stream = nullptr;
@@ -139,6 +139,7 @@ cudaError_t launch_traces2(dg_mesh* m, const void* U, void* T, const void* U1, v
 // per listed face |grad lambda| of its slot and of the matching one, Real [n_flist][2]
 cudaError_t launch_face_scales(dg_mesh* m, void* out, cudaStream_t s);
 cudaError_t launch_gather(dg_mesh* m, const double* user, void* internal, cudaStream_t s);   // caller -> internal
+cudaError_t launch_gather_f32(dg_mesh* m, const double* user, float* internal, cudaStream_t s);   // FP32 (a hi plane) only
 // Navier-Stokes lines: the BR1 gradient into Z, then the viscous volume and face terms added to
 // the residual R (internal order), in the mesh's arithmetic (FP64 meshes FP64; FP32 and mixed
 // meshes FP32, U the state's hi plane); Z holds 15 Nb and HB ns_face_buffer_values values per

@@ -7,6 +7,7 @@
 #include <cmath>
 
 #include "dg_internal.h"
+#include "ff_bits.cuh"
 #include "modal_ops.cuh"
 
 namespace dg {
@@ -56,10 +57,15 @@ __global__ void __launch_bounds__(MT2) k_gather(const double* __restrict__ user,
             *reinterpret_cast<double2*>(static_cast<double*>(internal) + o) = x;
         } else {
             float* p = static_cast<float*>(internal) + o;
-            const float2 h = make_float2((float)x.x, (float)x.y);
-            *reinterpret_cast<float2*>(p) = h;
-            if (FMT == MOVE_FF)   // lo = fl32(x - hi)
-                *reinterpret_cast<float2*>(p + ne * NV) = make_float2((float)(x.x - (double)h.x), (float)(x.y - (double)h.y));
+            if (FMT == MOVE_FF) {
+                float2 h, l;
+                ff::split(x.x, h.x, l.x);
+                ff::split(x.y, h.y, l.y);
+                *reinterpret_cast<float2*>(p) = h;
+                *reinterpret_cast<float2*>(p + ne * NV) = l;
+            } else {
+                *reinterpret_cast<float2*>(p) = make_float2(ff::narrow(x.x), ff::narrow(x.y));
+            }
         }
     }
 }
@@ -83,11 +89,11 @@ __global__ void __launch_bounds__(MT2) k_scatter(const void* __restrict__ intern
         } else {
             const float* p = static_cast<const float*>(internal) + o;
             const float2 h = *reinterpret_cast<const float2*>(p);
-            x = make_double2((double)h.x, (double)h.y);
             if (FMT == MOVE_FF) {
                 const float2 l = *reinterpret_cast<const float2*>(p + ne * NV);
-                x.x += (double)l.x;
-                x.y += (double)l.y;
+                x = make_double2(ff::join(h.x, l.x), ff::join(h.y, l.y));
+            } else {
+                x = make_double2(ff::widen(h.x), ff::widen(h.y));
             }
         }
         store2<VEC>(user + (int64_t)sp[e] * NV + k, x);
@@ -353,12 +359,10 @@ __global__ void __launch_bounds__(128) k_ke_grad(const double* __restrict__ U, d
     double r[NB];
 #pragma unroll
     for (int j = 0; j < NB; ++j) r[j] = 0.0;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int m = modal::kT<P>.vmir[q];
-        if (m < q) continue;
-        modal::moments<double, P, NB>(q, sU[q][t], m != q ? sU[m][t] : 0.0, r);
-    }
+    modal::unroll<0, NQ>([&](auto qc) {
+        constexpr int q = qc.value, m = modal::kT<P>.vmir[q];
+        if constexpr (m >= q) modal::moments<double, P, NB>(q, sU[q][t], m != q ? sU[m][t] : 0.0, r);
+    });
 #pragma unroll
     for (int j = 0; j < NB; ++j) out[row * NB + j] = r[j];
     if (v == 3) {   // the energy row
@@ -376,6 +380,10 @@ int grid_for(int64_t n, int block) {
 
 cudaError_t launch_gather(dg_mesh* m, const double* user, void* internal, cudaStream_t s) {
     return move_state(m, true, format_of(m), user, internal, s);
+}
+
+cudaError_t launch_gather_f32(dg_mesh* m, const double* user, float* internal, cudaStream_t s) {
+    return move_state(m, true, MOVE_F32, user, internal, s);
 }
 
 cudaError_t launch_scatter(dg_mesh* m, const void* internal, double* user, cudaStream_t s) {

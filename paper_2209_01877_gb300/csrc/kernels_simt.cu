@@ -36,9 +36,10 @@ namespace {
 constexpr int NT = 256;
 
 // ---- FP32 without a face buffer ------------------------------------------------------------------
-// One persistent kernel per residual that evaluates every face from both sides; used only where the
-// face buffer (80 Nqf bytes per element) cannot be allocated: a P2 stage takes twice the time of the
-// face-once form below.
+// One persistent kernel per residual that evaluates every face from both sides: the calls that return
+// an FP32 residual (their values stay those of this order of summation), and RK stages where the face
+// buffer (80 Nqf bytes per element) cannot be allocated (a P2 stage takes two and a half times the
+// time of the face-once form below).
 
 template <int P> struct Tile;
 template <> struct Tile<1> { static constexpr int EPB = 32; };
@@ -466,16 +467,16 @@ __global__ void __launch_bounds__(threads_of(EE)) k_element(ResArgs<Real> a) {
     };
     if (live) {
         if (S::F32) flux(NQ, G0);
+        modal::unroll<0, NQ>([&](auto qc) {
+            constexpr int q = qc.value, m = modal::kT<P>.vmir[q];
+            if constexpr (m >= q) {
+                Real g[3], gm[3] = {0, 0, 0};
+                flux(q, g);
+                if (m != q) flux(m, gm);
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            const int m = modal::kT<P>.vmir[q];
-            if (m < q) continue;
-            Real g[3], gm[3] = {0, 0, 0};
-            flux(q, g);
-            if (m != q) flux(m, gm);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) modal::moments<Real, P, NM>(q, g[k], gm[k], M[k]);
-        }
+                for (int k = 0; k < 3; ++k) modal::moments<Real, P, NM>(q, g[k], gm[k], M[k]);
+            }
+        });
     }
     if (S::F32) {
         __syncthreads();

@@ -506,12 +506,11 @@ __global__ void __launch_bounds__(threads_of(EE)) k_element_vjp(VjpArgs<Real> a,
         }
         __syncthreads();
         if (live) {
-#pragma unroll
-            for (int q = q0; q < q1; ++q) {
-                const int m = modal::kT<P>.vmir[q];
-                if (m < q) continue;
-                modal::moments<Real, P, NB>(q, sU[(q - q0) * ER + t], m != q ? sU[(m - q0) * ER + t] : Real(0), r);
-            }
+            modal::unroll<q0, q1>([&](auto qc) {
+                constexpr int q = qc.value, m = modal::kT<P>.vmir[q];
+                if constexpr (m >= q)
+                    modal::moments<Real, P, NB>(q, sU[(q - q0) * ER + t], m != q ? sU[(m - q0) * ER + t] : Real(0), r);
+            });
         }
     };
     chunk(std::integral_constant<int, 0>());

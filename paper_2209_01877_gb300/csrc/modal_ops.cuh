@@ -27,6 +27,9 @@
 // the rules integrate exactly); entries that vanish identically are exact zeros and cost nothing.
 #pragma once
 
+#include <type_traits>
+#include <utility>
+
 #include "dg_device.h"
 #include "tc_ops.cuh"
 
@@ -232,6 +235,18 @@ struct Tables {
 
 template <int P> static __device__ constexpr Tables<P> kT{};
 
+// f(integral_constant First), ..., f(integral_constant Last - 1): a loop whose index stays a constant
+// however large the body is (where a nest is too large for the compiler's unrolling, table entries
+// would become loads and conversions)
+template <int First, typename F, int... I>
+__device__ __forceinline__ void unroll_seq(F&& f, std::integer_sequence<int, I...>) {
+    (f(std::integral_constant<int, First + I>()), ...);
+}
+template <int First, int Last, typename F>
+__device__ __forceinline__ void unroll(F&& f) {
+    unroll_seq<First>(f, std::make_integer_sequence<int, Last - First>());
+}
+
 // r += c x with a compile-time constant; nothing where it is zero
 template <typename Real>
 __device__ __forceinline__ void axpy(Real& r, double c, Real x) {
@@ -242,24 +257,24 @@ __device__ __forceinline__ void axpy(Real& r, double c, Real x) {
 // modes, store(q, sum_j c[j] phi_j(x_q))
 template <typename Real, int P, int N, int Q0, int Q1, typename Store>
 __device__ __forceinline__ void interpolate(const Real* c, Store store) {
-    constexpr auto& T = kT<P>;
+    unroll<Q0, Q1>([&](auto qc) {
+        constexpr auto& T = kT<P>;
+        constexpr int q = qc.value, m = T.vmir[q];
+        if constexpr (m >= q) {
+            Real e = 0, o = 0;
 #pragma unroll
-    for (int q = Q0; q < Q1; ++q) {
-        const int m = T.vmir[q];
-        if (m < q) continue;
-        Real e = 0, o = 0;
-#pragma unroll
-        for (int j = N - 1; j >= 0; --j) {
-            if (!T.odd[j]) axpy(e, T.phi[q][j], c[j]);
-            else if (m != q) axpy(o, T.phi[q][j], c[j]);
+            for (int j = N - 1; j >= 0; --j) {
+                if (!T.odd[j]) axpy(e, T.phi[q][j], c[j]);
+                else if (m != q) axpy(o, T.phi[q][j], c[j]);
+            }
+            if constexpr (m == q) {
+                store(q, e);
+            } else {
+                store(q, e + o);
+                store(m, e - o);
+            }
         }
-        if (m == q) {
-            store(q, e);
-        } else {
-            store(q, e + o);
-            store(m, e - o);
-        }
-    }
+    });
 }
 
 // S[m] += sum over the point q and its mirror point of w phi_m g, for the modes of degree <= p - 1
@@ -338,6 +353,18 @@ __device__ __forceinline__ void face_moments(const Real* h, Real* b) {
             else if (n != q) axpy(b[m], T.wf[q] * T.psi[q][m], d);
         }
     }
+}
+
+// y[j] = sum_m E_f[m][j] b[m]: face f's lift of its moments
+template <typename Real, int P>
+__device__ __forceinline__ void face_lift(int f, const Real* b, Real* y) {
+    constexpr auto& T = kT<P>;
+#pragma unroll
+    for (int j = 0; j < T.NB; ++j) y[j] = 0;
+#pragma unroll
+    for (int m = 0; m < T.NF; ++m)
+#pragma unroll
+        for (int j = 0; j < T.NB; ++j) axpy(y[j], T.E[f][m][j], b[m]);
 }
 
 // traces at the points of the 4 faces; store(f, u) receives each face's NQF values

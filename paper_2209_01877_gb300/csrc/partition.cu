@@ -255,10 +255,10 @@ dg_status dg_partition_create(dg_mesh* m, int k, void* stream, dg_partition** ou
             PTRY(upload_vec(&sm->d_mhdr, hdr, s));
             PTRY(upload_vec(&sm->d_mxnbr, xnbr, s));
         }
-        // face-once form, with the whole mesh's owners and normals; the faces shared with halo elements
+        // FP64: the face-once form, with the whole mesh's owners and normals; the faces shared with halo elements
         // are evaluated here too, in their owner's orientation, so every own element receives the
         // flux the whole mesh would give it
-        if (m->face_once) {
+        if (m->precision == DG_FP64) {
             std::vector<dg::FaceRec> rec;
             std::vector<int32_t> owner;
             dg::build_face_list(m->host, sm->host, pl.first, rec, owner);
