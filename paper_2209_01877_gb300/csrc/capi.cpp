@@ -75,6 +75,7 @@ void free_mesh(dg_mesh* m) {
     cudaFree(m->d_io);
     cudaFree(m->d_Z);
     cudaFree(m->d_HB);
+    if (m->d_TN != m->d_T) cudaFree(m->d_TN);
     cudaFree(m->d_hs);
     cudaFree(m->d_wslot);
     cudaFree(m->d_farea);
@@ -452,6 +453,8 @@ dg_status ensure_ns_buffers(dg_mesh* m) {
     const size_t rs = m->precision == DG_FP64 ? sizeof(double) : sizeof(float);
     if (!m->d_Z) DG_CUDA(cudaMalloc(&m->d_Z, (size_t)m->host.ne * 15 * m->nb * rs));
     if (!m->d_HB) DG_CUDA(cudaMalloc(&m->d_HB, dg::ns_face_buffer_values(m->p, m->host.ne) * rs));
+    if (m->precision == DG_FP64) m->d_TN = m->d_T;   // the Euler residual is done with it
+    if (m->precision == DG_FP32 && !m->d_TN) DG_CUDA(cudaMalloc(&m->d_TN, (size_t)m->host.ne * 20 * m->nqf * rs));
     return DG_OK;
 }
 }  // namespace
@@ -472,7 +475,7 @@ dg_status dg_ns_residual(dg_mesh* m, const double* U, double* R, double mu, doub
     if (mu > 0.0) {
         st = ensure_ns_buffers(m);
         if (st != DG_OK) return st;
-        DG_CUDA(dg::launch_ns_viscous(m, in, m->d_Z, m->d_HB, m->d_W[1], mu, prandtl, s));
+        DG_CUDA(dg::launch_ns_viscous(m, in, m->d_TN, m->d_Z, m->d_HB, m->d_W[1], mu, prandtl, s));
     }
     if (is_mixed(m)) DG_CUDA(dg::launch_scatter_f32(m, static_cast<const float*>(m->d_W[1]), R, s));
     else DG_CUDA(dg::launch_scatter(m, m->d_W[1], R, s));
@@ -649,7 +652,7 @@ dg_status dg_ns_rk3_step(dg_mesh* m, double dt, int nsteps, double mu, double pr
     for (int k = 0; k < nsteps; ++k)
         for (const auto& g : stages) {
             DG_CUDA(euler_residual_internal(m, B[g.in], R, inner_faces(m, m->d_T), s));
-            if (mu > 0.0) DG_CUDA(dg::launch_ns_viscous(m, B[g.in], m->d_Z, m->d_HB, R, mu, prandtl, s));
+            if (mu > 0.0) DG_CUDA(dg::launch_ns_viscous(m, B[g.in], m->d_TN, m->d_Z, m->d_HB, R, mu, prandtl, s));
             DG_CUDA(dg::launch_rk_axpy(m, B[g.in], g.base >= 0 ? B[g.base] : nullptr, R, B[g.out], dt, g.a, g.b, s));
         }
     return DG_OK;

@@ -97,7 +97,8 @@ struct dg_mesh {
     double* h_red = nullptr;       // pinned host reduction result
     unsigned int* d_status = nullptr;
     double* d_Z = nullptr;         // Navier-Stokes auxiliary gradient [ne][3][5][Nb] (lazy)
-    double* d_HB = nullptr;        // Navier-Stokes own viscous face fluxes [ne][4][Nqf][4] (lazy)
+    double* d_HB = nullptr;        // Navier-Stokes own viscous face fluxes [ne][4][4][Nqf] (lazy)
+    void* d_TN = nullptr;          // Navier-Stokes traces of U [ne][4][5][Nqf] (lazy)
     // mixed precision, conservative mode-0 update (dg_set_conservative): per (element, face) flux
     // integrals [ne][4][5]; per slot the weight phi_0 2|S_f| / |det J| of the mode-0 pass and the
     // face's 2|S_f| (one value per face, in both slots)
@@ -142,10 +143,12 @@ cudaError_t launch_gather(dg_mesh* m, const double* user, void* internal, cudaSt
 cudaError_t launch_gather_f32(dg_mesh* m, const double* user, float* internal, cudaStream_t s);   // FP32 (a hi plane) only
 // Navier-Stokes lines: the BR1 gradient into Z, then the viscous volume and face terms added to
 // the residual R (internal order), in the mesh's arithmetic (FP64 meshes FP64; FP32 and mixed
-// meshes FP32, U the state's hi plane); Z holds 15 Nb and HB ns_face_buffer_values values per
-// element of that type
-cudaError_t launch_ns_viscous(dg_mesh* m, const void* U, void* Z, void* HB, void* R, double mu, double prandtl,
+// meshes FP32, U the state's hi plane); per element of that type T holds 20 Nqf values (the traces
+// of U; the mixed forms need none), Z 15 Nb and HB ns_face_buffer_values
+cudaError_t launch_ns_viscous(dg_mesh* m, const void* U, void* T, void* Z, void* HB, void* R, double mu, double prandtl,
                               cudaStream_t s);
+cudaError_t launch_ns_viscous_mixed(dg_mesh* m, const float* U, float* Z, float* HB, float* R, double mu, double prandtl,
+                                    cudaStream_t s);
 size_t ns_face_buffer_values(int p, int64_t ne);
 // SSP-RK3 stage from a stored residual, out = a U0 + b (U + dt R), in the mesh's state format (the
 // mixed forms: float-float planes, FP32 residual)
