@@ -66,6 +66,8 @@
 #include "euler_device.cuh"
 #include "tc_ops.cuh"
 #include "mixed_common.cuh"
+#include "ff_bits.cuh"
+#include "launch.cuh"
 
 namespace dg {
 
@@ -311,6 +313,7 @@ __device__ __forceinline__ void elem_setup(const StageArgs& a, int64_t ge, int e
 
 template <int P, int FLUX, bool BF, bool CONS>
 __global__ void __launch_bounds__(SPlan<P>::MT, 1) k_stage_mixed(StageArgs a) {
+    pdl_trigger();   // the next stage's set-up may start as this one's blocks finish
     using S = SPlan<P>;
     constexpr int MT = S::MT;
     constexpr int NB = S::NB, NQ = S::NQ, NQF = S::NQF, NQF4 = S::NQF4, FPAD = S::FPAD;
@@ -382,6 +385,7 @@ __global__ void __launch_bounds__(SPlan<P>::MT, 1) k_stage_mixed(StageArgs a) {
     const int qq = wc & 3, part = wc >> 2;           // TMEM lane quarter (warp % 4), column part (0, 1)
     const uint32_t lane_base = (uint32_t)(qq * 32) << 16;
 
+    pdl_wait();   // the set-up above reads the mesh's tables only
     const int64_t ntiles = (a.ne + ET - 1) / ET;
     // tiles go round the CTAs first, so that a mesh of few tiles uses every SM
     const int64_t tstride = S::NCTX * (int64_t)gridDim.x;
@@ -833,8 +837,7 @@ cudaError_t slaunch1(const StageArgs& sa, cudaStream_t s, int nsm) {
         init = true;
     }
     const int64_t ntiles = (sa.ne + ET - 1) / ET;
-    k<<<(int)std::min<int64_t>(ntiles, (int64_t)nsm), S::MT, S::BYTES, s>>>(sa);
-    return cudaGetLastError();
+    return pdl_launch(k, (int)std::min<int64_t>(ntiles, (int64_t)nsm), S::MT, S::BYTES, s, sa);
 }
 
 // the conservative mode's stage kernel is a separate instantiation, so that the default one
@@ -1032,27 +1035,25 @@ __global__ void __launch_bounds__(256) k_cons_mode0(ConsArgs c) {
             // two sides still add exact negatives
             const float* oth = c.hs + ((int64_t)n * 4 + (c.fcode[e * 4 + f] & 3)) * 5;
 #pragma unroll
-            for (int v = 0; v < 5; ++v) R0[v] -= w * (double)(0.5f * (own[v] - oth[v]));
+            for (int v = 0; v < 5; ++v) R0[v] -= w * ff::widen(0.5f * (own[v] - oth[v]));
         } else {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) R0[v] -= w * (double)own[v];
+            for (int v = 0; v < 5; ++v) R0[v] -= w * ff::widen(own[v]);
         }
     }
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
         const int64_t k = (e * 5 + v) * c.nb;
         if (c.mode == 0) {
-            c.out_hi[k] = (float)R0[v];
+            c.out_hi[k] = ff::narrow(R0[v]);
             continue;
         }
         // float-float planes hold <= 48 bits, so hi + lo is exact in FP64
-        const double u = (double)c.U_hi[k] + (double)c.U_lo[k];
+        const double u = ff::join(c.U_hi[k], c.U_lo[k]);
         double x = u;
-        if (c.U0_hi) x += c.a * (((double)c.U0_hi[k] + (double)c.U0_lo[k]) - u);
+        if (c.U0_hi) x += c.a * (ff::join(c.U0_hi[k], c.U0_lo[k]) - u);
         x += c.bdt * R0[v];
-        const float h = (float)x;
-        c.out_hi[k] = h;
-        c.out_lo[k] = (float)(x - (double)h);
+        ff::split(x, c.out_hi[k], c.out_lo[k]);
     }
 }
 
