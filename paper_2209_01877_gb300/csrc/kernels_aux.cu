@@ -18,11 +18,11 @@ constexpr int RT = 256;   // reduction block size
 constexpr double SQRT6 = 2.449489742783178098197284;
 
 // ---- caller order <-> internal order ------------------------------------------------------------
-// A block moves 32 elements, a thread two values at a time, 16 bytes of the caller's FP64 array where
+// A block moves 32 elements (8 on a small mesh), a thread two values at a time, 16 bytes of the caller's FP64 array where
 // that is aligned (8 where a caller's pointer is not).  Bound by memory; one value per thread with a
 // 64-bit division per value was bound by issue: FP32 P3, 14,586 elements 12 us per call.
 enum { MOVE_F64 = 0, MOVE_F32 = 1, MOVE_FF = 2 };   // internal format; FF: hi plane, then lo plane
-constexpr int ME = 32, MT2 = 256;
+constexpr int MT2 = 256;
 
 template <bool VEC>
 __device__ __forceinline__ double2 load2(const double* p) {
@@ -39,7 +39,7 @@ __device__ __forceinline__ void store2(double* p, double2 x) {
     }
 }
 
-template <int NV, int FMT, bool VEC>
+template <int NV, int FMT, bool VEC, int ME>
 __global__ void __launch_bounds__(MT2) k_gather(const double* __restrict__ user, void* __restrict__ internal,
                                                 const int32_t* __restrict__ perm, int64_t ne) {
     constexpr int H = NV / 2;
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(MT2) k_gather(const double* __restrict__ user,
     }
 }
 
-template <int NV, int FMT, bool VEC>
+template <int NV, int FMT, bool VEC, int ME>
 __global__ void __launch_bounds__(MT2) k_scatter(const void* __restrict__ internal, double* __restrict__ user,
                                                  const int32_t* __restrict__ perm, int64_t ne) {
     constexpr int H = NV / 2;
@@ -100,20 +100,26 @@ __global__ void __launch_bounds__(MT2) k_scatter(const void* __restrict__ intern
     }
 }
 
-template <int NV, int FMT>
+template <int NV, int FMT, int ME>
 void move_elements(bool gather, const void* from, void* to, const int32_t* perm, int64_t ne, cudaStream_t s) {
     const unsigned grid = (unsigned)((ne + ME - 1) / ME);
     const void* user = gather ? from : to;
     const bool vec = (reinterpret_cast<uintptr_t>(user) & 15) == 0;
     if (gather) {
         const double* u = static_cast<const double*>(from);
-        if (vec) k_gather<NV, FMT, true><<<grid, MT2, 0, s>>>(u, to, perm, ne);
-        else k_gather<NV, FMT, false><<<grid, MT2, 0, s>>>(u, to, perm, ne);
+        if (vec) k_gather<NV, FMT, true, ME><<<grid, MT2, 0, s>>>(u, to, perm, ne);
+        else k_gather<NV, FMT, false, ME><<<grid, MT2, 0, s>>>(u, to, perm, ne);
     } else {
         double* u = static_cast<double*>(to);
-        if (vec) k_scatter<NV, FMT, true><<<grid, MT2, 0, s>>>(from, u, perm, ne);
-        else k_scatter<NV, FMT, false><<<grid, MT2, 0, s>>>(from, u, perm, ne);
+        if (vec) k_scatter<NV, FMT, true, ME><<<grid, MT2, 0, s>>>(from, u, perm, ne);
+        else k_scatter<NV, FMT, false, ME><<<grid, MT2, 0, s>>>(from, u, perm, ne);
     }
+}
+
+template <int NV, int FMT>
+void move_elements(bool gather, const void* from, void* to, const int32_t* perm, int64_t ne, cudaStream_t s) {
+    if (small_tiles(ne)) move_elements<NV, FMT, 8>(gather, from, to, perm, ne, s);
+    else move_elements<NV, FMT, 32>(gather, from, to, perm, ne, s);
 }
 
 cudaError_t move_state(const dg_mesh* m, bool gather, int fmt, const void* from, void* to, cudaStream_t s) {
@@ -158,6 +164,9 @@ __device__ __forceinline__ double det3(const double* I) {
     return I[0] * (I[4] * I[8] - I[5] * I[7]) - I[1] * (I[3] * I[8] - I[5] * I[6]) + I[2] * (I[3] * I[7] - I[4] * I[6]);
 }
 
+__device__ __forceinline__ double to_double(double x) { return x; }
+__device__ __forceinline__ double to_double(float x) { return ff::widen(x); }
+
 template <typename Real>
 __global__ void __launch_bounds__(RT) k_dt_local(const Real* __restrict__ U, const Real* __restrict__ Ulo,
                                                  const double* __restrict__ jinv, int64_t ne,
@@ -168,7 +177,7 @@ __global__ void __launch_bounds__(RT) k_dt_local(const Real* __restrict__ U, con
     for (int64_t e = blockIdx.x * (int64_t)RT + threadIdx.x; e < ne; e += (int64_t)gridDim.x * RT) {
         double m[5];
         for (int v = 0; v < 5; ++v)   // element means
-            m[v] = SQRT6 * ((double)U[(e * 5 + v) * nb] + (Ulo ? (double)Ulo[(e * 5 + v) * nb] : 0.0));
+            m[v] = SQRT6 * (to_double(U[(e * 5 + v) * nb]) + (Ulo ? to_double(Ulo[(e * 5 + v) * nb]) : 0.0));
         const double rho = m[0];
         const double u2 = (m[1] * m[1] + m[2] * m[2] + m[3] * m[3]) / (rho * rho);
         const double pr = (gamma - 1.0) * (m[4] - 0.5 * rho * u2);
@@ -202,30 +211,34 @@ __global__ void __launch_bounds__(RT) k_min_final(const double* __restrict__ in,
 // a fixed order, a thread per element as far as the sums go.  The point values are a thread per
 // (element, point) from shared memory (coefficients converted to FP64 once): bound by the FP64 pipe.  A
 // thread per element reading tables and coefficients per point took 2.86 ms on 165,888 P3 elements in
-// the mixed form, waiting on memory.  Every operation and its order are that form's (the kinetic energy
-// is differenced at 1e-7 of the state by adjoint checks, which its last bit decides).
-template <typename Real, int P>
+// the mixed form, waiting on memory.  FP64 and FP32 meshes keep every operation of that form and its
+// order (adjoint checks difference the kinetic energy at 1e-7 of the state, which its last bit
+// decides); the mixed forms (FACTORED), which have no adjoint, interpolate a thread per (element,
+// density or momentum) row with the factored operator: 896 -> 540 us.
+template <typename Real, int P, bool FACTORED>
 struct IntPlan {
-    static constexpr int NB = nb_of(P), NQ = nq_of(P), SUB = 32, NR = 4 * NB;
-    // shared memory (doubles): coefficients of SUB elements (density and momenta), basis at the
-    // points [NB][NQ], per element and point the kinetic energy's term
-    static constexpr int PH = SUB * NR, TERM = PH + NB * NQ, REALS = TERM + RT * (NQ + 1);
+    static constexpr int NB = nb_of(P), NQ = nq_of(P), SUB = FACTORED ? 64 : 32, NR = 4 * NB;
+    // shared memory (doubles): coefficients of SUB elements (density and momenta) and the basis at the
+    // points [NB][NQ], or (FACTORED) the point values [NQ][RT]; per element and point the kinetic
+    // energy's term
+    static constexpr int PH = SUB * NR, TERM = FACTORED ? NQ * RT : PH + NB * NQ, REALS = TERM + RT * (NQ + 1);
     static constexpr size_t BYTES = REALS * sizeof(double);
 };
 
-template <typename Real, int P>
+template <typename Real, int P, bool FACTORED>
 __global__ void __launch_bounds__(RT) k_integrals_local(const Real* __restrict__ U, const Real* __restrict__ Ulo,
                                                         const double* __restrict__ jinv,
                                                         const double* __restrict__ tab, int64_t ne,
                                                         double* __restrict__ block_sum) {
-    using S = IntPlan<Real, P>;
+    using S = IntPlan<Real, P, FACTORED>;
     constexpr int NB = S::NB, NQ = S::NQ, SUB = S::SUB, NR = S::NR;
     constexpr TabLayout L(P);
     extern __shared__ double sm[];
     double *sC = sm, *sP = sm + S::PH, *sT = sm + S::TERM;
     __shared__ double red[6][RT];
     const int t = threadIdx.x;
-    for (int i = t; i < NB * NQ; i += RT) sP[i] = tab[L.phiq + i];
+    if (!FACTORED)
+        for (int i = t; i < NB * NQ; i += RT) sP[i] = tab[L.phiq + i];
     double acc[6] = {0, 0, 0, 0, 0, 0};
     for (int64_t base = blockIdx.x * (int64_t)RT; base < ne; base += (int64_t)gridDim.x * RT) {
         for (int sub = 0; sub < RT; sub += SUB) {
@@ -233,21 +246,39 @@ __global__ void __launch_bounds__(RT) k_integrals_local(const Real* __restrict__
             const int nel = ne - e0 < SUB ? (int)(ne - e0) : SUB;
             if (nel <= 0) break;
             __syncthreads();
-            for (int i = t; i < nel * NR; i += RT) {
-                const int e = i / NR, k = i - e * NR;
-                const int64_t at = (e0 + e) * 5 * NB + k;
-                sC[i] = (double)U[at] + (Ulo ? (double)Ulo[at] : 0.0);
+            if constexpr (FACTORED) {
+                if (t < 4 * nel) {
+                    const int64_t row = (e0 + (t >> 2)) * 5 + (t & 3);
+                    Real x[NB], y[NB];
+                    double c[NB];
+                    load_row<NB>(U + row * NB, x);
+                    load_row<NB>(Ulo + row * NB, y);
+#pragma unroll
+                    for (int j = 0; j < NB; ++j) c[j] = ff::join(x[j], y[j]);
+                    modal::interpolate<double, P, NB, 0, NQ>(c, [&](int q, double u) { sC[q * RT + t] = u; });
+                }
+            } else {
+                for (int i = t; i < nel * NR; i += RT) {
+                    const int e = i / NR, k = i - e * NR;
+                    const int64_t at = (e0 + e) * 5 * NB + k;
+                    sC[i] = to_double(U[at]) + (Ulo ? to_double(Ulo[at]) : 0.0);
+                }
             }
             __syncthreads();
             for (int i = t; i < nel * NQ; i += RT) {
-                const int e = i / NQ, q = i - e * NQ;
+                const int e = FACTORED ? i % nel : i / NQ, q = FACTORED ? i / nel : i - e * NQ;
                 double Uq[4];
+                if constexpr (FACTORED) {
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    double s = 0.0;
+                    for (int v = 0; v < 4; ++v) Uq[v] = sC[q * RT + 4 * e + v];
+                } else {
 #pragma unroll
-                    for (int j = 0; j < NB; ++j) s += sC[e * NR + v * NB + j] * sP[j * NQ + q];
-                    Uq[v] = s;
+                    for (int v = 0; v < 4; ++v) {
+                        double s = 0.0;
+#pragma unroll
+                        for (int j = 0; j < NB; ++j) s += sC[e * NR + v * NB + j] * sP[j * NQ + q];
+                        Uq[v] = s;
+                    }
                 }
                 sT[(sub + e) * (NQ + 1) + q] =
                     tab[L.wq + q] * 0.5 * (Uq[1] * Uq[1] + Uq[2] * Uq[2] + Uq[3] * Uq[3]) / Uq[0];
@@ -259,7 +290,7 @@ __global__ void __launch_bounds__(RT) k_integrals_local(const Real* __restrict__
             const double detJ = 1.0 / fabs(det3(jinv + 9 * e));
             const Real* c = U + e * 5 * NB;
             const Real* cl = Ulo ? Ulo + e * 5 * NB : nullptr;
-            for (int v = 0; v < 5; ++v) acc[v] += detJ * ((double)c[v * NB] + (cl ? (double)cl[v * NB] : 0.0)) / SQRT6;
+            for (int v = 0; v < 5; ++v) acc[v] += detJ * (to_double(c[v * NB]) + (cl ? to_double(cl[v * NB]) : 0.0)) / SQRT6;
             double ke = 0.0;
             for (int q = 0; q < NQ; ++q) ke += sT[t * (NQ + 1) + q];
             acc[5] += detJ * ke;
@@ -410,10 +441,10 @@ cudaError_t launch_stable_dt(dg_mesh* m, const void* U, double* d_out, cudaStrea
     return cudaGetLastError();
 }
 
-template <typename Real, int P>
+template <typename Real, int P, bool FACTORED>
 static cudaError_t integrals_local(dg_mesh* m, const Real* U, const Real* Ulo, int nblk, cudaStream_t s) {
-    constexpr size_t bytes = IntPlan<Real, P>::BYTES;
-    auto kern = k_integrals_local<Real, P>;
+    constexpr size_t bytes = IntPlan<Real, P, FACTORED>::BYTES;
+    auto kern = k_integrals_local<Real, P, FACTORED>;
     static bool init = false;
     if (!init) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -429,9 +460,10 @@ cudaError_t launch_integrals(dg_mesh* m, const void* U, double* d_out6, cudaStre
     const int64_t n = m->host.ne * 5 * m->nb;
     auto go = [&](auto p) {
         constexpr int P = decltype(p)::value;
-        if (m->precision == DG_FP64) return integrals_local<double, P>(m, static_cast<const double*>(U), nullptr, nblk, s);
+        if (m->precision == DG_FP64) return integrals_local<double, P, false>(m, static_cast<const double*>(U), nullptr, nblk, s);
         const float* u = static_cast<const float*>(U);
-        return integrals_local<float, P>(m, u, m->precision == DG_FP32 ? nullptr : u + n, nblk, s);
+        if (m->precision == DG_FP32) return integrals_local<float, P, false>(m, u, nullptr, nblk, s);
+        return integrals_local<float, P, true>(m, u, u + n, nblk, s);
     };
     const cudaError_t e = m->p == 1 ? go(std::integral_constant<int, 1>())
                           : m->p == 2 ? go(std::integral_constant<int, 2>())
