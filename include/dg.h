@@ -168,8 +168,9 @@ dg_status dg_residual(dg_mesh* mesh, const double* U, double* R, void* stream);
  * precision: FP64 meshes in FP64; FP32 meshes in FP32; the mixed forms take
  * their Euler lines from the tensor-core kernel and the viscous lines in FP32
  * from the state's leading FP32 plane.  The first call with mu > 0 allocates
- * the gradient buffer (15 Nb values per element) and a face-flux buffer
- * (16 Nqf values per element), in that arithmetic, owned by the mesh. */
+ * the gradient buffer (15 Nb values per element), a face-flux buffer
+ * (16 Nqf values per element) and, on FP32 meshes, a trace buffer (20 Nqf
+ * values per element), in that arithmetic, owned by the mesh. */
 dg_status dg_ns_residual(dg_mesh* mesh, const double* U, double* R, double mu, double prandtl, void* stream);
 
 /* nsteps SSP-RK3 steps of the Navier-Stokes equations on the internal state, in
@@ -249,7 +250,9 @@ dg_status dg_boundary_flux(dg_mesh* mesh, const double* U, int stage, double out
  * inverse mass, projection, pointwise flux and Riemann-solver Jacobians,
  * interpolation, on both sides of every face; at a kink of |.| or max the
  * derivative of the branch taken, ties to the interior side).  U, lambda,
- * out: device FP64 [ne][5][Nb] in caller order. */
+ * out: device FP64 [ne][5][Nb] in caller order.  The first call allocates the
+ * adjoint's work buffers (six of the state's size and two of 20 Nqf values per
+ * element), owned by the mesh. */
 dg_status dg_residual_vjp(dg_mesh* mesh, const double* U, const double* lambda, double* out, void* stream);
 
 /* out = (d U_{n+1} / d U_n)^T lambda for one SSP-RK3 step of size dt from

@@ -81,7 +81,7 @@ void free_mesh(dg_mesh* m) {
     cudaFree(m->d_farea);
     cudaFree(m->d_frec);
     cudaFree(m->d_fnorm);
-    if (m->d_TA != m->d_T) cudaFree(m->d_TA);
+    cudaFree(m->d_TA);
     cudaFree(m->d_TL);
     cudaFree(m->d_fscale);
     cudaFree(m->d_T);
@@ -233,7 +233,6 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
             free_mesh(m);
             return cuda_fail(e, "face buffers");
         }
-        if (m->precision == DG_FP64) m->d_TA = m->d_T;
     }
     if (m->precision == DG_FP64) {
         m->d_tab = m->d_tab64;   // shared; freed once below
@@ -735,7 +734,8 @@ namespace {
 dg_status ensure_adjoint_buffers(dg_mesh* m, cudaStream_t s) {
     for (auto& b : m->d_V)
         if (!b) DG_CUDA(cudaMalloc(&b, m->state_bytes() + 256));
-    dg_status st = m->precision == DG_FP64 ? DG_OK : ensure_face_buffer(m, m->d_TA, m->face_bytes());
+    // buffers apart from the RK steps', so that an adjoint call leaves a step on another stream alone
+    dg_status st = ensure_face_buffer(m, m->d_TA, m->face_bytes());
     if (st == DG_OK) st = ensure_face_buffer(m, m->d_TL, m->face_bytes());
     if (st != DG_OK || !m->face_once || m->d_fscale) return st;
     st = ensure_face_buffer(m, m->d_fscale, (size_t)std::max<int64_t>(m->n_flist, 1) * 2 * (m->precision == DG_FP64 ? 8 : 4));

@@ -109,9 +109,8 @@ struct dg_mesh {
     // one evaluation per face (FP64, FP32): the faces this mesh evaluates (boundary faces last) with
     // their owners' outward normals, the number of elements with traces (own + halo on a
     // partition's mesh), and the face buffers [n_trace][4][5][Nqf] (traces, then the fluxes in their
-    // place): d_T of the RK steps (FP64: of every residual) and d_TA of the adjoint (FP64: d_T too;
-    // FP32 lazy); d_TL the adjoint direction's traces, d_fscale Real [n_flist][2] the two sides'
-    // |grad lambda| (lazy)
+    // place): d_T of the RK steps (FP64: of every residual); lazy, the adjoint's own: d_TA, d_TL the
+    // direction's traces, d_fscale Real [n_flist][2] the two sides' |grad lambda|
     bool face_once = false;
     dg::FaceRec* d_frec = nullptr;
     void* d_fnorm = nullptr;       // Real [n_flist][3]
