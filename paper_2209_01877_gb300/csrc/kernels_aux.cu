@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(RT) k_min_final(const double* __restrict__ in,
 // the mixed form, waiting on memory.  FP64 and FP32 meshes keep every operation of that form and its
 // order (adjoint checks difference the kinetic energy at 1e-7 of the state, which its last bit
 // decides); the mixed forms (FACTORED), which have no adjoint, interpolate a thread per (element,
-// density or momentum) row with the factored operator: 896 -> 540 us.
+// density or momentum) row with the factored operator: 896 -> 600 us.
 template <typename Real, int P, bool FACTORED>
 struct IntPlan {
     static constexpr int NB = nb_of(P), NQ = nq_of(P), SUB = FACTORED ? 64 : 32, NR = 4 * NB;

@@ -119,8 +119,8 @@ struct SPlan {
     static constexpr int C_D1 = 0, C_D2 = r16(N1);
     // contexts of the CTA: three where shared memory and the 512 tensor-memory columns hold them (80
     // registers a thread then; P3 holds two).  A context's tile is a chain of phases of about 4 us
-    // whatever the order, so more chains per SM hide more of it: P1, 48,000 elements, 54 -> 42 us per
-    // stage; P2, 663,552 elements, 883 -> 740 us
+    // whatever the order, so more chains per SM hide more of it: P1, 48,000 elements, 54 -> 44 us per
+    // stage; P2, 663,552 elements, 883 -> 725 us
     static constexpr int NCTX = P < 3 ? 3 : 2, MT = NCTX * CT;
     static constexpr int CTX_COLS = P == 1 ? 64 : P == 2 ? 160 : 256, TMEM_COLS = P == 1 ? 256 : 512;
     static_assert(C_D2 + NCH * 2 * N2 <= CTX_COLS && NCTX * CTX_COLS <= TMEM_COLS, "tensor memory");

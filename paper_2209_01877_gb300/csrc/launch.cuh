@@ -3,9 +3,10 @@
 // completed and its writes are visible.  pdl_trigger() lets a successor started the same way in from
 // the moment all of a kernel's blocks are resident.
 // Used by the mixed stage kernel, whose set-up (tables, cleared operands, tensor memory) reads nothing
-// an earlier kernel writes: P1, 960 elements, 9 steps 200 -> 158 us; P1, 48,000 elements, 16 steps
-// 2.04 -> 1.95 ms; P3, 1,572,864 elements, unchanged.  The CUDA-core kernels have no such set-up and ran
-// slower with it (FP64 P1, 1,296 elements, 10 steps 542 -> 1,423 us; FP32 P2 2.51 -> 2.79 ms).
+// an earlier kernel writes: P1, 48,000 elements, 16 steps 2.04 -> 1.95 ms; P1, 960 elements, 9 steps
+// 205 -> 158 us together with the third context; P3, 1,572,864 elements, unchanged.  The CUDA-core
+// kernels have no such set-up and ran slower with it (FP64 P1, 1,296 elements, 10 steps 542 -> 1,423 us;
+// FP32 P2 2.51 -> 2.79 ms).
 #pragma once
 
 #include <cuda_runtime.h>
