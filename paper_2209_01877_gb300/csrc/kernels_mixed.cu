@@ -288,7 +288,7 @@ __device__ __forceinline__ void elem_setup(const StageArgs& a, int64_t ge, int e
 #pragma unroll
     for (int t = 0; t < 9; ++t) I[t] = __ldg(Ig + t);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) ub[v] = 2.449489743f * __ldg(a.U_hi + (ge * 5 + v) * NB);
+    for (int v = 0; v < 5; ++v) ub[v] = 2.449489743f * a.U_hi[(ge * 5 + v) * NB];
     const float ts = elem_flux_scale(ub, I, gamma);
 #pragma unroll
     for (int t = 0; t < 9; ++t) {
@@ -718,11 +718,11 @@ __global__ void __launch_bounds__(SPlan<P>::MT, 1) k_stage_mixed(StageArgs a) {
                 for (int pl = 0; pl < 4; ++pl) {
                     if (pl >= npl) break;
                     if (pair_in) {
-                        const float2 t2 = __ldg(reinterpret_cast<const float2*>(pls[pl] + g + j0));
+                        const float2 t2 = *reinterpret_cast<const float2*>(pls[pl] + g + j0);
                         u[rr][pl][0] = t2.x;
                         u[rr][pl][1] = t2.y;
                     }
-                    if (one_in) u[rr][pl][2] = __ldg(pls[pl] + g + j1);
+                    if (one_in) u[rr][pl][2] = pls[pl][g + j1];
                 }
             }
         }

@@ -1,6 +1,8 @@
 // Programmatic dependent launch: a kernel started by pdl_launch may become resident while its
 // predecessor on the stream drains; its pdl_wait() holds each thread until every earlier kernel has
-// completed and its writes are visible.  pdl_trigger() lets a successor started the same way in from
+// completed and its writes are visible.  What an earlier kernel writes is read after it and by plain
+// loads or cp.async, never by __ldg: the read-only path promises data that does not change during the
+// kernel, which here begins before its predecessor ends.  pdl_trigger() lets a successor started the same way in from
 // the moment all of a kernel's blocks are resident.
 // Used by the mixed stage kernel, whose set-up (tables, cleared operands, tensor memory) reads nothing
 // an earlier kernel writes: P1, 48,000 elements, 16 steps 2.04 -> 1.95 ms; P1, 960 elements, 9 steps

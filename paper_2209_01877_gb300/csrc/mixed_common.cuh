@@ -202,13 +202,13 @@ __device__ __forceinline__ bool roe_f32(const float UL[5], const float UR[5], co
 // split-f16 operand row from Nb FP32 coefficients: modes 1.. scaled by a power of two that brings
 // their largest magnitude into [8, 16); returns (mean = sqrt6 c_0, inv_beta1 / scale), the factors
 // that turn the row's MMA result (against the beta1-scaled table) into point values
-template <int NB, int K1, bool BF, bool GLOBAL = true>
-__device__ __forceinline__ float2 build_row(const float* __restrict__ c, __half* A, int r, float inv_beta1) {
+template <int NB, int K1, bool BF>
+__device__ __forceinline__ float2 build_row(const float* c, __half* A, int r, float inv_beta1) {
     float x[NB];
     if constexpr (NB % 4 == 0) {
 #pragma unroll
         for (int j = 0; j < NB; j += 4) {
-            const float4 t = GLOBAL ? __ldg(reinterpret_cast<const float4*>(c + j)) : *reinterpret_cast<const float4*>(c + j);
+            const float4 t = *reinterpret_cast<const float4*>(c + j);
             x[j] = t.x;
             x[j + 1] = t.y;
             x[j + 2] = t.z;
@@ -216,7 +216,7 @@ __device__ __forceinline__ float2 build_row(const float* __restrict__ c, __half*
         }
     } else {
 #pragma unroll
-        for (int j = 0; j < NB; ++j) x[j] = GLOBAL ? __ldg(c + j) : c[j];
+        for (int j = 0; j < NB; ++j) x[j] = c[j];
     }
     float mx = 0.f;
 #pragma unroll
