@@ -83,7 +83,6 @@ void free_mesh(dg_mesh* m) {
     cudaFree(m->d_fnorm);
     cudaFree(m->d_TA);
     cudaFree(m->d_TL);
-    cudaFree(m->d_fscale);
     cudaFree(m->d_T);
     if (m->rk_exec) cudaGraphExecDestroy(m->rk_exec);
     if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
@@ -731,18 +730,12 @@ dg_status dg_applied_boundary_flux(dg_mesh* m, double out[5], void* stream) {
 }
 
 namespace {
-dg_status ensure_adjoint_buffers(dg_mesh* m, cudaStream_t s) {
+dg_status ensure_adjoint_buffers(dg_mesh* m) {
     for (auto& b : m->d_V)
         if (!b) DG_CUDA(cudaMalloc(&b, m->state_bytes() + 256));
     // buffers apart from the RK steps', so that an adjoint call leaves a step on another stream alone
     dg_status st = ensure_face_buffer(m, m->d_TA, m->face_bytes());
     if (st == DG_OK) st = ensure_face_buffer(m, m->d_TL, m->face_bytes());
-    if (st != DG_OK || !m->face_once || m->d_fscale) return st;
-    st = ensure_face_buffer(m, m->d_fscale, (size_t)std::max<int64_t>(m->n_flist, 1) * 2 * (m->precision == DG_FP64 ? 8 : 4));
-    if (st == DG_OK && m->d_fscale) {
-        DG_CUDA(dg::launch_face_scales(m, m->d_fscale, s));
-        DG_CUDA(cudaStreamSynchronize(s));   // once per mesh: later calls may come on other streams
-    }
     return st;
 }
 }  // namespace
@@ -751,7 +744,7 @@ dg_status dg_residual_vjp(dg_mesh* m, const double* U, const double* lambda, dou
     if (!m || !U || !lambda || !out) return fail(DG_ERR_ARG, "mesh, U, lambda and out must be non-NULL");
     if (is_mixed(m)) return fail(DG_ERR_UNSUPPORTED, "the adjoint runs in FP64 or FP32 meshes");
     cudaStream_t s = as_stream(stream);
-    dg_status st = ensure_adjoint_buffers(m, s);
+    dg_status st = ensure_adjoint_buffers(m);
     if (st != DG_OK) return st;
     void** V = m->d_V;
     const double c[4] = {0.0, 0.0, 0.0, 1.0};
@@ -767,7 +760,7 @@ dg_status dg_rk3_step_vjp(dg_mesh* m, const double* U0, double dt, const double*
     if (is_mixed(m)) return fail(DG_ERR_UNSUPPORTED, "the adjoint runs in FP64 or FP32 meshes");
     if (!(dt >= 0.0)) return fail(DG_ERR_ARG, "dt must be >= 0");
     cudaStream_t s = as_stream(stream);
-    dg_status st = ensure_adjoint_buffers(m, s);
+    dg_status st = ensure_adjoint_buffers(m);
     if (st != DG_OK) return st;
     void** V = m->d_V;   // V0 = U0, V1 = lambda, V2 = U1, V3 = U2 (then result), V4 = m2, V5 = m1
     DG_CUDA(dg::launch_gather(m, U0, V[0], s));

@@ -110,13 +110,13 @@ struct dg_mesh {
     // their owners' outward normals, the number of elements with traces (own + halo on a
     // partition's mesh), and the face buffers [n_trace][4][5][Nqf] (traces, then the fluxes in their
     // place): d_T of the RK steps (FP64: of every residual); lazy, the adjoint's own: d_TA, d_TL the
-    // direction's traces, d_fscale Real [n_flist][2] the two sides' |grad lambda|
+    // direction's traces
     bool face_once = false;
     dg::FaceRec* d_frec = nullptr;
     void* d_fnorm = nullptr;       // Real [n_flist][3]
     int64_t n_flist = 0, n_interior = 0, n_trace = 0;   // listed faces, interior ones among them
     void* d_T = nullptr;
-    void *d_TA = nullptr, *d_TL = nullptr, *d_fscale = nullptr;
+    void *d_TA = nullptr, *d_TL = nullptr;
     size_t face_bytes() const;
     // small meshes: a CUDA graph of several captured RK3 steps at one dt (dg_rk3_step)
     cudaStream_t cap_stream = nullptr;
@@ -134,10 +134,10 @@ cudaError_t launch_residual(dg_mesh* m, const void* U, const void* U0, void* out
 // the face buffer of n_trace elements
 cudaError_t setup_face_once(dg_mesh* m, const std::vector<FaceRec>& rec, const std::vector<int32_t>& owner,
                             const double* d_jinv64_whole, int64_t n_trace, cudaStream_t s);
-// face traces of two states of the mesh's precision, into the face buffers T and T1
-cudaError_t launch_traces2(dg_mesh* m, const void* U, void* T, const void* U1, void* T1, cudaStream_t s);
-// per listed face |grad lambda| of its slot and of the matching one, Real [n_flist][2]
-cudaError_t launch_face_scales(dg_mesh* m, void* out, cudaStream_t s);
+// face traces of a state of the mesh's precision, into the face buffer T; the adjoint's: of U into T,
+// and of lam times each face's |grad lambda_f| into TL
+cudaError_t launch_traces(dg_mesh* m, const void* U, void* T, cudaStream_t s);
+cudaError_t launch_traces_vjp(dg_mesh* m, const void* U, void* T, const void* lam, void* TL, cudaStream_t s);
 cudaError_t launch_gather(dg_mesh* m, const double* user, void* internal, cudaStream_t s);   // caller -> internal
 cudaError_t launch_gather_f32(dg_mesh* m, const double* user, float* internal, cudaStream_t s);   // FP32 (a hi plane) only
 // Navier-Stokes lines: the BR1 gradient into Z, then the viscous volume and face terms added to

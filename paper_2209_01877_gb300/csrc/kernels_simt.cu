@@ -22,6 +22,7 @@
 // 1,296 elements 85 -> 62 us; FP32 P2 Rusanov, 663,552 elements, per stage 980 us (one kernel, each face
 // from both sides) -> 65 + 151 + 126 us.
 #include <algorithm>
+#include <type_traits>
 
 #include "dg_internal.h"
 #include "euler_device.cuh"
@@ -264,27 +265,51 @@ cudaError_t dispatch_flux(const ResArgs<Real>& args, int flux, bool rk, cudaStre
 constexpr int FT = 128;       // threads of k_faces; 32 where that would leave SMs without a block
 inline unsigned face_block(int64_t n) { return n < (int64_t)FT * 4 * 152 ? 32 : FT; }
 
+// |grad lambda_f| = 2 |S_f| / |det J| from the row-major J^-1
+__device__ __forceinline__ double face_scale(const double* I, int f) {
+    double g[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) g[d] = f == 0 ? -(I[d] + I[3 + d] + I[6 + d]) : I[3 * (f - 1) + d];
+    return sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+}
+
 // The trace of every (element, face, point) of one or (gridDim.y = 2) two states: thread per (element,
 // variable) row.  In FP32 the tile's
 // coefficients and traces pass through shared memory, so that the global accesses are whole lines:
 // rows written directly (24 to 48 bytes each) kept the load-store unit busy (P2, 663,552 elements:
 // 127 us at 39 % of the DRAM rate).  FP64 is bound by its pipe and writes its rows directly.
-template <typename Real, int P, int EE>
+// SCALED: the second state's traces are multiplied by |grad lambda_f| of the element's face (the
+// adjoint's direction), four square roots per element.
+template <typename Real, int P, int EE, bool SCALED>
 __global__ void __launch_bounds__(threads_of(EE), EE == 32 ? (sizeof(Real) == 8 ? (P == 3 ? 3 : P == 2 ? 6 : 10) : (P == 3 ? 5 : 10)) : 14)
-    k_traces(const Real* U0, Real* T0, const Real* U1, Real* T1, int64_t ne) {
+    k_traces(const Real* U0, Real* T0, const Real* U1, Real* T1, const double* __restrict__ jinv, int64_t ne) {
     constexpr int NB = nb_of(P), NQF = nqf_of(P), NT = threads_of(EE);
+    __shared__ Real sS[SCALED ? 4 * EE : 1];
     const Real* __restrict__ U = blockIdx.y == 0 ? U0 : U1;
     Real* __restrict__ T = blockIdx.y == 0 ? T0 : T1;
     const int t = threadIdx.x;
     const int64_t e0 = blockIdx.x * (int64_t)EE;
     const int nel = (ne - e0) < (int64_t)EE ? (int)(ne - e0) : EE;
     const int e = t / 5, v = t - 5 * e;
+    const bool scaled = SCALED && blockIdx.y == 1;
+    if (scaled) {
+        if (t < 4 * nel) sS[t] = (Real)face_scale(jinv + (e0 + (t >> 2)) * 9, t & 3);
+        __syncthreads();
+    }
+    // a face's traces, times its scale where one is asked for
+    auto put = [&](Real* o, int f, const Real* u) {
+        Real x[NQF];
+        const Real s = scaled ? sS[SCALED ? 4 * e + f : 0] : Real(1);
+#pragma unroll
+        for (int q = 0; q < NQF; ++q) x[q] = SCALED ? s * u[q] : u[q];
+        store_row<NQF>(o + f * 5 * NQF, x);
+    };
     if constexpr (sizeof(Real) == 8) {
         if (t >= 5 * nel) return;
         Real c[NB];
         load_row<NB>(U + (e0 * 5 + t) * NB, c);
         Real* o = T + ((e0 + e) * 20 + v) * NQF;
-        modal::traces<Real, P>(c, [&](int f, const Real* u) { store_row<NQF>(o + f * 5 * NQF, u); });
+        modal::traces<Real, P>(c, [&](int f, const Real* u) { put(o, f, u); });
     } else {
         __shared__ __align__(16) Real sU[rows_of(EE) * NB + 4], sT[EE * 20 * NQF];
         copy_tile<NT>(sU, U + e0 * 5 * NB, nel * 5 * NB * (int)sizeof(Real));
@@ -294,7 +319,7 @@ __global__ void __launch_bounds__(threads_of(EE), EE == 32 ? (sizeof(Real) == 8 
             Real c[NB];
             load_row<NB>(sU + t * NB, c);
             Real* o = sT + (e * 20 + v) * NQF;
-            modal::traces<Real, P>(c, [&](int f, const Real* u) { store_row<NQF>(o + f * 5 * NQF, u); });
+            modal::traces<Real, P>(c, [&](int f, const Real* u) { put(o, f, u); });
         }
         __syncthreads();
         float4* g = reinterpret_cast<float4*>(T + e0 * 20 * NQF);
@@ -302,14 +327,14 @@ __global__ void __launch_bounds__(threads_of(EE), EE == 32 ? (sizeof(Real) == 8 
     }
 }
 
-template <typename Real, int P>
-cudaError_t traces(const void* U, void* T, const void* U1, void* T1, int64_t ne, cudaStream_t s) {
+template <typename Real, int P, bool SCALED>
+cudaError_t traces(const void* U, void* T, const void* U1, void* T1, const double* jinv, int64_t ne, cudaStream_t s) {
     const Real *u = static_cast<const Real*>(U), *u1 = static_cast<const Real*>(U1);
     Real *t = static_cast<Real*>(T), *t1 = static_cast<Real*>(T1);
     if (small_tiles(ne))
-        k_traces<Real, P, 6><<<dim3((unsigned)((ne + 5) / 6), U1 ? 2 : 1), threads_of(6), 0, s>>>(u, t, u1, t1, ne);
+        k_traces<Real, P, 6, SCALED><<<dim3((unsigned)((ne + 5) / 6), U1 ? 2 : 1), threads_of(6), 0, s>>>(u, t, u1, t1, jinv, ne);
     else
-        k_traces<Real, P, 32><<<dim3((unsigned)((ne + 31) / 32), U1 ? 2 : 1), threads_of(32), 0, s>>>(u, t, u1, t1, ne);
+        k_traces<Real, P, 32, SCALED><<<dim3((unsigned)((ne + 31) / 32), U1 ? 2 : 1), threads_of(32), 0, s>>>(u, t, u1, t1, jinv, ne);
     return cudaGetLastError();
 }
 
@@ -567,7 +592,7 @@ cudaError_t launch_face_once(dg_mesh* m, ResArgs<Real>& r, bool rk, void* T, cud
     f.roe_eps = r.roe_eps;
     for (int v = 0; v < 5; ++v) f.finf[v] = r.finf[v];
     f.status = m->d_status;
-    cudaError_t e = traces<Real, P>(r.U, f.T, nullptr, nullptr, m->n_trace, s);
+    cudaError_t e = traces<Real, P, false>(r.U, f.T, nullptr, nullptr, nullptr, m->n_trace, s);
     if (e != cudaSuccess) return e;
     if (f.n > 0) {
         const unsigned nt = face_block(f.n), grid = (unsigned)((f.n + nt - 1) / nt);
@@ -638,31 +663,7 @@ __global__ void k_face_normals(const double* __restrict__ jinv, const int32_t* _
     const double gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
     for (int d = 0; d < 3; ++d) out[3 * i + d] = (Real)(-g[d] / gn);
 }
-
-template <typename Real>
-__global__ void k_face_scales(const double* __restrict__ jinv, const FaceRec* __restrict__ rec, int64_t n, Real* out) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    for (int side = 0; side < 2; ++side) {
-        const int32_t sl = side == 0 ? rec[i].slot : rec[i].other;
-        double g[3] = {0, 0, 0};
-        if (sl >= 0) {
-            const double* I = jinv + (int64_t)(sl >> 2) * 9;
-            const int f = sl & 3;
-            for (int d = 0; d < 3; ++d) g[d] = f == 0 ? -(I[d] + I[3 + d] + I[6 + d]) : I[3 * (f - 1) + d];
-        }
-        out[2 * i + side] = (Real)sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-    }
-}
 }  // namespace
-
-cudaError_t launch_face_scales(dg_mesh* m, void* out, cudaStream_t s) {
-    if (m->n_flist == 0) return cudaSuccess;
-    const unsigned grid = (unsigned)((m->n_flist + 255) / 256);
-    if (m->precision == DG_FP64) k_face_scales<double><<<grid, 256, 0, s>>>(m->d_jinv64, m->d_frec, m->n_flist, static_cast<double*>(out));
-    else k_face_scales<float><<<grid, 256, 0, s>>>(m->d_jinv64, m->d_frec, m->n_flist, static_cast<float*>(out));
-    return cudaGetLastError();
-}
 
 cudaError_t setup_face_once(dg_mesh* m, const std::vector<FaceRec>& rec, const std::vector<int32_t>& owner,
                             const double* d_jinv64_whole, int64_t n_trace, cudaStream_t s) {
@@ -696,14 +697,30 @@ cudaError_t setup_face_once(dg_mesh* m, const std::vector<FaceRec>& rec, const s
     return e;
 }
 
-cudaError_t launch_traces2(dg_mesh* m, const void* U, void* T, const void* U1, void* T1, cudaStream_t s) {
+cudaError_t launch_traces(dg_mesh* m, const void* U, void* T, cudaStream_t s) {
     const int64_t n = m->host.ne;
     const bool f64 = m->precision == DG_FP64;
-    switch (m->p) {
-        case 1: return f64 ? traces<double, 1>(U, T, U1, T1, n, s) : traces<float, 1>(U, T, U1, T1, n, s);
-        case 2: return f64 ? traces<double, 2>(U, T, U1, T1, n, s) : traces<float, 2>(U, T, U1, T1, n, s);
-        default: return f64 ? traces<double, 3>(U, T, U1, T1, n, s) : traces<float, 3>(U, T, U1, T1, n, s);
-    }
+    auto go = [&](auto p) {
+        constexpr int P = decltype(p)::value;
+        return f64 ? traces<double, P, false>(U, T, nullptr, nullptr, nullptr, n, s)
+                   : traces<float, P, false>(U, T, nullptr, nullptr, nullptr, n, s);
+    };
+    return m->p == 1 ? go(std::integral_constant<int, 1>())
+           : m->p == 2 ? go(std::integral_constant<int, 2>())
+                       : go(std::integral_constant<int, 3>());
+}
+
+cudaError_t launch_traces_vjp(dg_mesh* m, const void* U, void* T, const void* lam, void* TL, cudaStream_t s) {
+    const int64_t n = m->host.ne;
+    const bool f64 = m->precision == DG_FP64;
+    auto go = [&](auto p) {
+        constexpr int P = decltype(p)::value;
+        return f64 ? traces<double, P, true>(U, T, lam, TL, m->d_jinv64, n, s)
+                   : traces<float, P, true>(U, T, lam, TL, m->d_jinv64, n, s);
+    };
+    return m->p == 1 ? go(std::integral_constant<int, 1>())
+           : m->p == 2 ? go(std::integral_constant<int, 2>())
+                       : go(std::integral_constant<int, 3>());
 }
 
 cudaError_t launch_residual(dg_mesh* m, const void* U, const void* U0, void* out, int mode, double dt, double a,
