@@ -393,18 +393,26 @@ namespace {
 // and the faster form is used.
 void* residual_faces(const dg_mesh* m) { return m->precision == DG_FP64 ? m->d_T : nullptr; }
 
-// The face buffer of an FP32 RK stage, or null for the single kernel.  The single kernel is the faster one
-// while its tiles make one wave (P1, 900 elements: 75 us for two steps against 89 us for the three
-// launches; P3, 83,000 elements: 1,163 against 403 us).  On a mesh with boundary faces it is kept too:
-// dg_boundary_flux reports the boundary integral of the FP32 state in FP64, which shows the order of
-// summation at 1e-7.
-constexpr int64_t FP32_FACES_MIN_NE = 8192;
+// From how many elements on an FP32 stage of three launches is faster than the single kernel.  us per step, single
+// against three launches:
+//   P1, where the tiles of the single kernel make one wave up to 19,456 elements: Rusanov 16,464 38 : 50, 24,576
+//       50 : 50, 34,992 57 : 67, 48,000 75 : 78, 55,566 81 : 81, 82,944 112 : 107 (so from three waves on);
+//       Roe 16,464 38 : 50, 20,250 52 : 50, 34,992 62 : 65, 48,000 81 : 76 (from one wave on);
+//   P2: 8,712 58 : 55 (Rusanov), 62 : 55 (Roe), 12,168 77 : 57, 93,750 420 : 181;
+//   P3: 8,712 137 : 69, 93,750 1,150 : 353.
+int64_t fp32_faces_min_ne(const dg_mesh* m) {
+    if (m->p > 1) return 8192;
+    return m->flux == DG_ROE ? 19456 : 3 * 19456;
+}
+// The face buffer of an FP32 RK stage, or null for the single kernel.  On a mesh with boundary faces the
+// single kernel is kept: dg_boundary_flux reports the boundary integral of the FP32 state in FP64, which
+// shows the order of summation at 1e-7.
 void* stage_faces(const dg_mesh* m, void* T) {
-    return m->precision == DG_FP64 || (m->host.ne >= FP32_FACES_MIN_NE && !m->has_bc) ? T : nullptr;
+    return m->precision == DG_FP64 || (m->host.ne >= fp32_faces_min_ne(m) && !m->has_bc) ? T : nullptr;
 }
 // the same where no boundary integral is taken of the states: Navier-Stokes steps and the adjoint's stages
 void* inner_faces(const dg_mesh* m, void* T) {
-    return m->precision == DG_FP64 || m->host.ne >= FP32_FACES_MIN_NE ? T : nullptr;
+    return m->precision == DG_FP64 || m->host.ne >= fp32_faces_min_ne(m) ? T : nullptr;
 }
 
 // a caller's state as a residual's operand, in d_W[0]: the mixed forms' residual reads the hi plane
