@@ -738,9 +738,23 @@ dg_status dg_applied_boundary_flux(dg_mesh* m, double out[5], void* stream) {
 }
 
 namespace {
+// Whether the adjoint evaluates every face once (three launches, a fourth for boundary faces).  In FP32
+// the single kernel k_residual_vjp, whose tiles hold 16, 8, 4 elements, is faster while they are no
+// more than the SMs.  us per VJP, single against three launches, Rusanov | Roe | Rusanov with boundary
+// faces: P1 2,058 elements 23 : 25 | 23 : 25 | 23 : 32, 3,072 27 : 25 | 32 : 25 | 31 : 32; P2 750
+// 23 : 27 | 25 : 27 | 25 : 34, 1,296 30 : 27 | 34 : 28 | 34 : 34; P3 384 28 : 32 | 30 : 32 | 30 : 38,
+// 750 34 : 32 | 38 : 32 | 38 : 38.  With Rusanov and boundary faces the single kernel is ahead up to two
+// tiles per SM (P1 4,374 32 : 34, P2 2,058 34 : 35).
+bool vjp_by_faces(const dg_mesh* m) {
+    if (m->precision == DG_FP64) return true;
+    const int64_t wave = 152 * (m->p == 1 ? 16 : m->p == 2 ? 8 : 4);
+    return m->host.ne > (m->flux == DG_RUSANOV && m->has_bc ? 2 : 1) * wave;
+}
+
 dg_status ensure_adjoint_buffers(dg_mesh* m) {
     for (auto& b : m->d_V)
         if (!b) DG_CUDA(cudaMalloc(&b, m->state_bytes() + 256));
+    if (!vjp_by_faces(m)) return DG_OK;
     // buffers apart from the RK steps', so that an adjoint call leaves a step on another stream alone
     dg_status st = ensure_face_buffer(m, m->d_TA, m->face_bytes());
     if (st == DG_OK) st = ensure_face_buffer(m, m->d_TL, m->face_bytes());

@@ -32,7 +32,8 @@ namespace {
 constexpr int NT = 256;
 
 // ---- FP32 without face buffers: each element differentiates its faces from both sides in forward
-// mode; used only where the face buffers cannot be allocated
+// mode; the faster form on small meshes (capi.cpp has the rule), and the one that is left where the
+// face buffers cannot be allocated
 
 template <int P> struct VTile;
 template <> struct VTile<1> { static constexpr int EPB = 16; };
