@@ -455,12 +455,20 @@ cudaError_t euler_residual_internal(dg_mesh* m, const void* in, void* R, void* T
     return dg::launch_residual(m, in, nullptr, R, 0, 0.0, 0.0, 0.0, T, s);
 }
 
+// Whether the viscous passes take the traces of U (kernels_ns.cu); without them a mesh in FP32 arithmetic
+// runs the passes of the mixed forms, three launches instead of four, which are faster on small P1
+// meshes: us per residual, 1,296 elements 40 : 42, 4,374 with boundary faces 40 : 44, 6,000 44 : 44 and
+// equal or slower from there on; at P2 and P3 equal or slower at every size.
+bool ns_by_rows(const dg_mesh* m) {
+    return m->precision == DG_FP64 || (m->precision == DG_FP32 && (m->p > 1 || m->host.ne >= 6000));
+}
+
 dg_status ensure_ns_buffers(dg_mesh* m) {
     const size_t rs = m->precision == DG_FP64 ? sizeof(double) : sizeof(float);
     if (!m->d_Z) DG_CUDA(cudaMalloc(&m->d_Z, (size_t)m->host.ne * 15 * m->nb * rs));
     if (!m->d_HB) DG_CUDA(cudaMalloc(&m->d_HB, dg::ns_face_buffer_values(m->p, m->host.ne) * rs));
     if (m->precision == DG_FP64) m->d_TN = m->d_T;   // the Euler residual is done with it
-    if (m->precision == DG_FP32 && !m->d_TN) DG_CUDA(cudaMalloc(&m->d_TN, (size_t)m->host.ne * 20 * m->nqf * rs));
+    if (ns_by_rows(m) && m->precision == DG_FP32 && !m->d_TN) DG_CUDA(cudaMalloc(&m->d_TN, (size_t)m->host.ne * 20 * m->nqf * rs));
     return DG_OK;
 }
 }  // namespace

@@ -143,9 +143,11 @@ cudaError_t launch_gather_f32(dg_mesh* m, const double* user, float* internal, c
 // Navier-Stokes lines: the BR1 gradient into Z, then the viscous volume and face terms added to
 // the residual R (internal order), in the mesh's arithmetic (FP64 meshes FP64; FP32 and mixed
 // meshes FP32, U the state's hi plane); per element of that type T holds 20 Nqf values (the traces
-// of U; the mixed forms need none), Z 15 Nb and HB ns_face_buffer_values
+// of U; null for the passes that need none, which the mixed forms always take), Z 15 Nb and HB
+// ns_face_buffer_values
 cudaError_t launch_ns_viscous(dg_mesh* m, const void* U, void* T, void* Z, void* HB, void* R, double mu, double prandtl,
                               cudaStream_t s);
+// in FP32 without a trace buffer (mixed and FP32 meshes)
 cudaError_t launch_ns_viscous_mixed(dg_mesh* m, const float* U, float* Z, float* HB, float* R, double mu, double prandtl,
                                     cudaStream_t s);
 size_t ns_face_buffer_values(int p, int64_t ne);

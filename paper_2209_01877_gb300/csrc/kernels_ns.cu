@@ -1,6 +1,6 @@
 // Navier-Stokes lines of the weak form (Eq. 1 with ivis = 1; Eq. 11's auxiliary-gradient and
-// viscous-flux lines in BR1 form, Sec. II-B) on the CUDA cores, in FP64 or FP32 (the mixed forms:
-// kernels_ns_mixed.cu).  Three passes after
+// viscous-flux lines in BR1 form, Sec. II-B) on the CUDA cores, in FP64 or FP32 (the mixed forms and
+// FP32 without a trace buffer: kernels_ns_mixed.cu).  Three passes after
 // the Euler residual, on the traces of U at every face point ([ne][4][5][Nqf], kernels_simt.cu):
 //
 //   k_ns_grad   the auxiliary gradient Z = grad Q of Eq. 11's first line,
@@ -463,7 +463,7 @@ cudaError_t launch_rk_axpy(dg_mesh* m, const void* U, const void* U0, const void
 cudaError_t launch_ns_viscous(dg_mesh* m, const void* U, void* T, void* Z, void* HB, void* R, double mu, double prandtl,
                               cudaStream_t s) {
     if (m->precision == DG_FP64) return ns_dispatch<double>(m, U, T, Z, HB, R, mu, prandtl, s);
-    if (m->precision == DG_FP32) return ns_dispatch<float>(m, U, T, Z, HB, R, mu, prandtl, s);
+    if (m->precision == DG_FP32 && T) return ns_dispatch<float>(m, U, T, Z, HB, R, mu, prandtl, s);
     return launch_ns_viscous_mixed(m, static_cast<const float*>(U), static_cast<float*>(Z), static_cast<float*>(HB),
                                    static_cast<float*>(R), mu, prandtl, s);
 }
