@@ -402,6 +402,23 @@ __global__ void __launch_bounds__(FT) k_faces(FaceArgs<Real> a) {
     }
 }
 
+// contravariant velocity W_k = sum_d (J^-1)_kd u_d and pressure of the i-th (point, element) of a tile
+// (points from NQ on are no quadrature points: their states are not reported)
+template <typename Real, int EE, int ER>
+__device__ __forceinline__ void contravariant_point(const ResArgs<Real>& a, int nel, int i, int NQ, const Real* sU, Real* sW,
+                                                    const Real* sJ) {
+    const int e = i % EE, q = i / EE;
+    if (e >= nel) return;
+    const Real* u = sU + q * ER + 5 * e;
+    const Real rho = u[0], ri = recip(rho);
+    const Real x = u[1] * ri, y = u[2] * ri, z = u[3] * ri;
+    const Real p = (a.gamma - Real(1)) * (u[4] - Real(0.5) * (u[1] * x + u[2] * y + u[3] * z));
+    if (q < NQ && !(positive(rho) && positive(p))) atomicOr(a.status, 1u);
+    const Real* I = sJ + e * 9;
+    Real o[4] = {I[0] * x + I[1] * y + I[2] * z, I[3] * x + I[4] * y + I[5] * z, I[6] * x + I[7] * y + I[8] * z, p};
+    store_row<4>(sW + (q * EE + e) * 4, o);
+}
+
 template <typename Real, int P, int EE>
 struct ElemPlan {
     // FP32 projects the deviation from the flux of the element's mean state, which is point NQ, and
@@ -459,19 +476,7 @@ __global__ void __launch_bounds__(threads_of(EE)) k_element(ResArgs<Real> a) {
         for (int d = 0; d < 3; ++d) g[d] = f == 0 ? -(I[d] + I[3 + d] + I[6 + d]) : I[3 * (f - 1) + d];
         sG[t] = EulerOps<Real>::sqrt_(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
     }
-    // contravariant velocity W_k = sum_d (J^-1)_kd u_d and pressure at every (element, point)
-    for (int i = t; i < S::NP * EE; i += NT) {
-        const int e = i % EE, q = i / EE;
-        if (e >= nel) continue;
-        const Real* u = sU + q * ER + 5 * e;
-        const Real rho = u[0], ri = recip(rho);
-        const Real x = u[1] * ri, y = u[2] * ri, z = u[3] * ri;
-        const Real p = (a.gamma - Real(1)) * (u[4] - Real(0.5) * (u[1] * x + u[2] * y + u[3] * z));
-        if (q < NQ && !(positive(rho) && positive(p))) atomicOr(a.status, 1u);
-        const Real* I = sJ + e * 9;
-        Real o[4] = {I[0] * x + I[1] * y + I[2] * z, I[3] * x + I[4] * y + I[5] * z, I[6] * x + I[7] * y + I[8] * z, p};
-        store_row<4>(sW + (q * EE + e) * 4, o);
-    }
+    for (int i = t; i < S::NP * EE; i += NT) contravariant_point<Real, EE, ER>(a, nel, i, NQ, sU, sW, sJ);
     __syncthreads();
     const int e = t / 5, v = t - 5 * e;
     // G_k of variable v: W_k b + p J_k, b = U_v (+ p for the energy), J_k = (J^-1)_k,v-1 for a momentum
@@ -486,9 +491,9 @@ __global__ void __launch_bounds__(threads_of(EE)) k_element(ResArgs<Real> a) {
     auto flux = [&](int q, Real* g) {
         Real w[4];
         load_row<4>(sW + (q * EE + e) * 4, w);
-        const Real b = sU[q * ER + t] + s4 * w[3];
+        const Real b = fma(s4, w[3], sU[q * ER + t]);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) g[k] = w[k] * b + (w[3] * Jk[k] - G0[k]);
+        for (int k = 0; k < 3; ++k) g[k] = fma(w[k], b, fma(w[3], Jk[k], -G0[k]));
     };
     if (live) {
         if (S::F32) flux(NQ, G0);
@@ -575,8 +580,135 @@ cudaError_t launch_tiles(const ResArgs<Real>& r, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// Four warps share the rows of a tile of 6 elements (FP64).  A scheduler's FP64 pipe takes a warp's
+// instruction every 64 clocks however many of its lanes are active, so on a mesh of few tiles the time
+// is the instruction count of one warp: each of the four interpolates to a quarter of the volume points;
+// three take one component of the flux's moments each and the fourth the face moments; each
+// sums a quarter of the modes.  Every sum runs in the order of k_element, with the same fused operations,
+// so the results are bitwise its own (a partition may take this kernel where the whole mesh does not).
+// P3 (one warp per tile before), 162 elements: 72 -> 31 us, an SSP-RK3 step 282 -> 176 us; 1,296: 298 -> 232; 2,058:
+// 316 -> 300; 3,072: 372 -> 391, so the line lies between, at two and a half tiles per SM.
+constexpr int WIDE = 4;
+constexpr int64_t WIDE_MAX_NE = 16 * 152;
+
+// f(integral_constant w) for a warp's number w < WIDE
+template <typename F>
+__device__ __forceinline__ void by_warp(int w, F&& f) {
+    if (w == 0) f(std::integral_constant<int, 0>());
+    else if (w == 1) f(std::integral_constant<int, 1>());
+    else if (w == 2) f(std::integral_constant<int, 2>());
+    else f(std::integral_constant<int, 3>());
+}
+
+template <int P, bool RK>
+__global__ void __launch_bounds__(32 * WIDE) k_element_wide(ResArgs<double> a) {
+    using Real = double;
+    constexpr int EE = 6, ER = rows_of(EE), NT = 32 * WIDE;
+    constexpr int NB = nb_of(P), NQ = nq_of(P), NQF = nqf_of(P), NM = modal::Tables<P>::NM, NF = modal::Tables<P>::NF;
+    __shared__ __align__(16) Real sW[NQ * EE * 4];           // (W_0, W_1, W_2, p) at the points
+    __shared__ Real sU[NQ * ER], sM[3 * NM * ER], sA[4 * NF * ER], sJ[EE * 9], sG[EE * 4];
+    const int t = threadIdx.x, w = t >> 5, l = t & 31;
+    const int64_t e0 = blockIdx.x * (int64_t)EE;
+    const int nel = (a.ne - e0) < (int64_t)EE ? (int)(a.ne - e0) : EE;
+    const bool live = l < 5 * nel;
+    const int64_t row = e0 * 5 + l;
+    const int e = l / 5, v = l - 5 * e;
+    for (int i = t; i < nel * 9; i += NT) sJ[i] = a.jinv[e0 * 9 + i];
+    if (live) {
+        Real c[NB];
+        load_row<NB>(a.U + row * NB, c);
+        by_warp(w, [&](auto wc) {
+            modal::interpolate<Real, P, NB, 0, NQ, wc.value, WIDE>(c, [&](int q, Real u) { sU[q * ER + l] = u; });
+        });
+    }
+    __syncthreads();
+    if (t < nel * 4) sG[t] = face_scale(sJ + (t >> 2) * 9, t & 3);
+    for (int i = t; i < NQ * EE; i += NT) contravariant_point<Real, EE, ER>(a, nel, i, NQ, sU, sW, sJ);
+    __syncthreads();
+    if (live && w < 3) {
+        const Real s4 = v == 4 ? Real(1) : Real(0), Jk = v >= 1 && v <= 3 ? sJ[e * 9 + 3 * w + v - 1] : Real(0), G0 = 0;
+        Real M[NM];
+#pragma unroll
+        for (int m = 0; m < NM; ++m) M[m] = 0;
+        auto flux = [&](int q) {
+            const Real wk = sW[(q * EE + e) * 4 + w], p = sW[(q * EE + e) * 4 + 3];
+            return fma(wk, fma(s4, p, sU[q * ER + l]), fma(p, Jk, -G0));
+        };
+        modal::unroll<0, NQ>([&](auto qc) {
+            constexpr int q = qc.value, m = modal::kT<P>.vmir[q];
+            if constexpr (m >= q) {
+                const Real g = flux(q), gm = m != q ? flux(m) : Real(0);
+                modal::moments<Real, P, NM>(q, g, gm, M);
+            }
+        });
+#pragma unroll
+        for (int m = 0; m < NM; ++m) sM[(w * NM + m) * ER + l] = M[m];
+    } else if (live) {
+        const Real* h = a.Hs + (e0 + e) * 20 * NQF + v * NQF;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            Real x[NQF], b[NF];
+            load_row<NQF>(h + f * 5 * NQF, x);
+            modal::face_moments<Real, P>(x, b);
+#pragma unroll
+            for (int m = 0; m < NF; ++m) sA[(f * NF + m) * ER + l] = b[m];
+        }
+    }
+    __syncthreads();
+    if (!live) return;
+    by_warp(w, [&](auto wc) {
+        constexpr auto& T = modal::kT<P>;
+        constexpr int J0 = NB * wc.value / WIDE, J1 = NB * (wc.value + 1) / WIDE;
+        Real r[J1 - J0];
+#pragma unroll
+        for (int j = J0; j < J1; ++j) r[j - J0] = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int m = 0; m < NM; ++m) {
+                const Real s = sM[(k * NM + m) * ER + l];
+#pragma unroll
+                for (int j = J0; j < J1; ++j) modal::axpy(r[j - J0], T.D[k][m][j], s);
+            }
+        // modal::lift of the moments, the faces' scales as its factors
+        const Real s0 = -sG[4 * e], s1 = -sG[4 * e + 1];
+#pragma unroll
+        for (int m = 0; m < NF; ++m) {
+            const Real x = s0 * sA[m * ER + l], b = sA[(NF + m) * ER + l], ev = fma(s1, b, x), od = fma(s1, b, -x);
+#pragma unroll
+            for (int j = J0; j < J1; ++j) modal::axpy(r[j - J0], T.E[1][m][j], T.odd[j] ? od : ev);
+        }
+#pragma unroll
+        for (int f = 2; f < 4; ++f) {
+            const Real s = -sG[4 * e + f];
+#pragma unroll
+            for (int m = 0; m < NF; ++m) {
+                const Real x = s * sA[(f * NF + m) * ER + l];
+#pragma unroll
+                for (int j = J0; j < J1; ++j) modal::axpy(r[j - J0], T.E[f][m][j], x);
+            }
+        }
+        const int64_t g = row * NB;
+#pragma unroll
+        for (int j = J0; j < J1; ++j) {
+            Real x = r[j - J0];
+            if (RK) {
+                x = a.b * (a.U[g + j] + a.dt * x);
+                if (a.a != Real(0)) x += a.a * a.U0[g + j];
+            }
+            a.out[g + j] = x;
+        }
+    });
+}
+
 template <typename Real, int P, bool RK>
 cudaError_t launch_element(const ResArgs<Real>& r, cudaStream_t s) {
+    if constexpr (sizeof(Real) == 8 && P == 3) {
+        if (r.ne <= WIDE_MAX_NE) {
+            k_element_wide<P, RK><<<(unsigned)((r.ne + 5) / 6), 32 * WIDE, 0, s>>>(r);
+            return cudaGetLastError();
+        }
+    }
     return small_tiles(r.ne) ? launch_tiles<Real, P, RK, 6>(r, s) : launch_tiles<Real, P, RK, 32>(r, s);
 }
 

@@ -135,6 +135,7 @@ struct Tables {
     bool fodd[NF]{};             // of the face modes under the swap of the face's first two vertices
     int vmir[NQ]{};              // mirror point of a volume point, of a face point
     int fmir[NQF]{};
+    int vpair[NQ]{};             // number of a volume point's mirror pair, counted by its lower point
 
     static constexpr double chop(double x) { return cabs(x) < 1e-13 ? 0.0 : x; }
 
@@ -195,6 +196,7 @@ struct Tables {
         for (int d = 0; d <= P; ++d)
             for (int i = 0; i <= d; ++i)
                 for (int j = 0; i + j <= d; ++j) odd[n++] = i % 2 == 1;
+        for (q = 0, n = 0; q < NQ; ++q) vpair[q] = vmir[q] < q ? vpair[vmir[q]] : n++;
         for (q = 0; q < NQ; ++q) basis(bary[q], phi[q], grad[q]);
         for (int k = 0; k < 3; ++k)
             for (int m = 0; m < NM; ++m)
@@ -254,13 +256,13 @@ __device__ __forceinline__ void axpy(Real& r, double c, Real x) {
 }
 
 // values at the volume points Q0 .. Q1 - 1 (a range closed under the mirror) of a field of the first N
-// modes, store(q, sum_j c[j] phi_j(x_q))
-template <typename Real, int P, int N, int Q0, int Q1, typename Store>
+// modes, store(q, sum_j c[j] phi_j(x_q)); of PARTS shares of the points, share PART
+template <typename Real, int P, int N, int Q0, int Q1, int PART = 0, int PARTS = 1, typename Store>
 __device__ __forceinline__ void interpolate(const Real* c, Store store) {
     unroll<Q0, Q1>([&](auto qc) {
         constexpr auto& T = kT<P>;
         constexpr int q = qc.value, m = T.vmir[q];
-        if constexpr (m >= q) {
+        if constexpr (m >= q && T.vpair[q] % PARTS == PART) {
             Real e = 0, o = 0;
 #pragma unroll
             for (int j = N - 1; j >= 0; --j) {
@@ -415,7 +417,7 @@ __device__ __forceinline__ void lift(Load load, Real* r) {
         face_moments<Real, P>(h, b);
 #pragma unroll
         for (int m = 0; m < T.NF; ++m) {
-            const Real x = s0 * a[m], e = s1 * b[m] + x, o = s1 * b[m] - x;
+            const Real x = s0 * a[m], e = fma(s1, b[m], x), o = fma(s1, b[m], -x);
 #pragma unroll
             for (int j = 0; j < T.NB; ++j) axpy(r[j], T.E[1][m][j], T.odd[j] ? o : e);
         }
