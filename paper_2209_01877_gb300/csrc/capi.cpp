@@ -223,11 +223,6 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
         cudaError_t e = dg::setup_face_once(m, rec, owner, m->d_jinv64, m->host.ne, s);
         if (e == cudaErrorMemoryAllocation && m->precision == DG_FP32) {
             (void)cudaGetLastError();
-            cudaFree(m->d_frec);
-            cudaFree(m->d_fnorm);
-            m->d_frec = nullptr;
-            m->d_fnorm = nullptr;
-            m->d_T = nullptr;
         } else if (e != cudaSuccess) {
             free_mesh(m);
             return cuda_fail(e, "face buffers");

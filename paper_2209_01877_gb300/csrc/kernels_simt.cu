@@ -825,7 +825,16 @@ cudaError_t setup_face_once(dg_mesh* m, const std::vector<FaceRec>& rec, const s
         if (e == cudaSuccess) e = es;
     }
     cudaFree(d_owner);
-    if (e == cudaSuccess) m->face_once = true;
+    if (e == cudaSuccess) {
+        m->face_once = true;
+        return e;
+    }
+    // nothing half made stays: an FP32 mesh goes on without
+    cudaFree(m->d_frec);
+    cudaFree(m->d_fnorm);
+    cudaFree(m->d_T);
+    m->d_frec = nullptr;
+    m->d_fnorm = m->d_T = nullptr;
     return e;
 }
 
