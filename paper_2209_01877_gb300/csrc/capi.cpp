@@ -59,9 +59,9 @@ void free_mesh(dg_mesh* m) {
     cudaFree(m->d_bface);
     cudaFree(m->d_fcode);
     cudaFree(m->d_perm);
-    cudaFree(m->d_jinv);
+    if (m->d_jinv != m->d_jinv64) cudaFree(m->d_jinv);   // FP64 meshes share them
     cudaFree(m->d_jinv64);
-    cudaFree(m->d_tab);
+    if (m->d_tab != m->d_tab64) cudaFree(m->d_tab);
     cudaFree(m->d_tab64);
     cudaFree(m->d_fperm);
     cudaFree(m->d_tab16);
@@ -229,7 +229,7 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
         }
     }
     if (m->precision == DG_FP64) {
-        m->d_tab = m->d_tab64;   // shared; freed once below
+        m->d_tab = m->d_tab64;   // shared
         m->d_jinv = m->d_jinv64;
     } else {
         float* t = nullptr;
@@ -259,8 +259,6 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
 dg_status dg_mesh_destroy(dg_mesh* m) {
     if (!m) return fail(DG_ERR_ARG, "mesh is NULL");
     cudaDeviceSynchronize();
-    if (m->d_tab == m->d_tab64) m->d_tab = nullptr;
-    if (m->d_jinv == m->d_jinv64) m->d_jinv = nullptr;
     free_mesh(m);
     return DG_OK;
 }

@@ -25,6 +25,6 @@ def _child(shim, check, precision, p):
     assert r.returncode == 0 and "CHILD OK" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
 
 
-@pytest.mark.parametrize("precision,p", [("fp32", 2), ("mixed", 2)])
+@pytest.mark.parametrize("precision,p", [("fp64", 1), ("fp32", 2), ("mixed", 2)])
 def test_refused_allocations_of_a_creation_leave_nothing(shim, precision, p):
     _child(shim, "creation", precision, p)
