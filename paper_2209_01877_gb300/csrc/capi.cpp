@@ -217,10 +217,7 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
     if (!is_mixed(m)) {
         // every face's traces and flux once; an FP32 mesh without room for the face buffer runs the
         // kernel that needs none
-        std::vector<dg::FaceRec> rec;
-        std::vector<int32_t> owner;
-        dg::build_face_list(m->host, m->host, 0, rec, owner);
-        cudaError_t e = dg::setup_face_once(m, rec, owner, m->d_jinv64, m->host.ne, s);
+        cudaError_t e = dg::setup_face_once(m, m, 0, m->host.ne, s);
         if (e == cudaErrorMemoryAllocation && m->precision == DG_FP32) {
             (void)cudaGetLastError();
         } else if (e != cudaSuccess) {

@@ -45,19 +45,15 @@ bool build_mesh(const int32_t* tet_vid, const double* tet_xyz, const int8_t* bc_
                 int renumber, MeshHost& out, int& code, std::string& err);
 
 // A face that a mesh evaluates, from one of its slots 4 e + f (on its owner's side, unless the owner
-// is a halo element of a partition).
+// is a halo element of a partition).  A boundary face belongs to its element; an interior face to the element
+// with the smaller caller index, so the choice, like every other input of the face flux, does not
+// depend on the internal element order.
 struct FaceRec {
     int32_t slot;
     int32_t other;      // the matching slot, or -1 - bc_type
     int32_t code;       // bits 0-2 the orientation (face-point permutation), bit 3 set if slot owns the face
-    int32_t pad;
+    int32_t owner;      // the owning slot in the numbers of the whole mesh
 };
-
-// The faces of the elements [first, first + local.ne) of `whole`, whose connectivity in local numbers
-// (own elements, then halo) is `local`; boundary faces last.  owner: each face's owning slot in
-// whole's numbers.
-void build_face_list(const MeshHost& whole, const MeshHost& local, int64_t first, std::vector<FaceRec>& rec,
-                     std::vector<int32_t>& owner);
 
 }  // namespace dg
 
@@ -130,10 +126,10 @@ namespace dg {
 // T: the face buffer to use (null: the FP32 kernel that needs none)
 cudaError_t launch_residual(dg_mesh* m, const void* U, const void* U0, void* out, int mode,
                             double dt, double a, double b, void* T, cudaStream_t s);
-// the face-once path's device data: the face list, the owners' normals from the whole mesh's J^-1,
-// the face buffer of n_trace elements
-cudaError_t setup_face_once(dg_mesh* m, const std::vector<FaceRec>& rec, const std::vector<int32_t>& owner,
-                            const double* d_jinv64_whole, int64_t n_trace, cudaStream_t s);
+// the face-once path's device data for m, whose elements are [first, first + ne) of whole (m itself, or a
+// partition's mesh in local numbers, own elements and then halo): the face list, boundary faces last,
+// the owners' normals, the face buffer of n_trace elements
+cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int64_t n_trace, cudaStream_t s);
 // face traces of a state of the mesh's precision, into the face buffer T; the adjoint's: of U into T,
 // and of lam times each face's |grad lambda_f| into TL
 cudaError_t launch_traces(dg_mesh* m, const void* U, void* T, cudaStream_t s);

@@ -318,32 +318,4 @@ bool build_mesh(const int32_t* tet_vid, const double* tet_xyz, const int8_t* bc_
     return true;
 }
 
-// The faces evaluated once.  A boundary face belongs to its element; an interior face to the element
-// with the smaller caller index, so the choice, like every other input of the face flux, does not
-// depend on the internal element order.
-void build_face_list(const MeshHost& whole, const MeshHost& local, int64_t first, std::vector<FaceRec>& rec,
-                     std::vector<int32_t>& owner) {
-    rec.clear();
-    owner.clear();
-    rec.reserve(2 * local.ne + 64);
-    owner.reserve(2 * local.ne + 64);
-    std::vector<FaceRec> bnd;
-    for (int64_t e = 0; e < local.ne; ++e)
-        for (int f = 0; f < 4; ++f) {
-            const int32_t sl = (int32_t)(4 * e + f), ws = (int32_t)(4 * first + sl), n = local.nbr[sl];
-            if (n < 0) {
-                bnd.push_back({sl, n, 8, 0});
-                continue;
-            }
-            const int32_t wn = whole.nbr[ws];
-            const bool own = whole.perm[wn] > whole.perm[first + e];
-            if (!own && n < local.ne) continue;   // listed on the owner's side
-            const int fn = local.fcode[sl] & 3;
-            rec.push_back({sl, 4 * n + fn, (local.fcode[sl] >> 2) | (own ? 8 : 0), 0});
-            owner.push_back(own ? ws : 4 * wn + fn);
-        }
-    for (const FaceRec& b : bnd) owner.push_back((int32_t)(4 * first + b.slot));
-    rec.insert(rec.end(), bnd.begin(), bnd.end());
-}
-
 }  // namespace dg

@@ -783,13 +783,99 @@ cudaError_t dispatch(dg_mesh* m, const void* U, const void* U0, void* out, int m
 }  // namespace
 
 namespace {
-// outward unit normals -grad lambda_f / |grad lambda_f| of the listed slots
+// ---- the face list, from the connectivity on the device (on the host, with a branch per slot that is taken every
+// other time, it took 19 of the 240 ms of a 384,000-element creation, and its upload more) ----------
+
+struct ListArgs {
+    const int32_t* nbr;     // of the listing mesh, local numbers
+    const uint8_t* fcode;
+    const int32_t* wnbr;    // the whole mesh's neighbours and caller indices
+    const int32_t* perm;
+    int64_t ne, first;      // own elements; the first one's number in the whole mesh
+};
+
+// whether slot's face is listed from it, among the boundary faces (BND) or the interior ones, and its record
+template <bool BND>
+__device__ __forceinline__ bool listed(const ListArgs& a, int64_t slot, FaceRec& r) {
+    if (slot >= 4 * a.ne) return false;
+    const int32_t n = a.nbr[slot], ws = (int32_t)(4 * a.first + slot);
+    if (BND) {
+        r = {(int32_t)slot, n, 8, ws};
+        return n < 0;
+    }
+    if (n < 0) return false;
+    const int c = a.fcode[slot], fn = c & 3;
+    const int32_t wn = a.wnbr[ws];
+    const bool own = a.perm[wn] > a.perm[ws >> 2];
+    r = {(int32_t)slot, 4 * n + fn, (c >> 2) | (own ? 8 : 0), own ? ws : 4 * wn + fn};
+    return own || n >= a.ne;   // else listed on the owner's side
+}
+
+constexpr int LT = 256;
+
+template <bool BND>
+__global__ void __launch_bounds__(LT) k_list_count(ListArgs a, int32_t* counts) {
+    FaceRec r;
+    const int n = __syncthreads_count(listed<BND>(a, blockIdx.x * (int64_t)LT + threadIdx.x, r));
+    if (threadIdx.x == 0) counts[blockIdx.x] = n;
+}
+
+// exclusive sums, in place: one block, a piece of 1,024 after the other
+__global__ void __launch_bounds__(1024) k_list_scan(int32_t* counts, int64_t n) {
+    __shared__ int32_t s[1024];
+    __shared__ int32_t carry;
+    const int t = threadIdx.x;
+    if (t == 0) carry = 0;
+    for (int64_t base = 0; base < n; base += 1024) {
+        const int32_t x = base + t < n ? counts[base + t] : 0;
+        s[t] = x;
+        __syncthreads();
+        for (int d = 1; d < 1024; d *= 2) {
+            const int32_t y = t >= d ? s[t - d] : 0;
+            __syncthreads();
+            s[t] += y;
+            __syncthreads();
+        }
+        const int32_t c = carry, total = s[1023];
+        if (base + t < n) counts[base + t] = c + s[t] - x;
+        __syncthreads();
+        if (t == 0) carry = c + total;
+        __syncthreads();
+    }
+}
+
+template <bool BND>
+__global__ void __launch_bounds__(LT) k_list_write(ListArgs a, const int32_t* counts, FaceRec* out, int64_t n) {
+    __shared__ int32_t warp_n[LT / 32];
+    const int t = threadIdx.x, w = t >> 5, l = t & 31;
+    FaceRec r;
+    const bool on = listed<BND>(a, blockIdx.x * (int64_t)LT + t, r);
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    if (l == 0) warp_n[w] = __popc(m);
+    __syncthreads();
+    int64_t at = counts[blockIdx.x] + __popc(m & ((1u << l) - 1u));
+    for (int k = 0; k < w; ++k) at += warp_n[k];
+    if (on && at < n) out[at] = r;
+}
+
+template <bool BND>
+cudaError_t list_faces(const ListArgs& a, int32_t* counts, FaceRec* out, int64_t n, cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    const unsigned nblk = (unsigned)((4 * a.ne + LT - 1) / LT);
+    k_list_count<BND><<<nblk, LT, 0, s>>>(a, counts);
+    k_list_scan<<<1, 1024, 0, s>>>(counts, nblk);
+    k_list_write<BND><<<nblk, LT, 0, s>>>(a, counts, out, n);
+    return cudaGetLastError();
+}
+
+// outward unit normals -grad lambda_f / |grad lambda_f| of the listed faces' owning slots
 template <typename Real>
-__global__ void k_face_normals(const double* __restrict__ jinv, const int32_t* __restrict__ slot, int64_t n, Real* out) {
+__global__ void k_face_normals(const double* __restrict__ jinv, const FaceRec* __restrict__ rec, int64_t n, Real* out) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double* I = jinv + (int64_t)(slot[i] >> 2) * 9;
-    const int f = slot[i] & 3;
+    const int32_t slot = rec[i].owner;
+    const double* I = jinv + (int64_t)(slot >> 2) * 9;
+    const int f = slot & 3;
     double g[3];
     for (int d = 0; d < 3; ++d) g[d] = f == 0 ? -(I[d] + I[3 + d] + I[6 + d]) : I[3 * (f - 1) + d];
     const double gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
@@ -797,34 +883,32 @@ __global__ void k_face_normals(const double* __restrict__ jinv, const int32_t* _
 }
 }  // namespace
 
-cudaError_t setup_face_once(dg_mesh* m, const std::vector<FaceRec>& rec, const std::vector<int32_t>& owner,
-                            const double* d_jinv64_whole, int64_t n_trace, cudaStream_t s) {
-    const int64_t n = (int64_t)rec.size();
-    m->n_flist = n;
-    m->n_interior = 0;
-    while (m->n_interior < n && rec[m->n_interior].other >= 0) ++m->n_interior;
-    m->n_trace = n_trace;
-    const size_t nn = std::max<size_t>(rec.size(), 1);
-    int32_t* d_owner = nullptr;
-    cudaError_t e = cudaMalloc(&m->d_frec, nn * sizeof(FaceRec));
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_fnorm, nn * 3 * (m->precision == DG_FP64 ? 8 : 4));
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_T, m->face_bytes());
-    if (e == cudaSuccess) e = cudaMalloc(&d_owner, nn * sizeof(int32_t));
-    if (e == cudaSuccess && n > 0) {
-        e = cudaMemcpyAsync(m->d_frec, rec.data(), rec.size() * sizeof(FaceRec), cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(d_owner, owner.data(), owner.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-        const unsigned grid = (unsigned)((n + 255) / 256);
-        if (e == cudaSuccess) {
-            if (m->precision == DG_FP64)
-                k_face_normals<double><<<grid, 256, 0, s>>>(d_jinv64_whole, d_owner, n, static_cast<double*>(m->d_fnorm));
-            else
-                k_face_normals<float><<<grid, 256, 0, s>>>(d_jinv64_whole, d_owner, n, static_cast<float*>(m->d_fnorm));
-            e = cudaGetLastError();
-        }
-        const cudaError_t es = cudaStreamSynchronize(s);   // the host vectors go out of scope
-        if (e == cudaSuccess) e = es;
+cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int64_t n_trace, cudaStream_t s) {
+    const int64_t slots = 4 * m->host.ne;
+    int32_t nbnd = 0, nhalo = 0;
+    for (int64_t i = 0; i < slots; ++i) {
+        nbnd += m->host.nbr[i] < 0;
+        nhalo += m->host.nbr[i] >= (int32_t)m->host.ne;
     }
-    cudaFree(d_owner);
+    m->n_interior = (slots - nbnd - nhalo) / 2 + nhalo;
+    const int64_t n = m->n_flist = m->n_interior + nbnd;
+    m->n_trace = n_trace;
+    cudaError_t e = cudaMalloc(&m->d_frec, n * sizeof(FaceRec));
+    if (e == cudaSuccess) e = cudaMalloc(&m->d_fnorm, n * 3 * (m->precision == DG_FP64 ? 8 : 4));
+    if (e == cudaSuccess) e = cudaMalloc(&m->d_T, m->face_bytes());
+    const ListArgs a{m->d_nbr, m->d_fcode, whole->d_nbr, whole->d_perm, m->host.ne, first};
+    // the normals' place, written last, holds the counts: at least 24 bytes an element (n >= 2 ne) against 4 per LT slots
+    int32_t* counts = static_cast<int32_t*>(m->d_fnorm);
+    if (e == cudaSuccess) e = list_faces<false>(a, counts, m->d_frec, m->n_interior, s);
+    if (e == cudaSuccess) e = list_faces<true>(a, counts, m->d_frec + m->n_interior, nbnd, s);
+    if (e == cudaSuccess) {
+        const unsigned grid = (unsigned)((n + 255) / 256);
+        if (m->precision == DG_FP64)
+            k_face_normals<double><<<grid, 256, 0, s>>>(whole->d_jinv64, m->d_frec, n, static_cast<double*>(m->d_fnorm));
+        else
+            k_face_normals<float><<<grid, 256, 0, s>>>(whole->d_jinv64, m->d_frec, n, static_cast<float*>(m->d_fnorm));
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) {
         m->face_once = true;
         return e;

@@ -259,10 +259,7 @@ dg_status dg_partition_create(dg_mesh* m, int k, void* stream, dg_partition** ou
         // are evaluated here too, in their owner's orientation, so every own element receives the
         // flux the whole mesh would give it
         if (m->precision == DG_FP64) {
-            std::vector<dg::FaceRec> rec;
-            std::vector<int32_t> owner;
-            dg::build_face_list(m->host, sm->host, pl.first, rec, owner);
-            PTRY(dg::setup_face_once(sm, rec, owner, m->d_jinv64, pl.count + (int64_t)pl.halo.size(), s));
+            PTRY(dg::setup_face_once(sm, m, pl.first, pl.count + (int64_t)pl.halo.size(), s));
         }
         // local state: own then halo blocks (mixed: hi plane of own + halo, then the lo plane)
         const size_t nloc = (size_t)(pl.count + pl.halo.size()) * nv_of(m);
