@@ -178,7 +178,11 @@ dg_status dg_ns_residual(dg_mesh* mesh, const double* U, double* R, double mu, d
  * the viscous lines) and applies the stage update of dg_rk_stage in the mesh's
  * state format (the mixed forms: the FP32 increment added to the float-float
  * state without rounding error).  mu and prandtl as for dg_ns_residual; mu = 0
- * gives the Euler stages (as separate kernels instead of one fused stage).
+ * gives the Euler stages (as separate kernels instead of one fused stage, so
+ * to rounding).  FP32 meshes have two orders of summation for the Euler lines,
+ * chosen by size and, in dg_rk_stage and dg_rk3_step, by whether there are
+ * boundary faces; dg_residual and dg_ns_residual always use the first.  Each
+ * gives the residual to FP32 rounding of its terms.
  * DG_ERR_UNSUPPORTED on a mesh in the conservative mode (dg_set_conservative
  * applies to the Euler stages).  Uses the residual work buffer, so a
  * dg_residual call between steps is safe. */
@@ -256,7 +260,7 @@ dg_status dg_boundary_flux(dg_mesh* mesh, const double* U, int stage, double out
 dg_status dg_residual_vjp(dg_mesh* mesh, const double* U, const double* lambda, double* out, void* stream);
 
 /* out = (d U_{n+1} / d U_n)^T lambda for one SSP-RK3 step of size dt from
- * U0 (stages recomputed): m2 = 2/3 (lambda + dt J(U2)^T lambda),
+ * U0 (stages recomputed, in FP32 equal to dg_rk_stage's to rounding): m2 = 2/3 (lambda + dt J(U2)^T lambda),
  * m1 = 1/4 (m2 + dt J(U1)^T m2), out = lambda/3 + 3/4 m2 + m1 + dt J(U0)^T m1.
  * Device FP64 caller order. */
 dg_status dg_rk3_step_vjp(dg_mesh* mesh, const double* U0, double dt, const double* lambda, double* out,

@@ -396,11 +396,12 @@ int64_t fp32_faces_min_ne(const dg_mesh* m) {
 }
 // The face buffer of an FP32 RK stage, or null for the single kernel.  On a mesh with boundary faces the
 // single kernel is kept: dg_boundary_flux reports the boundary integral of the FP32 state in FP64, which
-// shows the order of summation at 1e-7.
+// shows the order of summation at 1e-7, the rounding of the state itself.
 void* stage_faces(const dg_mesh* m, void* T) {
     return m->precision == DG_FP64 || (m->host.ne >= fp32_faces_min_ne(m) && !m->has_bc) ? T : nullptr;
 }
-// the same where no boundary integral is taken of the states: Navier-Stokes steps and the adjoint's stages
+// The same for Navier-Stokes steps and for the stages that the adjoint recomputes, with boundary faces too:
+// their values differ from those of dg_rk3_step on such a mesh by FP32 rounding, as include/dg.h says.
 void* inner_faces(const dg_mesh* m, void* T) {
     return m->precision == DG_FP64 || m->host.ne >= fp32_faces_min_ne(m) ? T : nullptr;
 }

@@ -113,6 +113,50 @@ def test_fp32_ns_step_walled_odd(p, ne):
     assert np.abs(out["fp32"] - out["fp64"]).max() < bar
 
 
+@pytest.mark.parametrize("p", [1, 2, 3])
+def test_fp32_inviscid_ns_step_is_the_euler_step(p):
+    """With walls dg_rk3_step and dg_ns_rk3_step with mu = 0 sum the Euler lines in two orders: each within
+    the FP32 bar of the residual, so twice that of a step apart."""
+    arrays = _walled(9731)
+    scale_of = Problem(*arrays, p=1, flux="roe")
+    M = _mesh(arrays, p, "roe", "fp32")
+    U = _state(M)
+    dg.dg_set_state(M.handle, U)
+    dt = dg.dg_stable_dt(M.handle, 0.3)
+    out = []
+    for step in (lambda: dg.dg_rk3_step(M.handle, dt, 1), lambda: dg.dg_ns_rk3_step(M.handle, dt, 1, 0.0)):
+        dg.dg_set_state(M.handle, U)
+        step()
+        out.append(np.empty_like(U))
+        dg.dg_get_state(M.handle, out[-1])
+    bar = 2 * 3 * (dt * 1e-4 * max(residual_term_scale(scale_of, U)) + 2.0 ** -23 * np.abs(U).max())
+    assert np.abs(out[0] - U).max() > 20 * bar
+    assert np.abs(out[0] - out[1]).max() < bar
+    M.close()
+
+
+@pytest.mark.parametrize("p", [2, 3])
+def test_fp32_adjoint_of_a_walled_step(p):
+    """The stages that the adjoint recomputes on a mesh with boundary faces against those of the step it
+    differentiates: FP32 rounding of the states (1e-7 of them) through second derivatives of order one,
+    within the FP32 bar of the VJP.  Reference: the FP64 mesh, whose stages have one form."""
+    torch = torch_cuda()
+    arrays = _walled(9731)
+    V = {}
+    for precision in ("fp64", "fp32"):
+        M = _mesh(arrays, p, "roe", precision)
+        if precision == "fp64":
+            U = _state(M)
+            dg.dg_set_state(M.handle, U)
+            dt = dg.dg_stable_dt(M.handle, 0.1)
+            Ud, lam = torch.from_numpy(U).cuda(), torch.from_numpy(I.random_directions(U.shape, 1)[0]).cuda()
+        out = torch.full_like(Ud, float("nan"))
+        dg.dg_rk3_step_vjp(M.handle, Ud, dt, lam, out)
+        V[precision] = out.cpu().numpy()
+        M.close()
+    assert max_rel_err(V["fp32"], V["fp64"]) < 1e-4
+
+
 @pytest.mark.parametrize("p,flux", [(1, "roe"), (2, "rusanov"), (3, "roe")])
 def test_residual_and_vjp_ragged(p, flux):
     """FP64 against the oracle, FP32 against FP64, at 9,731 elements with walls."""
