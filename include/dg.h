@@ -169,8 +169,8 @@ dg_status dg_residual(dg_mesh* mesh, const double* U, double* R, void* stream);
  * their Euler lines from the tensor-core kernel and the viscous lines in FP32
  * from the state's leading FP32 plane.  The first call with mu > 0 allocates
  * the gradient buffer (15 Nb values per element), a face-flux buffer
- * (16 Nqf values per element) and, on FP32 meshes, a trace buffer (20 Nqf
- * values per element), in that arithmetic, owned by the mesh. */
+ * (16 Nqf values per element), in that arithmetic, and on FP32 meshes with
+ * room to spare a trace buffer (20 Nqf values per element); the mesh owns them. */
 dg_status dg_ns_residual(dg_mesh* mesh, const double* U, double* R, double mu, double prandtl, void* stream);
 
 /* nsteps SSP-RK3 steps of the Navier-Stokes equations on the internal state, in
@@ -180,7 +180,7 @@ dg_status dg_ns_residual(dg_mesh* mesh, const double* U, double* R, double mu, d
  * state without rounding error).  mu and prandtl as for dg_ns_residual; mu = 0
  * gives the Euler stages (as separate kernels instead of one fused stage, so
  * to rounding).  FP32 meshes have two orders of summation for the Euler lines,
- * chosen by size and, in dg_rk_stage and dg_rk3_step, by whether there are
+ * chosen by size and, in the steps without viscosity, by whether there are
  * boundary faces; dg_residual and dg_ns_residual always use the first.  Each
  * gives the residual to FP32 rounding of its terms.
  * DG_ERR_UNSUPPORTED on a mesh in the conservative mode (dg_set_conservative
@@ -255,8 +255,9 @@ dg_status dg_boundary_flux(dg_mesh* mesh, const double* U, int stage, double out
  * interpolation, on both sides of every face; at a kink of |.| or max the
  * derivative of the branch taken, ties to the interior side).  U, lambda,
  * out: device FP64 [ne][5][Nb] in caller order.  The first call allocates the
- * adjoint's work buffers (six of the state's size and two of 20 Nqf values per
- * element), owned by the mesh. */
+ * adjoint's work buffers, owned by the mesh: six of the state's size and, in FP32
+ * on larger meshes with room to spare and in FP64, two of 20 Nqf values per
+ * element. */
 dg_status dg_residual_vjp(dg_mesh* mesh, const double* U, const double* lambda, double* out, void* stream);
 
 /* out = (d U_{n+1} / d U_n)^T lambda for one SSP-RK3 step of size dt from

@@ -101,17 +101,76 @@ dg_status ensure_work_buffers(dg_mesh* m) {
     return DG_OK;
 }
 
-// a buffer of the face-once form, allocated on first use; left null on an FP32 mesh without room for
-// it, which then runs the kernels that need none
-dg_status ensure_face_buffer(dg_mesh* m, void*& buf, size_t bytes) {
-    if (!m->face_once || buf) return DG_OK;
-    const cudaError_t e = cudaMalloc(&buf, bytes);
-    if (e == cudaSuccess) return DG_OK;
-    buf = nullptr;
-    if (m->precision == DG_FP64 || e != cudaErrorMemoryAllocation) return cuda_fail(e, "cudaMalloc(face buffer)");
-    (void)cudaGetLastError();
-    return DG_OK;
+constexpr size_t ALLOC_GRAIN = 2 << 20;   // what an allocation may take from the device at least
+size_t grains(size_t bytes) { return (bytes + ALLOC_GRAIN - 1) / ALLOC_GRAIN * ALLOC_GRAIN; }
+
+// What the calls on a mesh may still allocate on their first use, for its FP64 and FP32 forms.
+size_t pending_bytes(const dg_mesh* m) {
+    const size_t ne = m->host.ne, rs = real_size(m->precision);
+    size_t n = 0;
+    auto want = [&](const void* p, size_t bytes) { n += p ? 0 : grains(bytes); };
+    for (const void* b : m->d_W) want(b, m->state_bytes() + 256);
+    for (const void* b : m->d_V) want(b, m->state_bytes() + 256);
+    want(m->d_io, ne * 5 * m->nb * sizeof(double));
+    want(m->d_Z, ne * 15 * m->nb * rs);
+    want(m->d_HB, dg::ns_face_buffer_values(m->p, ne) * rs);
+    return n;
 }
+
+// Whether `bytes` more leave room for those: a buffer that a mesh can do without must not be the reason for
+// which a later call on it runs out of memory.
+bool room_for(const dg_mesh* m, size_t bytes) {
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return free_bytes >= grains(bytes) + pending_bytes(m);
+}
+
+// a buffer that the mesh can do without: left null where there is no such room
+void optional_buffer(const dg_mesh* m, void** buf, size_t bytes) {
+    if (!room_for(m, bytes)) return;
+    if (cudaMalloc(buf, bytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        *buf = nullptr;
+    }
+}
+
+// ---- which meshes evaluate every face once: FP64 all; FP32 by size -----------------------------------
+
+// From how many elements on an FP32 stage of three launches is faster than the single kernel.  us per step, single
+// against three launches:
+//   P1, where the tiles of the single kernel make one wave up to 19,456 elements: Rusanov 16,464 38 : 50, 24,576
+//       50 : 50, 34,992 57 : 67, 48,000 75 : 78, 55,566 81 : 81, 82,944 112 : 107 (so from three waves on);
+//       Roe 16,464 38 : 50, 20,250 52 : 50, 34,992 62 : 65, 48,000 81 : 76 (from one wave on);
+//   P2: 8,712 58 : 55 (Rusanov), 62 : 55 (Roe), 12,168 77 : 57, 93,750 420 : 181;
+//   P3: 8,712 137 : 69, 93,750 1,150 : 353.
+int64_t fp32_faces_min_ne(const dg_mesh* m) {
+    if (m->p > 1) return 8192;
+    return m->flux == DG_ROE ? 19456 : 3 * 19456;
+}
+
+// Whether the FP32 stages of the Euler steps do.  On a mesh with boundary faces the single kernel is kept:
+// dg_boundary_flux reports the boundary integral of the FP32 state in FP64, which shows the order of
+// summation at 1e-7, the rounding of the state itself.
+bool fp32_stage_faces(const dg_mesh* m) { return m->host.ne >= fp32_faces_min_ne(m) && !m->has_bc; }
+
+// Whether the adjoint evaluates every face once (three launches, a fourth for boundary faces).  In FP32
+// the single kernel k_residual_vjp, whose tiles hold 16, 8, 4 elements, is faster while they are no
+// more than the SMs.  us per VJP, single against three launches, Rusanov | Roe | Rusanov with boundary
+// faces: P1 2,058 elements 23 : 25 | 23 : 25 | 23 : 32, 3,072 27 : 25 | 32 : 25 | 31 : 32; P2 750
+// 23 : 27 | 25 : 27 | 25 : 34, 1,296 30 : 27 | 34 : 28 | 34 : 34; P3 384 28 : 32 | 30 : 32 | 30 : 38,
+// 750 34 : 32 | 38 : 32 | 38 : 38.  With Rusanov and boundary faces the single kernel is ahead up to two
+// tiles per SM (P1 4,374 32 : 34, P2 2,058 34 : 35).
+bool vjp_by_faces(const dg_mesh* m) {
+    if (m->precision == DG_FP64) return true;
+    const int64_t wave = 152 * (m->p == 1 ? 16 : m->p == 2 ? 8 : 4);
+    return m->host.ne > (m->flux == DG_RUSANOV && m->has_bc ? 2 : 1) * wave;
+}
+
+// whether any call on an FP32 mesh uses the face list
+bool faces_in_use(const dg_mesh* m) { return vjp_by_faces(m) || m->host.ne >= fp32_faces_min_ne(m); }
 
 }  // namespace
 
@@ -214,16 +273,10 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
         DG_TRY(upload(&m->d_mhdr, cnt.data(), cnt.size(), s));
         DG_TRY(upload(&m->d_mxnbr, xnbr.data(), xnbr.size(), s));
     }
-    if (!is_mixed(m)) {
-        // every face's traces and flux once; an FP32 mesh without room for the face buffer runs the
-        // kernel that needs none
-        cudaError_t e = dg::setup_face_once(m, m, 0, m->host.ne, s);
-        if (e == cudaErrorMemoryAllocation && m->precision == DG_FP32) {
-            (void)cudaGetLastError();
-        } else if (e != cudaSuccess) {
-            free_mesh(m);
-            return cuda_fail(e, "face buffers");
-        }
+    if (m->precision == DG_FP64) {
+        cudaError_t e = dg::setup_face_once(m, m, 0, ne, s);
+        if (e == cudaSuccess) e = cudaMalloc(&m->d_T, m->face_bytes());
+        if (e != cudaSuccess) { free_mesh(m); return cuda_fail(e, "face buffers"); }
     }
     if (m->precision == DG_FP64) {
         m->d_tab = m->d_tab64;   // shared
@@ -245,6 +298,15 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
         if (e == cudaSuccess) e = cudaMalloc(&m->d_status, sizeof(unsigned int));
         if (e == cudaSuccess) e = cudaMemsetAsync(m->d_status, 0, sizeof(unsigned int), s);
         if (e == cudaSuccess) e = cudaMallocHost(&m->h_red, 16 * sizeof(double));
+        // FP32: the face list and, where the Euler stages use it, the face buffer; last, and only with room
+        // to spare: without them the mesh runs the kernels that need none
+        if (e == cudaSuccess && m->precision == DG_FP32 && faces_in_use(m) &&
+            room_for(m, m->host.n_faces * (sizeof(dg::FaceRec) + 3 * sizeof(float)))) {
+            e = dg::setup_face_once(m, m, 0, ne, s);
+            if (e == cudaErrorMemoryAllocation) e = (cudaGetLastError(), cudaSuccess);
+        }
+        if (e == cudaSuccess && m->face_once && m->precision == DG_FP32 && fp32_stage_faces(m))
+            optional_buffer(m, &m->d_T, m->face_bytes());
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) { free_mesh(m); return cuda_fail(e, "mesh buffers"); }
     }
@@ -383,27 +445,12 @@ namespace {
 // and the faster form is used.
 void* residual_faces(const dg_mesh* m) { return m->precision == DG_FP64 ? m->d_T : nullptr; }
 
-// From how many elements on an FP32 stage of three launches is faster than the single kernel.  us per step, single
-// against three launches:
-//   P1, where the tiles of the single kernel make one wave up to 19,456 elements: Rusanov 16,464 38 : 50, 24,576
-//       50 : 50, 34,992 57 : 67, 48,000 75 : 78, 55,566 81 : 81, 82,944 112 : 107 (so from three waves on);
-//       Roe 16,464 38 : 50, 20,250 52 : 50, 34,992 62 : 65, 48,000 81 : 76 (from one wave on);
-//   P2: 8,712 58 : 55 (Rusanov), 62 : 55 (Roe), 12,168 77 : 57, 93,750 420 : 181;
-//   P3: 8,712 137 : 69, 93,750 1,150 : 353.
-int64_t fp32_faces_min_ne(const dg_mesh* m) {
-    if (m->p > 1) return 8192;
-    return m->flux == DG_ROE ? 19456 : 3 * 19456;
-}
-// The face buffer of an FP32 RK stage, or null for the single kernel.  On a mesh with boundary faces the
-// single kernel is kept: dg_boundary_flux reports the boundary integral of the FP32 state in FP64, which
-// shows the order of summation at 1e-7, the rounding of the state itself.
-void* stage_faces(const dg_mesh* m, void* T) {
-    return m->precision == DG_FP64 || (m->host.ne >= fp32_faces_min_ne(m) && !m->has_bc) ? T : nullptr;
-}
+// The face buffer of an RK stage, or null for the single kernel.
+void* stage_faces(const dg_mesh* m, void* T) { return m->precision == DG_FP64 || fp32_stage_faces(m) ? T : nullptr; }
 // The same for Navier-Stokes steps and for the stages that the adjoint recomputes, with boundary faces too:
 // their values differ from those of dg_rk3_step on such a mesh by FP32 rounding, as include/dg.h says.
 void* inner_faces(const dg_mesh* m, void* T) {
-    return m->precision == DG_FP64 || m->host.ne >= fp32_faces_min_ne(m) ? T : nullptr;
+    return m->precision == DG_FP64 || (m->face_once && m->host.ne >= fp32_faces_min_ne(m)) ? T : nullptr;
 }
 
 // a caller's state as a residual's operand, in d_W[0]: the mixed forms' residual reads the hi plane
@@ -458,8 +505,10 @@ dg_status ensure_ns_buffers(dg_mesh* m) {
     const size_t rs = m->precision == DG_FP64 ? sizeof(double) : sizeof(float);
     if (!m->d_Z) DG_CUDA(cudaMalloc(&m->d_Z, (size_t)m->host.ne * 15 * m->nb * rs));
     if (!m->d_HB) DG_CUDA(cudaMalloc(&m->d_HB, dg::ns_face_buffer_values(m->p, m->host.ne) * rs));
-    if (m->precision == DG_FP64) m->d_TN = m->d_T;   // the Euler residual is done with it
-    if (ns_by_rows(m) && m->precision == DG_FP32 && !m->d_TN) DG_CUDA(cudaMalloc(&m->d_TN, (size_t)m->host.ne * 20 * m->nqf * rs));
+    if (m->precision == DG_FP64) m->d_TN = m->d_T;
+    if (m->precision == DG_FP32 && ns_by_rows(m) && !m->ns_set)
+        optional_buffer(m, &m->d_TN, (size_t)m->host.ne * 20 * m->nqf * rs);
+    m->ns_set = true;   // refused once, not asked for again on every call
     return DG_OK;
 }
 }  // namespace
@@ -654,9 +703,10 @@ dg_status dg_ns_rk3_step(dg_mesh* m, double dt, int nsteps, double mu, double pr
     // the stages of dg_rk_stage, each as residual (Euler + viscous lines) then update
     const struct { int in, base, out; double a, b; } stages[3] = {{0, -1, 1, 0.0, 1.0}, {1, 0, 2, 0.75, 0.25},
                                                                   {2, 0, 0, 1.0 / 3.0, 2.0 / 3.0}};
+    void* T = inner_faces(m, mu > 0.0 ? m->d_TN : m->d_T);   // the viscous passes' buffer: the Euler pass is done with it
     for (int k = 0; k < nsteps; ++k)
         for (const auto& g : stages) {
-            DG_CUDA(euler_residual_internal(m, B[g.in], R, inner_faces(m, m->d_T), s));
+            DG_CUDA(euler_residual_internal(m, B[g.in], R, T, s));
             if (mu > 0.0) DG_CUDA(dg::launch_ns_viscous(m, B[g.in], m->d_TN, m->d_Z, m->d_HB, R, mu, prandtl, s));
             DG_CUDA(dg::launch_rk_axpy(m, B[g.in], g.base >= 0 ? B[g.base] : nullptr, R, B[g.out], dt, g.a, g.b, s));
         }
@@ -737,27 +787,26 @@ dg_status dg_applied_boundary_flux(dg_mesh* m, double out[5], void* stream) {
 }
 
 namespace {
-// Whether the adjoint evaluates every face once (three launches, a fourth for boundary faces).  In FP32
-// the single kernel k_residual_vjp, whose tiles hold 16, 8, 4 elements, is faster while they are no
-// more than the SMs.  us per VJP, single against three launches, Rusanov | Roe | Rusanov with boundary
-// faces: P1 2,058 elements 23 : 25 | 23 : 25 | 23 : 32, 3,072 27 : 25 | 32 : 25 | 31 : 32; P2 750
-// 23 : 27 | 25 : 27 | 25 : 34, 1,296 30 : 27 | 34 : 28 | 34 : 34; P3 384 28 : 32 | 30 : 32 | 30 : 38,
-// 750 34 : 32 | 38 : 32 | 38 : 38.  With Rusanov and boundary faces the single kernel is ahead up to two
-// tiles per SM (P1 4,374 32 : 34, P2 2,058 34 : 35).
-bool vjp_by_faces(const dg_mesh* m) {
-    if (m->precision == DG_FP64) return true;
-    const int64_t wave = 152 * (m->p == 1 ? 16 : m->p == 2 ? 8 : 4);
-    return m->host.ne > (m->flux == DG_RUSANOV && m->has_bc ? 2 : 1) * wave;
-}
-
 dg_status ensure_adjoint_buffers(dg_mesh* m) {
     for (auto& b : m->d_V)
         if (!b) DG_CUDA(cudaMalloc(&b, m->state_bytes() + 256));
-    if (!vjp_by_faces(m)) return DG_OK;
-    // buffers apart from the RK steps', so that an adjoint call leaves a step on another stream alone
-    dg_status st = ensure_face_buffer(m, m->d_TA, m->face_bytes());
-    if (st == DG_OK) st = ensure_face_buffer(m, m->d_TL, m->face_bytes());
-    return st;
+    // face buffers apart from the RK steps', so that an adjoint call leaves a step on another stream alone
+    if (m->precision == DG_FP64) {
+        if (!m->d_TA) DG_CUDA(cudaMalloc(&m->d_TA, m->face_bytes()));
+        if (!m->d_TL) DG_CUDA(cudaMalloc(&m->d_TL, m->face_bytes()));
+        return DG_OK;
+    }
+    // FP32: both, or the single kernel
+    if (m->face_once && vjp_by_faces(m) && !m->adj_set && room_for(m, 2 * m->face_bytes())) {
+        optional_buffer(m, &m->d_TA, m->face_bytes());
+        if (m->d_TA) optional_buffer(m, &m->d_TL, m->face_bytes());
+        if (!m->d_TL) {
+            cudaFree(m->d_TA);
+            m->d_TA = nullptr;
+        }
+    }
+    m->adj_set = true;   // refused once, not asked for again on every call
+    return DG_OK;
 }
 }  // namespace
 

@@ -105,14 +105,15 @@ struct dg_mesh {
     // one evaluation per face (FP64, FP32): the faces this mesh evaluates (boundary faces last) with
     // their owners' outward normals, the number of elements with traces (own + halo on a
     // partition's mesh), and the face buffers [n_trace][4][5][Nqf] (traces, then the fluxes in their
-    // place): d_T of the RK steps (FP64: of every residual); lazy, the adjoint's own: d_TA, d_TL the
-    // direction's traces
+    // place): d_T of the RK steps (FP64: of every residual; FP32: where the stages use it and there is
+    // room); lazy, the adjoint's own: d_TA, d_TL the direction's traces
     bool face_once = false;
     dg::FaceRec* d_frec = nullptr;
     void* d_fnorm = nullptr;       // Real [n_flist][3]
     int64_t n_flist = 0, n_interior = 0, n_trace = 0;   // listed faces, interior ones among them
     void* d_T = nullptr;
     void *d_TA = nullptr, *d_TL = nullptr;
+    bool ns_set = false, adj_set = false;   // the optional buffers of these calls have been asked for
     size_t face_bytes() const;
     // small meshes: a CUDA graph of several captured RK3 steps at one dt (dg_rk3_step)
     cudaStream_t cap_stream = nullptr;
@@ -127,8 +128,8 @@ namespace dg {
 cudaError_t launch_residual(dg_mesh* m, const void* U, const void* U0, void* out, int mode,
                             double dt, double a, double b, void* T, cudaStream_t s);
 // the face-once path's device data for m, whose elements are [first, first + ne) of whole (m itself, or a
-// partition's mesh in local numbers, own elements and then halo): the face list, boundary faces last,
-// the owners' normals, the face buffer of n_trace elements
+// partition's mesh in local numbers, own elements and then halo): the face list, boundary faces last, and
+// the owners' normals; n_trace is the number of elements with traces
 cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int64_t n_trace, cudaStream_t s);
 // face traces of a state of the mesh's precision, into the face buffer T; the adjoint's: of U into T,
 // and of lam times each face's |grad lambda_f| into TL

@@ -895,7 +895,6 @@ cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int
     m->n_trace = n_trace;
     cudaError_t e = cudaMalloc(&m->d_frec, n * sizeof(FaceRec));
     if (e == cudaSuccess) e = cudaMalloc(&m->d_fnorm, n * 3 * (m->precision == DG_FP64 ? 8 : 4));
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_T, m->face_bytes());
     const ListArgs a{m->d_nbr, m->d_fcode, whole->d_nbr, whole->d_perm, m->host.ne, first};
     // the normals' place, written last, holds the counts: at least 24 bytes an element (n >= 2 ne) against 4 per LT slots
     int32_t* counts = static_cast<int32_t*>(m->d_fnorm);
@@ -916,9 +915,8 @@ cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int
     // nothing half made stays: an FP32 mesh goes on without
     cudaFree(m->d_frec);
     cudaFree(m->d_fnorm);
-    cudaFree(m->d_T);
     m->d_frec = nullptr;
-    m->d_fnorm = m->d_T = nullptr;
+    m->d_fnorm = nullptr;
     return e;
 }
 

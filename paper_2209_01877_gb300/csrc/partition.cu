@@ -260,6 +260,7 @@ dg_status dg_partition_create(dg_mesh* m, int k, void* stream, dg_partition** ou
         // flux the whole mesh would give it
         if (m->precision == DG_FP64) {
             PTRY(dg::setup_face_once(sm, m, pl.first, pl.count + (int64_t)pl.halo.size(), s));
+            PTRY(cudaMalloc(&sm->d_T, sm->face_bytes()));
         }
         // local state: own then halo blocks (mixed: hi plane of own + halo, then the lo plane)
         const size_t nloc = (size_t)(pl.count + pl.halo.size()) * nv_of(m);

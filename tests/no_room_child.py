@@ -71,5 +71,124 @@ def creation():
     print("allocations", n, "made without", made)
 
 
-{"creation": creation}[CHECK]()
+def rel(a, b):
+    return float(np.abs(a - b).max() / max(np.abs(b).max(), 1e-300))
+
+
+def calls(M, Ud, ld, out, dt):
+    """Every call of a mesh that may allocate, each with a result to compare (out: device scratch of the caller,
+    so that nothing but the mesh allocates)."""
+    host = np.empty(tuple(Ud.shape))
+
+    def device(f):
+        def run():
+            out.fill_(float("nan"))
+            f()
+            return out.cpu().numpy().copy()
+        return run
+
+    def stepped(f):
+        def run():
+            dg.dg_set_state(M.handle, Uh)      # through the staging buffer of host copies
+            f()
+            dg.dg_get_state(M.handle, host)
+            return host.copy()
+        return run
+    Uh = Ud.cpu().numpy()
+    return {
+        "step": stepped(lambda: dg.dg_rk3_step(M.handle, dt, 1)),
+        "residual": device(lambda: dg.dg_residual(M.handle, Ud, out)),
+        "ns_step": stepped(lambda: dg.dg_ns_rk3_step(M.handle, dt, 1, 0.05)),
+        "ns_residual": device(lambda: dg.dg_ns_residual(M.handle, Ud, out, 0.05)),
+        "vjp": device(lambda: dg.dg_residual_vjp(M.handle, Ud, ld, out)),
+        "step_vjp": device(lambda: dg.dg_rk3_step_vjp(M.handle, Ud, dt, ld, out)),
+    }
+
+
+def room():
+    """Memory for exactly the buffers that the calls cannot do without, then for a little more at a time: every
+    call runs, in any order, and gives what it gives on a mesh with room."""
+    m = I.make_box_mesh((12, 11, 11), jitter=0.1)
+    M = mesh(m)
+    U = torch.from_numpy(state(M)).cuda()
+    lam = torch.from_numpy(I.random_directions(U.shape, 1)[0]).cuda()
+    dt = 1e-3
+    out = torch.empty_like(U)
+    ref = {k: f() for k, f in calls(M, U, lam, out, dt).items()}
+    nb, nqf, ne, rs = M.nb, M.nqf, M.ne, 8 if PRECISION == "fp64" else 4
+    M.close()
+    for k in ref:
+        assert np.isfinite(ref[k]).all(), k
+    base = shim.fake_in_use()
+    face = 20 * nqf * ne * rs
+    need = ne * (16 + 4 + 4 + 72) + (1 << 20)                                     # connectivity, geometry; tables
+    need += ne * 36 if PRECISION == "fp32" else ne * (12 + 96) + 2 * face         # FP32 geometry; FP64 faces
+    need += 11 * (5 * nb * ne * rs + 256) + 5 * nb * ne * 8                       # state, work, adjoint; host copies
+    need += 15 * nb * ne * rs + 16 * nqf * ne * rs                                # viscous passes
+    # the size of one Euler term, |F| |grad lambda|, and of one viscous term, kappa |U| |grad lambda|^2
+    E = np.linalg.inv((m.tet_xyz[:, 1:] - m.tet_xyz[:, :1]).transpose(0, 2, 1))
+    inv_h = max(np.linalg.norm(E, axis=2).max(), np.linalg.norm(E.sum(1), axis=1).max())
+    mean = np.sqrt(6.0) * np.abs(U.cpu().numpy()[:, :, 0])
+    speed = (mean[:, 1:4] / mean[:, :1]).max()
+    euler_size = inv_h * (mean[:, 4].max() * 1.4 * speed + 0.4 * mean[:, 4].max())
+    viscous_size = 0.05 * 1.4 / (0.4 * 0.72) * mean.max() * inv_h ** 2
+    names = list(ref)
+    for extra in (0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 8.0):
+        for order in (names, names[::-1]):
+            shim.fake_limit(base + need + int(extra * face))
+            M = mesh(m)
+            got = calls(M, U, lam, out, dt)
+            for k in order + order:
+                r = got[k]()
+                if PRECISION == "fp64":
+                    assert np.array_equal(r, ref[k]), (extra, k)
+                elif k in ("step", "ns_step"):
+                    # two FP32 evaluations, each within 1e-4 of the size of the residual's terms, over three stages
+                    size = euler_size + (viscous_size if k == "ns_step" else 0.0)
+                    bar = 2 * 3 * (dt * 1e-4 * size + 2.0 ** -23 * np.abs(ref[k]).max())
+                    assert np.abs(r - ref[k]).max() < bar, (extra, k, np.abs(r - ref[k]).max(), bar)
+                else:
+                    assert rel(r, ref[k]) < 1e-4, (extra, k, rel(r, ref[k]))
+            M.close()
+            shim.fake_limit(2 ** 64 - 1)
+            assert shim.fake_in_use() == base and shim.fake_bad_frees() == 0
+
+
+def streams():
+    """An adjoint call on one stream leaves steps on another alone, with room for buffers of its own and
+    without."""
+    m = I.make_box_mesh((12, 11, 11), jitter=0.1)
+    M = mesh(m)
+    U = torch.from_numpy(state(M)).cuda()
+    lam = torch.from_numpy(I.random_directions(U.shape, 1)[0]).cuda()
+    out, ref, got = torch.empty_like(U), torch.empty_like(U), torch.empty_like(U)
+    dt, n = 1e-4, 40
+    face = 20 * M.nqf * M.ne * 8
+    dg.dg_set_state(M.handle, U)
+    dg.dg_rk3_step(M.handle, dt, n)
+    dg.dg_get_state(M.handle, ref)
+    dg.dg_residual_vjp(M.handle, U, lam, out)
+    want = out.clone()
+    used = shim.fake_in_use()
+    M.close()
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    for tight in (False, True):
+        # without the adjoint's second face buffer, or any room beyond it
+        shim.fake_limit(used - face // 2 if tight else 2 ** 64 - 1)
+        M = mesh(m)
+        for _ in range(3):
+            dg.dg_set_state(M.handle, U)
+            torch.cuda.synchronize()
+            dg.dg_rk3_step(M.handle, dt, n, stream=a)
+            for _ in range(4):
+                dg.dg_residual_vjp(M.handle, U, lam, out, stream=b)
+            dg.dg_get_state(M.handle, got, stream=a)
+            torch.cuda.synchronize()
+            assert torch.equal(got, ref) and torch.equal(out, want), tight
+        M.close()
+        shim.fake_limit(2 ** 64 - 1)
+
+
+{"creation": creation, "room": room, "streams": streams}[CHECK]()
 print("CHILD OK")

@@ -115,8 +115,8 @@ def test_fp32_ns_step_walled_odd(p, ne):
 
 @pytest.mark.parametrize("p", [1, 2, 3])
 def test_fp32_inviscid_ns_step_is_the_euler_step(p):
-    """With walls dg_rk3_step and dg_ns_rk3_step with mu = 0 sum the Euler lines in two orders: each within
-    the FP32 bar of the residual, so twice that of a step apart."""
+    """dg_rk3_step and dg_ns_rk3_step with mu = 0 may sum the Euler lines in two orders: each within the FP32
+    bar of the residual, so twice that of a step apart."""
     arrays = _walled(9731)
     scale_of = Problem(*arrays, p=1, flux="roe")
     M = _mesh(arrays, p, "roe", "fp32")

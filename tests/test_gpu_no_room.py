@@ -28,3 +28,10 @@ def _child(shim, check, precision, p):
 @pytest.mark.parametrize("precision,p", [("fp64", 1), ("fp32", 2), ("mixed", 2)])
 def test_refused_allocations_of_a_creation_leave_nothing(shim, precision, p):
     _child(shim, "creation", precision, p)
+
+
+@pytest.mark.parametrize("p", [1, 2, 3])
+@pytest.mark.parametrize("precision", ["fp32"])
+def test_calls_run_in_the_memory_they_cannot_do_without(shim, precision, p):
+    _child(shim, "room", precision, p)
+
