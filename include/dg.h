@@ -255,9 +255,11 @@ dg_status dg_boundary_flux(dg_mesh* mesh, const double* U, int stage, double out
  * interpolation, on both sides of every face; at a kink of |.| or max the
  * derivative of the branch taken, ties to the interior side).  U, lambda,
  * out: device FP64 [ne][5][Nb] in caller order.  The first call allocates the
- * adjoint's work buffers, owned by the mesh: six of the state's size and, in FP32
- * on larger meshes with room to spare and in FP64, two of 20 Nqf values per
- * element. */
+ * adjoint's work buffers, owned by the mesh: six of the state's size, and two of
+ * 20 Nqf values per element in FP64 and, with room to spare, on larger FP32
+ * meshes.  An FP64 mesh without room for the second of these works in the one
+ * of its RK steps: the call then waits for the device before it begins and for
+ * the stream before it returns. */
 dg_status dg_residual_vjp(dg_mesh* mesh, const double* U, const double* lambda, double* out, void* stream);
 
 /* out = (d U_{n+1} / d U_n)^T lambda for one SSP-RK3 step of size dt from

@@ -81,7 +81,7 @@ void free_mesh(dg_mesh* m) {
     cudaFree(m->d_farea);
     cudaFree(m->d_frec);
     cudaFree(m->d_fnorm);
-    cudaFree(m->d_TA);
+    if (m->d_TA != m->d_T) cudaFree(m->d_TA);
     cudaFree(m->d_TL);
     cudaFree(m->d_T);
     if (m->rk_exec) cudaGraphExecDestroy(m->rk_exec);
@@ -114,6 +114,7 @@ size_t pending_bytes(const dg_mesh* m) {
     want(m->d_io, ne * 5 * m->nb * sizeof(double));
     want(m->d_Z, ne * 15 * m->nb * rs);
     want(m->d_HB, dg::ns_face_buffer_values(m->p, ne) * rs);
+    if (m->precision == DG_FP64) want(m->d_TL, m->face_bytes());
     return n;
 }
 
@@ -792,8 +793,12 @@ dg_status ensure_adjoint_buffers(dg_mesh* m) {
         if (!b) DG_CUDA(cudaMalloc(&b, m->state_bytes() + 256));
     // face buffers apart from the RK steps', so that an adjoint call leaves a step on another stream alone
     if (m->precision == DG_FP64) {
-        if (!m->d_TA) DG_CUDA(cudaMalloc(&m->d_TA, m->face_bytes()));
         if (!m->d_TL) DG_CUDA(cudaMalloc(&m->d_TL, m->face_bytes()));
+        if (!m->adj_set) optional_buffer(m, &m->d_TA, m->face_bytes());
+        m->adj_set = true;
+        // without room for the second one, the steps' own, and nothing else may run meanwhile
+        if (!m->d_TA) m->d_TA = m->d_T;
+        if (m->d_TA == m->d_T) DG_CUDA(cudaDeviceSynchronize());
         return DG_OK;
     }
     // FP32: both, or the single kernel
@@ -806,6 +811,12 @@ dg_status ensure_adjoint_buffers(dg_mesh* m) {
         }
     }
     m->adj_set = true;   // refused once, not asked for again on every call
+    return DG_OK;
+}
+
+// the end of an adjoint call: on the steps' face buffer, it is done before the next call may begin
+dg_status leave_adjoint(dg_mesh* m, cudaStream_t s) {
+    if (m->d_TA && m->d_TA == m->d_T) DG_CUDA(cudaStreamSynchronize(s));
     return DG_OK;
 }
 }  // namespace
@@ -822,7 +833,7 @@ dg_status dg_residual_vjp(dg_mesh* m, const double* U, const double* lambda, dou
     DG_CUDA(dg::launch_gather(m, lambda, V[1], s));
     DG_CUDA(dg::launch_residual_vjp(m, V[0], V[1], nullptr, nullptr, nullptr, c, V[2], s));
     DG_CUDA(dg::launch_scatter(m, V[2], out, s));
-    return DG_OK;
+    return leave_adjoint(m, s);
 }
 
 dg_status dg_rk3_step_vjp(dg_mesh* m, const double* U0, double dt, const double* lambda, double* out, void* stream) {
@@ -844,7 +855,7 @@ dg_status dg_rk3_step_vjp(dg_mesh* m, const double* U0, double dt, const double*
     const double c0[4] = {1.0 / 3.0, 0.75, 1.0, dt};              // lambda/3 + 3/4 m2 + m1 + dt J(U0)^T m1
     DG_CUDA(dg::launch_residual_vjp(m, V[0], V[5], V[1], V[4], V[5], c0, V[3], s));
     DG_CUDA(dg::launch_scatter(m, V[3], out, s));
-    return DG_OK;
+    return leave_adjoint(m, s);
 }
 
 dg_status dg_kinetic_energy_grad(dg_mesh* m, const double* U, double* out, void* stream) {

@@ -31,7 +31,10 @@ def test_refused_allocations_of_a_creation_leave_nothing(shim, precision, p):
 
 
 @pytest.mark.parametrize("p", [1, 2, 3])
-@pytest.mark.parametrize("precision", ["fp32"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
 def test_calls_run_in_the_memory_they_cannot_do_without(shim, precision, p):
     _child(shim, "room", precision, p)
 
+
+def test_adjoint_leaves_steps_on_another_stream_alone(shim):
+    _child(shim, "streams", "fp64", 3)
