@@ -84,7 +84,9 @@ struct dg_mesh {
     int32_t* d_mhdr = nullptr;
     int32_t* d_mxnbr = nullptr;
     void* d_B[3] = {nullptr, nullptr, nullptr};   // state buffers (internal precision)
-    void* d_V[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};   // adjoint work buffers (lazy)
+    // adjoint work buffers, one allocation d_adj (lazy): states d_V, and the face buffers below
+    void* d_adj = nullptr;
+    void* d_V[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     // residual / totals work buffers (lazy): a caller's state in internal order, and the residual
     // in internal order; kept apart from d_B so these calls never touch an RK step in progress
     void* d_W[2] = {nullptr, nullptr};
@@ -113,7 +115,7 @@ struct dg_mesh {
     int64_t n_flist = 0, n_interior = 0, n_trace = 0;   // listed faces, interior ones among them
     void* d_T = nullptr;
     void *d_TA = nullptr, *d_TL = nullptr;
-    bool ns_set = false, adj_set = false;   // the optional buffers of these calls have been asked for
+    bool ns_set = false;           // the optional buffer of the viscous passes has been asked for
     size_t face_bytes() const;
     // small meshes: a CUDA graph of several captured RK3 steps at one dt (dg_rk3_step)
     cudaStream_t cap_stream = nullptr;
