@@ -491,9 +491,9 @@ __global__ void __launch_bounds__(threads_of(EE)) k_element(ResArgs<Real> a) {
     auto flux = [&](int q, Real* g) {
         Real w[4];
         load_row<4>(sW + (q * EE + e) * 4, w);
-        const Real b = fma(s4, w[3], sU[q * ER + t]);
+        const Real b = modal::madd(s4, w[3], sU[q * ER + t]);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) g[k] = fma(w[k], b, fma(w[3], Jk[k], -G0[k]));
+        for (int k = 0; k < 3; ++k) g[k] = modal::madd(w[k], b, modal::madd(w[3], Jk[k], -G0[k]));
     };
     if (live) {
         if (S::F32) flux(NQ, G0);
@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(32 * WIDE) k_element_wide(ResArgs<double> a) {
         for (int m = 0; m < NM; ++m) M[m] = 0;
         auto flux = [&](int q) {
             const Real wk = sW[(q * EE + e) * 4 + w], p = sW[(q * EE + e) * 4 + 3];
-            return fma(wk, fma(s4, p, sU[q * ER + l]), fma(p, Jk, -G0));
+            return modal::madd(wk, modal::madd(s4, p, sU[q * ER + l]), modal::madd(p, Jk, -G0));
         };
         modal::unroll<0, NQ>([&](auto qc) {
             constexpr int q = qc.value, m = modal::kT<P>.vmir[q];
@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(32 * WIDE) k_element_wide(ResArgs<double> a) {
         const Real s0 = -sG[4 * e], s1 = -sG[4 * e + 1];
 #pragma unroll
         for (int m = 0; m < NF; ++m) {
-            const Real x = s0 * sA[m * ER + l], b = sA[(NF + m) * ER + l], ev = fma(s1, b, x), od = fma(s1, b, -x);
+            const Real x = s0 * sA[m * ER + l], b = sA[(NF + m) * ER + l], ev = modal::madd(s1, b, x), od = modal::madd(s1, b, -x);
 #pragma unroll
             for (int j = J0; j < J1; ++j) modal::axpy(r[j - J0], T.E[1][m][j], T.odd[j] ? od : ev);
         }

@@ -249,6 +249,11 @@ __device__ __forceinline__ void unroll(F&& f) {
     unroll_seq<First>(f, std::make_integer_sequence<int, Last - First>());
 }
 
+// a b + c: in FP64 one rounding by definition, since kernels that must agree bitwise share the expression (in
+// FP32 left to the compiler, which needs fewer registers for it)
+__device__ __forceinline__ double madd(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float madd(float a, float b, float c) { return a * b + c; }
+
 // r += c x with a compile-time constant; nothing where it is zero
 template <typename Real>
 __device__ __forceinline__ void axpy(Real& r, double c, Real x) {
@@ -417,7 +422,7 @@ __device__ __forceinline__ void lift(Load load, Real* r) {
         face_moments<Real, P>(h, b);
 #pragma unroll
         for (int m = 0; m < T.NF; ++m) {
-            const Real x = s0 * a[m], e = fma(s1, b[m], x), o = fma(s1, b[m], -x);
+            const Real x = s0 * a[m], e = madd(s1, b[m], x), o = madd(s1, b[m], -x);
 #pragma unroll
             for (int j = 0; j < T.NB; ++j) axpy(r[j], T.E[1][m][j], T.odd[j] ? o : e);
         }
