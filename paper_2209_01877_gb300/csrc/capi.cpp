@@ -79,7 +79,6 @@ void free_mesh(dg_mesh* m) {
     cudaFree(m->d_wslot);
     cudaFree(m->d_farea);
     cudaFree(m->d_frec);
-    cudaFree(m->d_fnorm);
     cudaFree(m->d_adj);
     cudaFree(m->d_T);
     if (m->rk_exec) cudaGraphExecDestroy(m->rk_exec);
@@ -276,7 +275,7 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
         DG_TRY(upload(&m->d_mxnbr, xnbr.data(), xnbr.size(), s));
     }
     if (m->precision == DG_FP64) {
-        cudaError_t e = dg::setup_face_once(m, m, 0, ne, s);
+        cudaError_t e = dg::setup_face_once(m, m, 0, ne, true, s);
         if (e == cudaSuccess) e = cudaMalloc(&m->d_T, m->face_bytes());
         if (e != cudaSuccess) { free_mesh(m); return cuda_fail(e, "face buffers"); }
     }
@@ -303,8 +302,8 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
         // FP32: the face list and, where the Euler stages use it, the face buffer; last, and only with room
         // to spare: without them the mesh runs the kernels that need none
         if (e == cudaSuccess && m->precision == DG_FP32 && faces_in_use(m) &&
-            room_for(m, m->host.n_faces * (sizeof(dg::FaceRec) + 3 * sizeof(float)))) {
-            e = dg::setup_face_once(m, m, 0, ne, s);
+            room_for(m, dg::face_list_bytes(m->host.n_faces, DG_FP32, vjp_by_faces(m)))) {
+            e = dg::setup_face_once(m, m, 0, ne, vjp_by_faces(m), s);
             if (e == cudaErrorMemoryAllocation) e = (cudaGetLastError(), cudaSuccess);
         }
         if (e == cudaSuccess && m->face_once && m->precision == DG_FP32 && fp32_stage_faces(m))

@@ -110,8 +110,9 @@ struct dg_mesh {
     // place): d_T of the RK steps (FP64: of every residual; FP32: where the stages use it and there is
     // room); lazy, the adjoint's own: d_TA, d_TL the direction's traces
     bool face_once = false;
-    dg::FaceRec* d_frec = nullptr;
+    dg::FaceRec* d_frec = nullptr;   // the allocation that holds the next two as well
     void* d_fnorm = nullptr;       // Real [n_flist][3]
+    void* d_fscale = nullptr;      // Real [n_flist][2], the two sides' |grad lambda| (the adjoint)
     int64_t n_flist = 0, n_interior = 0, n_trace = 0;   // listed faces, interior ones among them
     void* d_T = nullptr;
     void *d_TA = nullptr, *d_TL = nullptr;
@@ -130,13 +131,13 @@ namespace dg {
 cudaError_t launch_residual(dg_mesh* m, const void* U, const void* U0, void* out, int mode,
                             double dt, double a, double b, void* T, cudaStream_t s);
 // the face-once path's device data for m, whose elements are [first, first + ne) of whole (m itself, or a
-// partition's mesh in local numbers, own elements and then halo): the face list, boundary faces last, and
-// the owners' normals; n_trace is the number of elements with traces
-cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int64_t n_trace, cudaStream_t s);
-// face traces of a state of the mesh's precision, into the face buffer T; the adjoint's: of U into T,
-// and of lam times each face's |grad lambda_f| into TL
-cudaError_t launch_traces(dg_mesh* m, const void* U, void* T, cudaStream_t s);
-cudaError_t launch_traces_vjp(dg_mesh* m, const void* U, void* T, const void* lam, void* TL, cudaStream_t s);
+// partition's mesh in local numbers, own elements and then halo): the face list, boundary faces last,
+// the owners' normals and, where the adjoint may want them, the two sides' scales, in one allocation; n_trace is the
+// number of elements with traces
+cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int64_t n_trace, bool scales, cudaStream_t s);
+size_t face_list_bytes(int64_t n, int precision, bool scales);
+// face traces of two states of the mesh's precision (U1 may be null), into the face buffers T and T1
+cudaError_t launch_traces2(dg_mesh* m, const void* U, void* T, const void* U1, void* T1, cudaStream_t s);
 cudaError_t launch_gather(dg_mesh* m, const double* user, void* internal, cudaStream_t s);   // caller -> internal
 cudaError_t launch_gather_f32(dg_mesh* m, const double* user, float* internal, cudaStream_t s);   // FP32 (a hi plane) only
 // Navier-Stokes lines: the BR1 gradient into Z, then the viscous volume and face terms added to

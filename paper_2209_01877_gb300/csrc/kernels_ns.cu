@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(256) k_rk_axpy_ff(const float* __restrict__ U,
 template <typename Real>
 cudaError_t ns_dispatch(dg_mesh* m, const void* U, void* T, void* Z, void* HB, void* R, double mu, double prandtl,
                         cudaStream_t s) {
-    cudaError_t e = launch_traces(m, U, T, s);
+    cudaError_t e = launch_traces2(m, U, T, nullptr, nullptr, s);
     if (e != cudaSuccess) return e;
     NSArgs<Real> a;
     a.U = static_cast<const Real*>(U);

@@ -278,38 +278,22 @@ __device__ __forceinline__ double face_scale(const double* I, int f) {
 // coefficients and traces pass through shared memory, so that the global accesses are whole lines:
 // rows written directly (24 to 48 bytes each) kept the load-store unit busy (P2, 663,552 elements:
 // 127 us at 39 % of the DRAM rate).  FP64 is bound by its pipe and writes its rows directly.
-// SCALED: the second state's traces are multiplied by |grad lambda_f| of the element's face (the
-// adjoint's direction), four square roots per element.
-template <typename Real, int P, int EE, bool SCALED>
+template <typename Real, int P, int EE>
 __global__ void __launch_bounds__(threads_of(EE), EE == 32 ? (sizeof(Real) == 8 ? (P == 3 ? 3 : P == 2 ? 6 : 10) : (P == 3 ? 5 : 10)) : 14)
-    k_traces(const Real* U0, Real* T0, const Real* U1, Real* T1, const double* __restrict__ jinv, int64_t ne) {
+    k_traces(const Real* U0, Real* T0, const Real* U1, Real* T1, int64_t ne) {
     constexpr int NB = nb_of(P), NQF = nqf_of(P), NT = threads_of(EE);
-    __shared__ Real sS[SCALED ? 4 * EE : 1];
     const Real* __restrict__ U = blockIdx.y == 0 ? U0 : U1;
     Real* __restrict__ T = blockIdx.y == 0 ? T0 : T1;
     const int t = threadIdx.x;
     const int64_t e0 = blockIdx.x * (int64_t)EE;
     const int nel = (ne - e0) < (int64_t)EE ? (int)(ne - e0) : EE;
     const int e = t / 5, v = t - 5 * e;
-    const bool scaled = SCALED && blockIdx.y == 1;
-    if (scaled) {
-        if (t < 4 * nel) sS[t] = (Real)face_scale(jinv + (e0 + (t >> 2)) * 9, t & 3);
-        __syncthreads();
-    }
-    // a face's traces, times its scale where one is asked for
-    auto put = [&](Real* o, int f, const Real* u) {
-        Real x[NQF];
-        const Real s = scaled ? sS[SCALED ? 4 * e + f : 0] : Real(1);
-#pragma unroll
-        for (int q = 0; q < NQF; ++q) x[q] = SCALED ? s * u[q] : u[q];
-        store_row<NQF>(o + f * 5 * NQF, x);
-    };
     if constexpr (sizeof(Real) == 8) {
         if (t >= 5 * nel) return;
         Real c[NB];
         load_row<NB>(U + (e0 * 5 + t) * NB, c);
         Real* o = T + ((e0 + e) * 20 + v) * NQF;
-        modal::traces<Real, P>(c, [&](int f, const Real* u) { put(o, f, u); });
+        modal::traces<Real, P>(c, [&](int f, const Real* u) { store_row<NQF>(o + f * 5 * NQF, u); });
     } else {
         __shared__ __align__(16) Real sU[rows_of(EE) * NB + 4], sT[EE * 20 * NQF];
         copy_tile<NT>(sU, U + e0 * 5 * NB, nel * 5 * NB * (int)sizeof(Real));
@@ -319,7 +303,7 @@ __global__ void __launch_bounds__(threads_of(EE), EE == 32 ? (sizeof(Real) == 8 
             Real c[NB];
             load_row<NB>(sU + t * NB, c);
             Real* o = sT + (e * 20 + v) * NQF;
-            modal::traces<Real, P>(c, [&](int f, const Real* u) { put(o, f, u); });
+            modal::traces<Real, P>(c, [&](int f, const Real* u) { store_row<NQF>(o + f * 5 * NQF, u); });
         }
         __syncthreads();
         float4* g = reinterpret_cast<float4*>(T + e0 * 20 * NQF);
@@ -327,14 +311,14 @@ __global__ void __launch_bounds__(threads_of(EE), EE == 32 ? (sizeof(Real) == 8 
     }
 }
 
-template <typename Real, int P, bool SCALED>
-cudaError_t traces(const void* U, void* T, const void* U1, void* T1, const double* jinv, int64_t ne, cudaStream_t s) {
+template <typename Real, int P>
+cudaError_t traces(const void* U, void* T, const void* U1, void* T1, int64_t ne, cudaStream_t s) {
     const Real *u = static_cast<const Real*>(U), *u1 = static_cast<const Real*>(U1);
     Real *t = static_cast<Real*>(T), *t1 = static_cast<Real*>(T1);
     if (small_tiles(ne))
-        k_traces<Real, P, 6, SCALED><<<dim3((unsigned)((ne + 5) / 6), U1 ? 2 : 1), threads_of(6), 0, s>>>(u, t, u1, t1, jinv, ne);
+        k_traces<Real, P, 6><<<dim3((unsigned)((ne + 5) / 6), U1 ? 2 : 1), threads_of(6), 0, s>>>(u, t, u1, t1, ne);
     else
-        k_traces<Real, P, 32, SCALED><<<dim3((unsigned)((ne + 31) / 32), U1 ? 2 : 1), threads_of(32), 0, s>>>(u, t, u1, t1, jinv, ne);
+        k_traces<Real, P, 32><<<dim3((unsigned)((ne + 31) / 32), U1 ? 2 : 1), threads_of(32), 0, s>>>(u, t, u1, t1, ne);
     return cudaGetLastError();
 }
 
@@ -724,7 +708,7 @@ cudaError_t launch_face_once(dg_mesh* m, ResArgs<Real>& r, bool rk, void* T, cud
     f.roe_eps = r.roe_eps;
     for (int v = 0; v < 5; ++v) f.finf[v] = r.finf[v];
     f.status = m->d_status;
-    cudaError_t e = traces<Real, P, false>(r.U, f.T, nullptr, nullptr, nullptr, m->n_trace, s);
+    cudaError_t e = traces<Real, P>(r.U, f.T, nullptr, nullptr, m->n_trace, s);
     if (e != cudaSuccess) return e;
     if (f.n > 0) {
         const unsigned nt = face_block(f.n), grid = (unsigned)((f.n + nt - 1) / nt);
@@ -868,22 +852,34 @@ cudaError_t list_faces(const ListArgs& a, int32_t* counts, FaceRec* out, int64_t
     return cudaGetLastError();
 }
 
-// outward unit normals -grad lambda_f / |grad lambda_f| of the listed faces' owning slots
+// per listed face the owner's outward unit normal -grad lambda_f / |grad lambda_f| and, with scales, the
+// |grad lambda| of the slot's element and of the matching one
 template <typename Real>
-__global__ void k_face_normals(const double* __restrict__ jinv, const FaceRec* __restrict__ rec, int64_t n, Real* out) {
+__global__ void k_face_geometry(const double* __restrict__ jinv, const FaceRec* __restrict__ rec, int64_t n, Real* normal,
+                                Real* scale) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int32_t slot = rec[i].owner;
-    const double* I = jinv + (int64_t)(slot >> 2) * 9;
-    const int f = slot & 3;
+    auto gradient = [&](int32_t slot, double* g) {
+        const double* I = jinv + (int64_t)(slot >> 2) * 9;
+        const int f = slot & 3;
+        for (int d = 0; d < 3; ++d) g[d] = f == 0 ? -(I[d] + I[3 + d] + I[6 + d]) : I[3 * (f - 1) + d];
+        return sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
+    };
+    const FaceRec r = rec[i];
     double g[3];
-    for (int d = 0; d < 3; ++d) g[d] = f == 0 ? -(I[d] + I[3 + d] + I[6 + d]) : I[3 * (f - 1) + d];
-    const double gn = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
-    for (int d = 0; d < 3; ++d) out[3 * i + d] = (Real)(-g[d] / gn);
+    const double gn = gradient(r.owner, g);
+    for (int d = 0; d < 3; ++d) normal[3 * i + d] = (Real)(-g[d] / gn);
+    if (!scale) return;
+    scale[2 * i] = (Real)gradient(r.slot, g);
+    scale[2 * i + 1] = r.other >= 0 ? (Real)gradient(r.other, g) : Real(0);
 }
 }  // namespace
 
-cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int64_t n_trace, cudaStream_t s) {
+size_t face_list_bytes(int64_t n, int precision, bool scales) {
+    return n * (sizeof(FaceRec) + (scales ? 5 : 3) * (precision == DG_FP64 ? 8 : 4));
+}
+
+cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int64_t n_trace, bool scales, cudaStream_t s) {
     const int64_t slots = 4 * m->host.ne;
     int32_t nbnd = 0, nhalo = 0;
     for (int64_t i = 0; i < slots; ++i) {
@@ -893,57 +889,38 @@ cudaError_t setup_face_once(dg_mesh* m, const dg_mesh* whole, int64_t first, int
     m->n_interior = (slots - nbnd - nhalo) / 2 + nhalo;
     const int64_t n = m->n_flist = m->n_interior + nbnd;
     m->n_trace = n_trace;
-    cudaError_t e = cudaMalloc(&m->d_frec, n * sizeof(FaceRec));
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_fnorm, n * 3 * (m->precision == DG_FP64 ? 8 : 4));
+    cudaError_t e = cudaMalloc(&m->d_frec, face_list_bytes(n, m->precision, scales));   // records, normals, scales
+    if (e != cudaSuccess) return e;
+    const bool f64 = m->precision == DG_FP64;
+    m->d_fnorm = m->d_frec + n;
+    m->d_fscale = scales ? static_cast<char*>(m->d_fnorm) + 3 * n * (f64 ? 8 : 4) : nullptr;
     const ListArgs a{m->d_nbr, m->d_fcode, whole->d_nbr, whole->d_perm, m->host.ne, first};
     // the normals' place, written last, holds the counts: at least 24 bytes an element (n >= 2 ne) against 4 per LT slots
     int32_t* counts = static_cast<int32_t*>(m->d_fnorm);
-    if (e == cudaSuccess) e = list_faces<false>(a, counts, m->d_frec, m->n_interior, s);
+    e = list_faces<false>(a, counts, m->d_frec, m->n_interior, s);
     if (e == cudaSuccess) e = list_faces<true>(a, counts, m->d_frec + m->n_interior, nbnd, s);
     if (e == cudaSuccess) {
         const unsigned grid = (unsigned)((n + 255) / 256);
-        if (m->precision == DG_FP64)
-            k_face_normals<double><<<grid, 256, 0, s>>>(whole->d_jinv64, m->d_frec, n, static_cast<double*>(m->d_fnorm));
+        if (f64)
+            k_face_geometry<double><<<grid, 256, 0, s>>>(whole->d_jinv64, m->d_frec, n, static_cast<double*>(m->d_fnorm),
+                                                         static_cast<double*>(m->d_fscale));
         else
-            k_face_normals<float><<<grid, 256, 0, s>>>(whole->d_jinv64, m->d_frec, n, static_cast<float*>(m->d_fnorm));
+            k_face_geometry<float><<<grid, 256, 0, s>>>(whole->d_jinv64, m->d_frec, n, static_cast<float*>(m->d_fnorm),
+                                                        static_cast<float*>(m->d_fscale));
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) {
-        m->face_once = true;
-        return e;
+    m->face_once = e == cudaSuccess;
+    return e;   // a mesh whose launch failed is given up
+}
+
+cudaError_t launch_traces2(dg_mesh* m, const void* U, void* T, const void* U1, void* T1, cudaStream_t s) {
+    const int64_t n = m->host.ne;
+    const bool f64 = m->precision == DG_FP64;
+    switch (m->p) {
+        case 1: return f64 ? traces<double, 1>(U, T, U1, T1, n, s) : traces<float, 1>(U, T, U1, T1, n, s);
+        case 2: return f64 ? traces<double, 2>(U, T, U1, T1, n, s) : traces<float, 2>(U, T, U1, T1, n, s);
+        default: return f64 ? traces<double, 3>(U, T, U1, T1, n, s) : traces<float, 3>(U, T, U1, T1, n, s);
     }
-    // nothing half made stays: an FP32 mesh goes on without
-    cudaFree(m->d_frec);
-    cudaFree(m->d_fnorm);
-    m->d_frec = nullptr;
-    m->d_fnorm = nullptr;
-    return e;
-}
-
-cudaError_t launch_traces(dg_mesh* m, const void* U, void* T, cudaStream_t s) {
-    const int64_t n = m->host.ne;
-    const bool f64 = m->precision == DG_FP64;
-    auto go = [&](auto p) {
-        constexpr int P = decltype(p)::value;
-        return f64 ? traces<double, P, false>(U, T, nullptr, nullptr, nullptr, n, s)
-                   : traces<float, P, false>(U, T, nullptr, nullptr, nullptr, n, s);
-    };
-    return m->p == 1 ? go(std::integral_constant<int, 1>())
-           : m->p == 2 ? go(std::integral_constant<int, 2>())
-                       : go(std::integral_constant<int, 3>());
-}
-
-cudaError_t launch_traces_vjp(dg_mesh* m, const void* U, void* T, const void* lam, void* TL, cudaStream_t s) {
-    const int64_t n = m->host.ne;
-    const bool f64 = m->precision == DG_FP64;
-    auto go = [&](auto p) {
-        constexpr int P = decltype(p)::value;
-        return f64 ? traces<double, P, true>(U, T, lam, TL, m->d_jinv64, n, s)
-                   : traces<float, P, true>(U, T, lam, TL, m->d_jinv64, n, s);
-    };
-    return m->p == 1 ? go(std::integral_constant<int, 1>())
-           : m->p == 2 ? go(std::integral_constant<int, 2>())
-                       : go(std::integral_constant<int, 3>());
 }
 
 cudaError_t launch_residual(dg_mesh* m, const void* U, const void* U0, void* out, int mode, double dt, double a,

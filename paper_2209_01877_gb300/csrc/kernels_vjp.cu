@@ -1,8 +1,8 @@
 // Adjoint of the residual: out = (dR/dU)^T lambda (FP64 / FP32, CUDA cores).
 // The paper has no adjoint; this is the reverse of the forward kernels' steps, in the same three
 // launches with every face once:
-//   k_traces       (kernels_simt.cu) the traces of U and of s lambda at the points of every face, to
-//                  two face buffers (s = |grad lambda_f| of the element's own face);
+//   k_traces       (kernels_simt.cu) the traces of U and of lambda at the points of every face, to
+//                  two face buffers;
 //   k_faces_vjp    thread per (interior face, point): the flux H(U_owner, U_other, n_owner) enters the
 //                  owner's residual with -s wf and the other's with +s' wf, so its cotangent is
 //                  s' lambda_other - s lambda_owner (wf is applied by the lift below); one reverse
@@ -341,9 +341,10 @@ inline unsigned vface_block(int64_t n) { return n < (int64_t)VF * 4 * 152 ? 32 :
 template <typename Real>
 struct FaceVjpArgs {
     Real* T;                // traces of U in, face adjoints out [ne][4][5][Nqf]
-    const Real* TL;         // traces of lambda times the face's |grad lambda_f|
+    const Real* TL;         // traces of lambda
     const FaceRec* rec;
     const Real* normal;     // [faces][3]
+    const Real* scale;      // [faces][2] |grad lambda_f| of the slot and of the matching one
     const int8_t* fperm;
     int64_t n;              // faces x Nqf
     Real gamma, roe_eps;
@@ -359,14 +360,15 @@ __global__ void __launch_bounds__(VF) k_faces_vjp(FaceVjpArgs<Real> a) {
     const int q = (int)(i - li * NQF);
     const int4 f = *reinterpret_cast<const int4*>(a.rec + li);   // slot (the owner's), other, code
     const Real n[3] = {a.normal[3 * li], a.normal[3 * li + 1], a.normal[3 * li + 2]};
+    const Real so = a.scale[2 * li], sn = a.scale[2 * li + 1];
     const int64_t oe = (int64_t)f.x * 5 * NQF + q, on = (int64_t)f.y * 5 * NQF + a.fperm[(f.z & 7) * NQF + q];
     Real L[5], R[5], Ho[5], Hn[5], Hb[5], Lb[5], Rb[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
         L[v] = a.T[oe + v * NQF];
         R[v] = a.T[on + v * NQF];
-        Ho[v] = -a.TL[oe + v * NQF];
-        Hn[v] = a.TL[on + v * NQF];
+        Ho[v] = -so * a.TL[oe + v * NQF];
+        Hn[v] = sn * a.TL[on + v * NQF];
         Hb[v] = Ho[v] + Hn[v];
     }
     if (face_reverse<Real, FLUX>(L, R, n, a.gamma, a.roe_eps, Hb, Real(1), Lb, Rb)) {
@@ -395,6 +397,7 @@ __global__ void __launch_bounds__(VF) k_bfaces_vjp(FaceVjpArgs<Real> a) {
     const int64_t li = i / NQF;
     const int q = (int)(i - li * NQF);
     const int4 f = *reinterpret_cast<const int4*>(a.rec + li);
+    const Real s = a.scale[2 * li];
     const int64_t oe = (int64_t)f.x * 5 * NQF + q;
     D5 U[5], G[5], n[3], Fi[5], H[5];
     const D5 g = D5(a.gamma), eps = D5(a.roe_eps);
@@ -412,7 +415,7 @@ __global__ void __launch_bounds__(VF) k_bfaces_vjp(FaceVjpArgs<Real> a) {
     Real ub[5] = {0, 0, 0, 0, 0};
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
-        const Real hb = -a.TL[oe + v * NQF];
+        const Real hb = -s * a.TL[oe + v * NQF];
 #pragma unroll
         for (int k = 0; k < 5; ++k) ub[k] += H[v].d[k] * hb;
     }
@@ -557,13 +560,14 @@ cudaError_t vlaunch_tiles(const VjpArgs<Real>& r, const Real* UB, cudaStream_t s
 template <typename Real, int P, int FLUX>
 cudaError_t vlaunch_faces(dg_mesh* m, const VjpArgs<Real>& r, cudaStream_t s) {
     constexpr int NQF = nqf_of(P);
-    cudaError_t e = launch_traces_vjp(m, r.U, m->d_TA, r.lam, m->d_TL, s);
+    cudaError_t e = launch_traces2(m, r.U, m->d_TA, r.lam, m->d_TL, s);
     if (e != cudaSuccess) return e;
     FaceVjpArgs<Real> f;
     f.T = static_cast<Real*>(m->d_TA);
     f.TL = static_cast<const Real*>(m->d_TL);
     f.rec = m->d_frec;
     f.normal = static_cast<const Real*>(m->d_fnorm);
+    f.scale = static_cast<const Real*>(m->d_fscale);
     f.fperm = m->d_fperm;
     f.n = m->n_interior * NQF;
     f.gamma = r.gamma;
@@ -575,6 +579,7 @@ cudaError_t vlaunch_faces(dg_mesh* m, const VjpArgs<Real>& r, cudaStream_t s) {
     if (nb > 0) {
         f.rec += m->n_interior;
         f.normal += 3 * m->n_interior;
+        f.scale += 2 * m->n_interior;
         f.n = nb * NQF;
         nt = vface_block(f.n);
         k_bfaces_vjp<Real, P, FLUX><<<(unsigned)((f.n + nt - 1) / nt), nt, 0, s>>>(f);

@@ -156,7 +156,6 @@ void free_sub(dg_mesh* s) {
     cudaFree(s->d_jinv64);
     cudaFree(s->d_red);
     cudaFree(s->d_frec);
-    cudaFree(s->d_fnorm);
     cudaFree(s->d_T);
     delete s;
 }
@@ -259,7 +258,7 @@ dg_status dg_partition_create(dg_mesh* m, int k, void* stream, dg_partition** ou
         // are evaluated here too, in their owner's orientation, so every own element receives the
         // flux the whole mesh would give it
         if (m->precision == DG_FP64) {
-            PTRY(dg::setup_face_once(sm, m, pl.first, pl.count + (int64_t)pl.halo.size(), s));
+            PTRY(dg::setup_face_once(sm, m, pl.first, pl.count + (int64_t)pl.halo.size(), false, s));
             PTRY(cudaMalloc(&sm->d_T, sm->face_bytes()));
         }
         // local state: own then halo blocks (mixed: hi plane of own + halo, then the lo plane)
