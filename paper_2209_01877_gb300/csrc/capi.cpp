@@ -73,8 +73,6 @@ void free_mesh(dg_mesh* m) {
     for (auto& b : m->d_W) cudaFree(b);
     cudaFree(m->d_io);
     cudaFree(m->d_Z);
-    cudaFree(m->d_HB);
-    if (m->d_TN != m->d_T) cudaFree(m->d_TN);
     cudaFree(m->d_hs);
     cudaFree(m->d_wslot);
     cudaFree(m->d_farea);
@@ -101,37 +99,37 @@ dg_status ensure_work_buffers(dg_mesh* m) {
 constexpr size_t ALLOC_GRAIN = 2 << 20;   // what an allocation may take from the device at least
 size_t grains(size_t bytes) { return (bytes + ALLOC_GRAIN - 1) / ALLOC_GRAIN * ALLOC_GRAIN; }
 
-// What the calls on a mesh may still allocate on their first use, for its FP64 and FP32 forms; the adjoint's alone.
-enum Pending { PENDING_ALL, PENDING_ADJOINT };
+size_t whole(size_t bytes) { return (bytes + 255) / 256 * 256; }   // parts of one allocation
+
+// What the calls on an FP64 or FP32 mesh may still allocate on their first use: the adjoint's, the viscous
+// passes', all.
 size_t pending_adjoint(const dg_mesh* m) {
     return m->d_adj ? 0 : grains(6 * (m->state_bytes() + 512) + (m->precision == DG_FP64 ? m->face_bytes() + 256 : 0));
 }
+size_t pending_ns(const dg_mesh* m) {
+    const size_t ne = m->host.ne, values = ne * 15 * m->nb + dg::ns_face_buffer_values(m->p, ne);
+    return m->d_Z ? 0 : grains(values * real_size(m->precision) + 256);
+}
 size_t pending_bytes(const dg_mesh* m) {
-    const size_t ne = m->host.ne, rs = real_size(m->precision);
-    size_t n = 0;
-    auto want = [&](const void* p, size_t bytes) { n += p ? 0 : grains(bytes); };
-    for (const void* b : m->d_W) want(b, m->state_bytes() + 256);
-    want(m->d_io, ne * 5 * m->nb * sizeof(double));
-    want(m->d_Z, ne * 15 * m->nb * rs);
-    want(m->d_HB, dg::ns_face_buffer_values(m->p, ne) * rs);
-    return n + pending_adjoint(m);
+    size_t n = pending_adjoint(m) + pending_ns(m);
+    for (const void* b : m->d_W) n += b ? 0 : grains(m->state_bytes() + 256);
+    return n + (m->d_io ? 0 : grains((size_t)m->host.ne * 5 * m->nb * sizeof(double)));
 }
 
-// Whether `bytes` more leave room for those: a buffer that a mesh can do without must not be the reason for
-// which a later call on it runs out of memory.
-bool room_for(const dg_mesh* m, size_t bytes, Pending part_of = PENDING_ALL) {
+// Whether `bytes` more leave room for those, less `covered` of them that the bytes stand for: a buffer that a
+// mesh can do without must not be the reason for which a later call on it runs out of memory.
+bool room_for(const dg_mesh* m, size_t bytes, size_t covered = 0) {
     size_t free_bytes = 0, total = 0;
     if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
-    // a buffer that holds the adjoint's needs too stands for them
-    return free_bytes >= grains(bytes) + pending_bytes(m) - (part_of == PENDING_ADJOINT ? pending_adjoint(m) : 0);
+    return free_bytes >= grains(bytes) + pending_bytes(m) - covered;
 }
 
 // a buffer that the mesh can do without: left null where there is no such room
-void optional_buffer(const dg_mesh* m, void** buf, size_t bytes, Pending part_of = PENDING_ALL) {
-    if (!room_for(m, bytes, part_of)) return;
+void optional_buffer(const dg_mesh* m, void** buf, size_t bytes, size_t covered = 0) {
+    if (!room_for(m, bytes, covered)) return;
     if (cudaMalloc(buf, bytes) != cudaSuccess) {
         (void)cudaGetLastError();
         *buf = nullptr;
@@ -502,14 +500,22 @@ bool ns_by_rows(const dg_mesh* m) {
     return m->precision == DG_FP64 || (m->precision == DG_FP32 && (m->p > 1 || m->host.ne >= 6000));
 }
 
+// One allocation: the gradient, the face fluxes and, in FP32 with room to spare, the traces of U (FP64 has the
+// steps' face buffer for them: the Euler residual is done with it).
 dg_status ensure_ns_buffers(dg_mesh* m) {
-    const size_t rs = m->precision == DG_FP64 ? sizeof(double) : sizeof(float);
-    if (!m->d_Z) DG_CUDA(cudaMalloc(&m->d_Z, (size_t)m->host.ne * 15 * m->nb * rs));
-    if (!m->d_HB) DG_CUDA(cudaMalloc(&m->d_HB, dg::ns_face_buffer_values(m->p, m->host.ne) * rs));
+    if (m->d_Z) return DG_OK;
+    const size_t rs = m->precision == DG_FP64 ? sizeof(double) : sizeof(float), ne = m->host.ne;
+    const size_t z = ne * 15 * m->nb * rs, hb = dg::ns_face_buffer_values(m->p, ne) * rs, tn = ne * 20 * m->nqf * rs;
+    bool traces = false;
+    if (m->precision == DG_FP32 && ns_by_rows(m)) {
+        optional_buffer(m, reinterpret_cast<void**>(&m->d_Z), whole(z) + whole(hb) + tn, pending_ns(m));
+        traces = m->d_Z != nullptr;
+    }
+    if (!m->d_Z) DG_CUDA(cudaMalloc(&m->d_Z, whole(z) + hb));
+    char* p = reinterpret_cast<char*>(m->d_Z) + whole(z);
+    m->d_HB = reinterpret_cast<double*>(p);
     if (m->precision == DG_FP64) m->d_TN = m->d_T;
-    if (m->precision == DG_FP32 && ns_by_rows(m) && !m->ns_set)
-        optional_buffer(m, &m->d_TN, (size_t)m->host.ne * 20 * m->nqf * rs);
-    m->ns_set = true;   // refused once, not asked for again on every call
+    if (traces) m->d_TN = p + whole(hb);
     return DG_OK;
 }
 }  // namespace
@@ -792,7 +798,6 @@ namespace {
 // call of a 1,296-element FP32 P3 mesh 270 us where one makes it 140).  The face buffers are apart from the RK
 // steps', so that an adjoint call leaves a step on another stream alone.
 dg_status ensure_adjoint_buffers(dg_mesh* m) {
-    auto whole = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
     if (!m->d_adj) {
         const size_t state = whole(m->state_bytes() + 256), face = whole(m->face_bytes());
         const bool f64 = m->precision == DG_FP64;
@@ -800,7 +805,7 @@ dg_status ensure_adjoint_buffers(dg_mesh* m) {
         // kernel)
         int faces = m->face_once && vjp_by_faces(m) ? 2 : 0;
         if (faces) {
-            optional_buffer(m, &m->d_adj, 6 * state + 2 * face, PENDING_ADJOINT);
+            optional_buffer(m, &m->d_adj, 6 * state + 2 * face, pending_adjoint(m));
             if (!m->d_adj) faces = f64 ? 1 : 0;
         }
         if (!m->d_adj) DG_CUDA(cudaMalloc(&m->d_adj, 6 * state + faces * face));

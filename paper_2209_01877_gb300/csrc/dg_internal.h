@@ -94,9 +94,11 @@ struct dg_mesh {
     double* d_red = nullptr;       // reduction scratch
     double* h_red = nullptr;       // pinned host reduction result
     unsigned int* d_status = nullptr;
-    double* d_Z = nullptr;         // Navier-Stokes auxiliary gradient [ne][3][5][Nb] (lazy)
-    double* d_HB = nullptr;        // Navier-Stokes own viscous face fluxes [ne][4][4][Nqf] (lazy)
-    void* d_TN = nullptr;          // Navier-Stokes traces of U [ne][4][5][Nqf] (lazy)
+    // Navier-Stokes, one allocation (lazy): auxiliary gradient [ne][3][5][Nb], own viscous face fluxes
+    // [ne][4][4][Nqf] and, in FP32 where there is room, traces of U [ne][4][5][Nqf] (FP64: d_T)
+    double* d_Z = nullptr;
+    double* d_HB = nullptr;
+    void* d_TN = nullptr;
     // mixed precision, conservative mode-0 update (dg_set_conservative): per (element, face) flux
     // integrals [ne][4][5]; per slot the weight phi_0 2|S_f| / |det J| of the mode-0 pass and the
     // face's 2|S_f| (one value per face, in both slots)
@@ -116,7 +118,6 @@ struct dg_mesh {
     int64_t n_flist = 0, n_interior = 0, n_trace = 0;   // listed faces, interior ones among them
     void* d_T = nullptr;
     void *d_TA = nullptr, *d_TL = nullptr;
-    bool ns_set = false;           // the optional buffer of the viscous passes has been asked for
     size_t face_bytes() const;
     // small meshes: a CUDA graph of several captured RK3 steps at one dt (dg_rk3_step)
     cudaStream_t cap_stream = nullptr;
