@@ -138,17 +138,16 @@ void optional_buffer(const dg_mesh* m, void** buf, size_t bytes, size_t covered 
 
 // ---- which meshes evaluate every face once: FP64 all; FP32 by size -----------------------------------
 
-// From how many elements on an FP32 stage of three launches is faster than the single kernel.  us per step, single
-// against three launches:
-//   P1, where the tiles of the single kernel make one wave up to 19,456 elements: Rusanov 16,464 38 : 50, 24,576
-//       50 : 50, 34,992 57 : 67, 48,000 75 : 78, 55,566 81 : 81, 82,944 112 : 107 (so from three waves on);
-//       Roe 16,464 38 : 50, 20,250 52 : 50, 34,992 62 : 65, 48,000 81 : 76 (from one wave on);
-//   P2: 8,712 58 : 55 (Rusanov), 62 : 55 (Roe), 12,168 77 : 57, 93,750 420 : 181;
-//   P3: 8,712 137 : 69, 93,750 1,150 : 353.
-int64_t fp32_faces_min_ne(const dg_mesh* m) {
-    if (m->p > 1) return 8192;
-    return m->flux == DG_ROE ? 19456 : 3 * 19456;
-}
+// From how many elements on an FP32 mesh takes the three launches of a stage in place of the single kernel.  us per step,
+// single : three launches, launched one by one | replayed from the graph of dg_rk3_step (up to 65,536 elements):
+//   P1, where the tiles of the single kernel make one wave up to 19,456 elements: Rusanov 12,168 33 : 51 | 27 : 25,
+//       20,250 50 : 50 | 42 : 32, 29,478 56 : 56 | 47 : 39, 34,992 57 : 67 | 51 : 46, 48,000 75 : 78 | 67 : 55, 82,944
+//       112 : 107; Roe 12,168 38 : 51 | 28 : 25, 20,250 52 : 50 | 44 : 32, 34,992 62 : 65 | 54 : 45, 48,000 81 : 76 | 71 :
+//       54.  Below one wave the single kernel's lead when launched (18 us) outweighs the other's in the graph (3 us); above
+//       it the graph's gain (6 to 16 us) outweighs what is lost when launched (10 us at one size, else at most 3);
+//   P2: 8,712 58 : 55 (Rusanov), 62 : 55 (Roe), 10,368 69 : 57 | 61 : 34, 93,750 420 : 181;
+//   P3: 8,712 137 : 69, 10,368 149 : 75 | 140 : 55, 93,750 1,150 : 353.
+int64_t fp32_faces_min_ne(const dg_mesh* m) { return m->p > 1 ? 8192 : 19456; }
 
 // Whether the FP32 stages of the Euler steps do.  On a mesh with boundary faces the single kernel is kept:
 // dg_boundary_flux reports the boundary integral of the FP32 state in FP64, which shows the order of
@@ -710,7 +709,13 @@ dg_status dg_ns_rk3_step(dg_mesh* m, double dt, int nsteps, double mu, double pr
     // the stages of dg_rk_stage, each as residual (Euler + viscous lines) then update
     const struct { int in, base, out; double a, b; } stages[3] = {{0, -1, 1, 0.0, 1.0}, {1, 0, 2, 0.75, 0.25},
                                                                   {2, 0, 0, 1.0 / 3.0, 2.0 / 3.0}};
-    void* T = inner_faces(m, mu > 0.0 ? m->d_TN : m->d_T);   // the viscous passes' buffer: the Euler pass is done with it
+    // the viscous passes' trace buffer (the Euler pass is done with it when they begin), or the Euler stages', which
+    // a mesh with boundary faces has for this call alone
+    if (mu == 0.0 && m->face_once && !m->d_T && !m->faces_asked && inner_faces(m, m)) {
+        optional_buffer(m, &m->d_T, m->face_bytes());
+        m->faces_asked = true;
+    }
+    void* T = inner_faces(m, mu > 0.0 ? m->d_TN : m->d_T);
     for (int k = 0; k < nsteps; ++k)
         for (const auto& g : stages) {
             DG_CUDA(euler_residual_internal(m, B[g.in], R, T, s));

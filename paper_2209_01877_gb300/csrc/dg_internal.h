@@ -118,6 +118,7 @@ struct dg_mesh {
     int64_t n_flist = 0, n_interior = 0, n_trace = 0;   // listed faces, interior ones among them
     void* d_T = nullptr;
     void *d_TA = nullptr, *d_TL = nullptr;
+    bool faces_asked = false;      // d_T has been asked for after the creation
     size_t face_bytes() const;
     // small meshes: a CUDA graph of several captured RK3 steps at one dt (dg_rk3_step)
     cudaStream_t cap_stream = nullptr;
