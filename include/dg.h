@@ -188,8 +188,9 @@ dg_status dg_ns_residual(dg_mesh* mesh, const double* U, double* R, double mu, d
  * dg_residual call between steps is safe. */
 dg_status dg_ns_rk3_step(dg_mesh* mesh, double dt, int nsteps, double mu, double prandtl, void* stream);
 
-/* One SSP-RK3 stage on the internal state, fused with the residual (one
- * kernel launch): stage 1 U1 = U0 + dt R(U0); stage 2 U2 = 3/4 U0 + 1/4 (U1
+/* One SSP-RK3 stage on the internal state, fused with the residual (the mixed
+ * forms and FP32 meshes that are small or have boundary faces: one kernel
+ * launch; FP64 and larger FP32 meshes: three, every face evaluated once): stage 1 U1 = U0 + dt R(U0); stage 2 U2 = 3/4 U0 + 1/4 (U1
  * + dt R(U1)); stage 3 U0 <- 1/3 U0 + 2/3 (U2 + dt R(U2)). */
 dg_status dg_rk_stage(dg_mesh* mesh, int stage, double dt, void* stream);
 

@@ -22,10 +22,10 @@
 //     b dt R is formed in FP32 -- it is small against U, so its rounding sits
 //     far below the FP32 residual's own.
 //
-// One persistent CTA per SM (512 threads, 512 TMEM columns) runs two
-// independent pipelines ("contexts" of 256 threads, 256 TMEM columns and their
-// own shared-memory buffers; the basis tables are shared).  While one context
-// waits on the tensor cores or on memory, the other computes.  A context walks
+// One persistent CTA per SM runs two (P3) or three (P1, P2) independent pipelines
+// ("contexts" of 256 threads, 64 / 160 / 256 TMEM columns at P1 / P2 / P3 and
+// their own shared-memory buffers; the basis tables are shared).  While one context
+// waits on the tensor cores or on memory, the others compute.  A context walks
 // over tiles of ET = 12 consecutive elements (5 ET = 60 rows of a 64-row MMA;
 // an M = 64 accumulator occupies TMEM lanes 0-15 of each 32-lane quarter).  A
 // face whose two elements lie in the same tile is evaluated once (by the
@@ -55,7 +55,7 @@
 //            the wait for MMA 2), so each warp goes on to the next tile.
 // Every wait on the tensor cores is bounded; on time-out the context sets a
 // status bit and leaves its tile loop (all its threads together); the CTA
-// frees its tensor memory when both contexts are done.
+// frees its tensor memory when all contexts are done.
 #include <algorithm>
 #include <cstring>
 

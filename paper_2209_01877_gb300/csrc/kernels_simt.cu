@@ -1,5 +1,7 @@
-// Residual and SSP-RK3 stage on the CUDA cores (FP64 and FP32), with every face's traces and
-// numerical flux evaluated once.  Three launches per residual or stage:
+// Residual and SSP-RK3 stage on the CUDA cores: FP64, and the FP32 stages of larger meshes, with every
+// face's traces and numerical flux evaluated once (FP32 residual calls, the stages of smaller
+// meshes and of meshes with boundary faces: the single kernel k_residual below; capi.cpp has
+// the rules).  Three launches per residual or stage:
 //   k_traces  thread per (element, variable): the element's own trace at the points of its 4 faces,
 //             to a face buffer T[e][f][v][q];
 //   k_faces   thread per (listed face, point): the flux in the owner's orientation,
@@ -20,7 +22,7 @@
 // Measured, one SSP-RK3 step between set and get of the state, dense operators and one thread per
 // point before -> factored operators: FP64 P3 Roe, 196,608 elements 27.7 -> 17.1 ms; FP64 P1 Rusanov,
 // 1,296 elements 85 -> 62 us; FP32 P2 Rusanov, 663,552 elements, per stage 980 us (one kernel, each face
-// from both sides) -> 65 + 151 + 126 us.
+// from both sides) -> 65 + 153 + 147 us.
 #include <algorithm>
 #include <type_traits>
 
@@ -38,9 +40,10 @@ constexpr int NT = 256;
 
 // ---- FP32 without a face buffer ------------------------------------------------------------------
 // One persistent kernel per residual that evaluates every face from both sides: the calls that return
-// an FP32 residual (their values stay those of this order of summation), and RK stages where the face
-// buffer (80 Nqf bytes per element) cannot be allocated (a P2 stage takes two and a half times the
-// time of the face-once form below).
+// an FP32 residual (their values stay those of this order of summation), the RK stages of meshes on which
+// it is the faster form, of meshes with boundary faces, and of meshes without room for the face
+// buffer (80 Nqf bytes per element; on large meshes a P2 stage takes two and a half times the time of
+// the face-once form below).
 
 template <int P> struct Tile;
 template <> struct Tile<1> { static constexpr int EPB = 32; };
