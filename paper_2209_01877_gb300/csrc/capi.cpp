@@ -154,22 +154,6 @@ int64_t fp32_faces_min_ne(const dg_mesh* m) { return m->p > 1 ? 8192 : 19456; }
 // summation at 1e-7, the rounding of the state itself.
 bool fp32_stage_faces(const dg_mesh* m) { return m->host.ne >= fp32_faces_min_ne(m) && !m->has_bc; }
 
-// Whether the adjoint evaluates every face once (three launches, a fourth for boundary faces).  In FP32
-// the single kernel k_residual_vjp, whose tiles hold 16, 8, 4 elements, is faster while they are no
-// more than the SMs.  us per VJP, single against three launches, Rusanov | Roe | Rusanov with boundary
-// faces: P1 2,058 elements 23 : 25 | 23 : 25 | 23 : 32, 3,072 27 : 25 | 32 : 25 | 31 : 32; P2 750
-// 23 : 27 | 25 : 27 | 25 : 34, 1,296 30 : 27 | 34 : 28 | 34 : 34; P3 384 28 : 32 | 30 : 32 | 30 : 38,
-// 750 34 : 32 | 38 : 32 | 38 : 38.  With Rusanov and boundary faces the single kernel is ahead up to two
-// tiles per SM (P1 4,374 32 : 34, P2 2,058 34 : 35).
-bool vjp_by_faces(const dg_mesh* m) {
-    if (m->precision == DG_FP64) return true;
-    const int64_t wave = 152 * (m->p == 1 ? 16 : m->p == 2 ? 8 : 4);
-    return m->host.ne > (m->flux == DG_RUSANOV && m->has_bc ? 2 : 1) * wave;
-}
-
-// whether any call on an FP32 mesh uses the face list
-bool faces_in_use(const dg_mesh* m) { return vjp_by_faces(m) || m->host.ne >= fp32_faces_min_ne(m); }
-
 }  // namespace
 
 namespace dg {
@@ -298,9 +282,8 @@ dg_status dg_mesh_create(const int32_t* tet_vid, const double* tet_xyz, const in
         if (e == cudaSuccess) e = cudaMallocHost(&m->h_red, 16 * sizeof(double));
         // FP32: the face list and, where the Euler stages use it, the face buffer; last, and only with room
         // to spare: without them the mesh runs the kernels that need none
-        if (e == cudaSuccess && m->precision == DG_FP32 && faces_in_use(m) &&
-            room_for(m, dg::face_list_bytes(m->host.n_faces, DG_FP32, vjp_by_faces(m)))) {
-            e = dg::setup_face_once(m, m, 0, ne, vjp_by_faces(m), s);
+        if (e == cudaSuccess && m->precision == DG_FP32 && room_for(m, dg::face_list_bytes(m->host.n_faces, DG_FP32, true))) {
+            e = dg::setup_face_once(m, m, 0, ne, true, s);
             if (e == cudaErrorMemoryAllocation) e = (cudaGetLastError(), cudaSuccess);
         }
         if (e == cudaSuccess && m->face_once && m->precision == DG_FP32 && fp32_stage_faces(m))
@@ -808,7 +791,7 @@ dg_status ensure_adjoint_buffers(dg_mesh* m) {
         const bool f64 = m->precision == DG_FP64;
         // both face buffers, or what the call cannot do without: FP64 the direction's, FP32 none (the single
         // kernel)
-        int faces = m->face_once && vjp_by_faces(m) ? 2 : 0;
+        int faces = m->face_once ? 2 : 0;
         if (faces) {
             optional_buffer(m, &m->d_adj, 6 * state + 2 * face, pending_adjoint(m));
             if (!m->d_adj) faces = f64 ? 1 : 0;
@@ -842,8 +825,7 @@ dg_status dg_residual_vjp(dg_mesh* m, const double* U, const double* lambda, dou
     if (st != DG_OK) return st;
     void** V = m->d_V;
     const double c[4] = {0.0, 0.0, 0.0, 1.0};
-    DG_CUDA(dg::launch_gather(m, U, V[0], s));
-    DG_CUDA(dg::launch_gather(m, lambda, V[1], s));
+    DG_CUDA(dg::launch_gather2(m, U, V[0], lambda, V[1], s));
     DG_CUDA(dg::launch_residual_vjp(m, V[0], V[1], nullptr, nullptr, nullptr, c, V[2], s));
     DG_CUDA(dg::launch_scatter(m, V[2], out, s));
     return leave_adjoint(m, s);
@@ -857,8 +839,7 @@ dg_status dg_rk3_step_vjp(dg_mesh* m, const double* U0, double dt, const double*
     dg_status st = ensure_adjoint_buffers(m);
     if (st != DG_OK) return st;
     void** V = m->d_V;   // V0 = U0, V1 = lambda, V2 = U1, V3 = U2 (then result), V4 = m2, V5 = m1
-    DG_CUDA(dg::launch_gather(m, U0, V[0], s));
-    DG_CUDA(dg::launch_gather(m, lambda, V[1], s));
+    DG_CUDA(dg::launch_gather2(m, U0, V[0], lambda, V[1], s));
     DG_CUDA(dg::launch_residual(m, V[0], nullptr, V[2], 1, dt, 0.0, 1.0, inner_faces(m, m->d_TA), s));
     DG_CUDA(dg::launch_residual(m, V[2], V[0], V[3], 1, dt, 0.75, 0.25, inner_faces(m, m->d_TA), s));
     const double c2[4] = {2.0 / 3.0, 0.0, 0.0, 2.0 / 3.0 * dt};   // m2 = 2/3 (lambda + dt J(U2)^T lambda)

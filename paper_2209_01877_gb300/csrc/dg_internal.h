@@ -141,6 +141,8 @@ size_t face_list_bytes(int64_t n, int precision, bool scales);
 // face traces of two states of the mesh's precision (U1 may be null), into the face buffers T and T1
 cudaError_t launch_traces2(dg_mesh* m, const void* U, void* T, const void* U1, void* T1, cudaStream_t s);
 cudaError_t launch_gather(dg_mesh* m, const double* user, void* internal, cudaStream_t s);   // caller -> internal
+cudaError_t launch_gather2(dg_mesh* m, const double* user, void* internal, const double* user1, void* internal1,
+                           cudaStream_t s);   // two at once
 cudaError_t launch_gather_f32(dg_mesh* m, const double* user, float* internal, cudaStream_t s);   // FP32 (a hi plane) only
 // Navier-Stokes lines: the BR1 gradient into Z, then the viscous volume and face terms added to
 // the residual R (internal order), in the mesh's arithmetic (FP64 meshes FP64; FP32 and mixed

@@ -40,9 +40,12 @@ __device__ __forceinline__ void store2(double* p, double2 x) {
 }
 
 template <int NV, int FMT, bool VEC, int ME>
-__global__ void __launch_bounds__(MT2) k_gather(const double* __restrict__ user, void* __restrict__ internal,
+__global__ void __launch_bounds__(MT2) k_gather(const double* __restrict__ user0, void* __restrict__ internal0,
+                                                const double* __restrict__ user1, void* __restrict__ internal1,
                                                 const int32_t* __restrict__ perm, int64_t ne) {
     constexpr int H = NV / 2;
+    const double* __restrict__ user = blockIdx.y == 0 ? user0 : user1;   // one or (gridDim.y = 2) two arrays
+    void* __restrict__ internal = blockIdx.y == 0 ? internal0 : internal1;
     const int64_t e0 = blockIdx.x * (int64_t)ME;
     const int n = (ne - e0 < ME ? (int)(ne - e0) : ME) * H;
     __shared__ int32_t sp[ME];
@@ -100,35 +103,42 @@ __global__ void __launch_bounds__(MT2) k_scatter(const void* __restrict__ intern
     }
 }
 
+// user -> internal (gather; user1, internal1: a second pair, or null) or internal -> user
+struct Move {
+    bool gather;
+    const void *from, *from1;
+    void *to, *to1;
+};
+
 template <int NV, int FMT, int ME>
-void move_elements(bool gather, const void* from, void* to, const int32_t* perm, int64_t ne, cudaStream_t s) {
+void move_elements(const Move& v, const int32_t* perm, int64_t ne, cudaStream_t s) {
     const unsigned grid = (unsigned)((ne + ME - 1) / ME);
-    const void* user = gather ? from : to;
-    const bool vec = (reinterpret_cast<uintptr_t>(user) & 15) == 0;
-    if (gather) {
-        const double* u = static_cast<const double*>(from);
-        if (vec) k_gather<NV, FMT, true, ME><<<grid, MT2, 0, s>>>(u, to, perm, ne);
-        else k_gather<NV, FMT, false, ME><<<grid, MT2, 0, s>>>(u, to, perm, ne);
+    auto at16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    if (v.gather) {
+        const double *u = static_cast<const double*>(v.from), *u1 = static_cast<const double*>(v.from1);
+        const dim3 g(grid, u1 ? 2 : 1);
+        if (at16(u) && at16(u1)) k_gather<NV, FMT, true, ME><<<g, MT2, 0, s>>>(u, v.to, u1, v.to1, perm, ne);
+        else k_gather<NV, FMT, false, ME><<<g, MT2, 0, s>>>(u, v.to, u1, v.to1, perm, ne);
     } else {
-        double* u = static_cast<double*>(to);
-        if (vec) k_scatter<NV, FMT, true, ME><<<grid, MT2, 0, s>>>(from, u, perm, ne);
-        else k_scatter<NV, FMT, false, ME><<<grid, MT2, 0, s>>>(from, u, perm, ne);
+        double* u = static_cast<double*>(v.to);
+        if (at16(u)) k_scatter<NV, FMT, true, ME><<<grid, MT2, 0, s>>>(v.from, u, perm, ne);
+        else k_scatter<NV, FMT, false, ME><<<grid, MT2, 0, s>>>(v.from, u, perm, ne);
     }
 }
 
 template <int NV, int FMT>
-void move_elements(bool gather, const void* from, void* to, const int32_t* perm, int64_t ne, cudaStream_t s) {
-    if (small_tiles(ne)) move_elements<NV, FMT, 8>(gather, from, to, perm, ne, s);
-    else move_elements<NV, FMT, 32>(gather, from, to, perm, ne, s);
+void move_elements(const Move& v, const int32_t* perm, int64_t ne, cudaStream_t s) {
+    if (small_tiles(ne)) move_elements<NV, FMT, 8>(v, perm, ne, s);
+    else move_elements<NV, FMT, 32>(v, perm, ne, s);
 }
 
-cudaError_t move_state(const dg_mesh* m, bool gather, int fmt, const void* from, void* to, cudaStream_t s) {
+cudaError_t move_state(const dg_mesh* m, int fmt, const Move& v, cudaStream_t s) {
     const int64_t ne = m->host.ne;
     auto go = [&](auto nv) {
         constexpr int NV = decltype(nv)::value;
-        if (fmt == MOVE_F64) move_elements<NV, MOVE_F64>(gather, from, to, m->d_perm, ne, s);
-        else if (fmt == MOVE_F32) move_elements<NV, MOVE_F32>(gather, from, to, m->d_perm, ne, s);
-        else move_elements<NV, MOVE_FF>(gather, from, to, m->d_perm, ne, s);
+        if (fmt == MOVE_F64) move_elements<NV, MOVE_F64>(v, m->d_perm, ne, s);
+        else if (fmt == MOVE_F32) move_elements<NV, MOVE_F32>(v, m->d_perm, ne, s);
+        else move_elements<NV, MOVE_FF>(v, m->d_perm, ne, s);
     };
     if (m->p == 1) go(std::integral_constant<int, 20>());
     else if (m->p == 2) go(std::integral_constant<int, 50>());
@@ -410,19 +420,23 @@ int grid_for(int64_t n, int block) {
 }  // namespace
 
 cudaError_t launch_gather(dg_mesh* m, const double* user, void* internal, cudaStream_t s) {
-    return move_state(m, true, format_of(m), user, internal, s);
+    return move_state(m, format_of(m), {true, user, nullptr, internal, nullptr}, s);
+}
+
+cudaError_t launch_gather2(dg_mesh* m, const double* user, void* internal, const double* user1, void* internal1, cudaStream_t s) {
+    return move_state(m, format_of(m), {true, user, user1, internal, internal1}, s);
 }
 
 cudaError_t launch_gather_f32(dg_mesh* m, const double* user, float* internal, cudaStream_t s) {
-    return move_state(m, true, MOVE_F32, user, internal, s);
+    return move_state(m, MOVE_F32, {true, user, nullptr, internal, nullptr}, s);
 }
 
 cudaError_t launch_scatter(dg_mesh* m, const void* internal, double* user, cudaStream_t s) {
-    return move_state(m, false, format_of(m), internal, user, s);
+    return move_state(m, format_of(m), {false, internal, nullptr, user, nullptr}, s);
 }
 
 cudaError_t launch_scatter_f32(dg_mesh* m, const float* internal, double* user, cudaStream_t s) {
-    return move_state(m, false, MOVE_F32, internal, user, s);
+    return move_state(m, MOVE_F32, {false, internal, nullptr, user, nullptr}, s);
 }
 
 int reduction_blocks(int64_t ne) { return (int)std::max<int64_t>(1, std::min<int64_t>((ne + RT - 1) / RT, 1024)); }

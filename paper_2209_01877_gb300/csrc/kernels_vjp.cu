@@ -8,7 +8,8 @@
 //                  s' lambda_other - s lambda_owner (wf is applied by the lift below); one reverse
 //                  sweep gives both states' adjoints, written over the traces of U.  At a kink, where
 //                  the two residuals take different branches, a sweep for each;
-//   k_bfaces_vjp   the same on boundary faces, through the ghost state (dual numbers: few faces);
+//   k_bfaces_vjp   the same on boundary faces, through the ghost state (dual numbers: few faces); on small FP32
+//                  meshes both in one launch, k_allfaces_vjp;
 //   k_element_vjp  tiles of 32 elements, thread per (element, variable) row: U and the three
 //                  derivatives of lambda at the volume points; thread per (element, point): the
 //                  reverse of the contravariant Euler flux; rows again: the transposed interpolation,
@@ -32,8 +33,7 @@ namespace {
 constexpr int NT = 256;
 
 // ---- FP32 without face buffers: each element differentiates its faces from both sides in forward
-// mode; the faster form on small meshes (capi.cpp has the rule), and the one that is left where the
-// face buffers cannot be allocated
+// mode; used only where there is no room for the face buffers
 
 template <int P> struct VTile;
 template <> struct VTile<1> { static constexpr int EPB = 16; };
@@ -351,10 +351,10 @@ struct FaceVjpArgs {
     Real finf[5];
 };
 
+// the i-th (interior face, point)
 template <typename Real, int P, int FLUX>
-__global__ void __launch_bounds__(VF) k_faces_vjp(FaceVjpArgs<Real> a) {
+__device__ __forceinline__ void face_vjp(const FaceVjpArgs<Real>& a, int64_t i) {
     constexpr int NQF = nqf_of(P);
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     const int64_t li = i / NQF;
     const int q = (int)(i - li * NQF);
@@ -388,11 +388,11 @@ __global__ void __launch_bounds__(VF) k_faces_vjp(FaceVjpArgs<Real> a) {
     }
 }
 
+// the i-th (boundary face, point)
 template <typename Real, int P, int FLUX>
-__global__ void __launch_bounds__(VF) k_bfaces_vjp(FaceVjpArgs<Real> a) {
+__device__ __forceinline__ void bface_vjp(const FaceVjpArgs<Real>& a, int64_t i) {
     using D5 = Dual<Real, 5>;
     constexpr int NQF = nqf_of(P);
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     const int64_t li = i / NQF;
     const int q = (int)(i - li * NQF);
@@ -421,6 +421,25 @@ __global__ void __launch_bounds__(VF) k_bfaces_vjp(FaceVjpArgs<Real> a) {
     }
 #pragma unroll
     for (int v = 0; v < 5; ++v) a.T[oe + v * NQF] = ub[v];
+}
+
+template <typename Real, int P, int FLUX>
+__global__ void __launch_bounds__(VF) k_faces_vjp(FaceVjpArgs<Real> a) {
+    face_vjp<Real, P, FLUX>(a, blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+}
+template <typename Real, int P, int FLUX>
+__global__ void __launch_bounds__(VF) k_bfaces_vjp(FaceVjpArgs<Real> a) {
+    bface_vjp<Real, P, FLUX>(a, blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+}
+
+// Both in one launch of one-warp blocks, side by side: on a small mesh the boundary faces' long chain (dual
+// numbers) and its launch were a quarter of a VJP (FP32 P2 Rusanov with boundary faces, 750 elements, with the
+// two gathers in one launch 33.8 -> 25.4 us; the single kernel 25.5).  The registers of the longer part allow 10 warps an SM, so larger meshes keep two launches.
+constexpr int64_t BOTH_MAX_WARPS = 8 * 152;
+template <typename Real, int P, int FLUX>
+__global__ void __launch_bounds__(32) k_allfaces_vjp(FaceVjpArgs<Real> a, FaceVjpArgs<Real> b, unsigned interior) {
+    if (blockIdx.x < interior) face_vjp<Real, P, FLUX>(a, blockIdx.x * (int64_t)32 + threadIdx.x);
+    else bface_vjp<Real, P, FLUX>(b, (blockIdx.x - interior) * (int64_t)32 + threadIdx.x);
 }
 
 template <typename Real, int P, int EE>
@@ -573,16 +592,21 @@ cudaError_t vlaunch_faces(dg_mesh* m, const VjpArgs<Real>& r, cudaStream_t s) {
     f.gamma = r.gamma;
     f.roe_eps = r.roe_eps;
     for (int v = 0; v < 5; ++v) f.finf[v] = r.finf[v];
-    unsigned nt = vface_block(f.n);
-    if (f.n > 0) k_faces_vjp<Real, P, FLUX><<<(unsigned)((f.n + nt - 1) / nt), nt, 0, s>>>(f);
-    const int64_t nb = m->n_flist - m->n_interior;
-    if (nb > 0) {
-        f.rec += m->n_interior;
-        f.normal += 3 * m->n_interior;
-        f.scale += 2 * m->n_interior;
-        f.n = nb * NQF;
-        nt = vface_block(f.n);
-        k_bfaces_vjp<Real, P, FLUX><<<(unsigned)((f.n + nt - 1) / nt), nt, 0, s>>>(f);
+    FaceVjpArgs<Real> b = f;   // the boundary faces
+    b.rec += m->n_interior;
+    b.normal += 3 * m->n_interior;
+    b.scale += 2 * m->n_interior;
+    b.n = (m->n_flist - m->n_interior) * NQF;
+    const int64_t wi = (f.n + 31) / 32, wb = (b.n + 31) / 32;
+    bool both = false;
+    if constexpr (sizeof(Real) == 4) both = wi > 0 && wb > 0 && wi + wb <= BOTH_MAX_WARPS;
+    if (both) {
+        if constexpr (sizeof(Real) == 4) k_allfaces_vjp<Real, P, FLUX><<<(unsigned)(wi + wb), 32, 0, s>>>(f, b, (unsigned)wi);
+    } else {
+        unsigned nt = vface_block(f.n);
+        if (f.n > 0) k_faces_vjp<Real, P, FLUX><<<(unsigned)((f.n + nt - 1) / nt), nt, 0, s>>>(f);
+        nt = vface_block(b.n);
+        if (b.n > 0) k_bfaces_vjp<Real, P, FLUX><<<(unsigned)((b.n + nt - 1) / nt), nt, 0, s>>>(b);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
