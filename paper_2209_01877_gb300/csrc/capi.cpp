@@ -474,14 +474,6 @@ cudaError_t euler_residual_internal(dg_mesh* m, const void* in, void* R, void* T
     return dg::launch_residual(m, in, nullptr, R, 0, 0.0, 0.0, 0.0, T, s);
 }
 
-// Whether the viscous passes take the traces of U (kernels_ns.cu); without them a mesh in FP32 arithmetic
-// runs the passes of the mixed forms, three launches instead of four, which are faster on small P1
-// meshes: us per residual, 1,296 elements 40 : 42, 4,374 with boundary faces 40 : 44, 6,000 44 : 44 and
-// equal or slower from there on; at P2 and P3 equal or slower at every size.
-bool ns_by_rows(const dg_mesh* m) {
-    return m->precision == DG_FP64 || (m->precision == DG_FP32 && (m->p > 1 || m->host.ne >= 6000));
-}
-
 // One allocation: the gradient, the face fluxes and, in FP32 with room to spare, the traces of U (FP64 has the
 // steps' face buffer for them: the Euler residual is done with it).
 dg_status ensure_ns_buffers(dg_mesh* m) {
@@ -489,7 +481,7 @@ dg_status ensure_ns_buffers(dg_mesh* m) {
     const size_t rs = m->precision == DG_FP64 ? sizeof(double) : sizeof(float), ne = m->host.ne;
     const size_t z = ne * 15 * m->nb * rs, hb = dg::ns_face_buffer_values(m->p, ne) * rs, tn = ne * 20 * m->nqf * rs;
     bool traces = false;
-    if (m->precision == DG_FP32 && ns_by_rows(m)) {
+    if (m->precision == DG_FP32) {
         optional_buffer(m, reinterpret_cast<void**>(&m->d_Z), whole(z) + whole(hb) + tn, pending_ns(m));
         traces = m->d_Z != nullptr;
     }

@@ -66,7 +66,9 @@ __device__ __forceinline__ void scaled_normal(const Real* I, int f, Real* g) {
     for (int d = 0; d < 3; ++d) g[d] = f == 0 ? I[d] + I[3 + d] + I[6 + d] : -I[3 * (f - 1) + d];
 }
 
-template <typename Real, int P, int EE>
+// TR: the traces come from the buffer T; without it (small P1 meshes) each row evaluates its own and its
+// neighbours', 55 multiply-adds a face at most, and the launch that fills the buffer is saved
+template <typename Real, int P, int EE, bool TR>
 __global__ void __launch_bounds__(threads_of(EE)) k_ns_grad(NSArgs<Real> a) {
     constexpr int NB = nb_of(P), NQF = nqf_of(P), NM = modal::Tables<P>::NM, NF = modal::Tables<P>::NF, NT = threads_of(EE);
     __shared__ Real sJ[EE * 9];
@@ -86,14 +88,13 @@ __global__ void __launch_bounds__(threads_of(EE)) k_ns_grad(NSArgs<Real> a) {
     if (t >= 5 * nel) return;
     const int e = t / 5, v = t - 5 * e;
     const Real* I = sJ + 9 * e;
-    Real z[3][NB];
+    Real z[3][NB], c[NB];
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
         for (int j = 0; j < NB; ++j) z[d][j] = 0;
+    load_row<NB>(a.U + (e0 * 5 + t) * NB, c);
     {
-        Real c[NB];
-        load_row<NB>(a.U + (e0 * 5 + t) * NB, c);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             Real s[NM];
@@ -104,21 +105,45 @@ __global__ void __launch_bounds__(threads_of(EE)) k_ns_grad(NSArgs<Real> a) {
                 for (int m = 0; m < NM; ++m) z[d][m] += I[3 * k + d] * s[m];
         }
     }
-    const Real* own = a.T + (e0 + e) * 20 * NQF;
+    const Real* own = TR ? a.T + (e0 + e) * 20 * NQF : nullptr;
     modal::unroll<0, 4>([&](auto fc) {
         constexpr int f = fc.value;
         // Qhat - Q- at the face's points
         const int n = snbr[4 * e + f];
         Real x[NQF], b[NF], y[NB], g[3];
-        load_row<NQF>(own + (f * 5 + v) * NQF, x);
+        if constexpr (TR) load_row<NQF>(own + (f * 5 + v) * NQF, x);
+        else modal::face_trace<Real, P, f>(c, x);
         if (n >= 0) {
             const int code = sfc[4 * e + f];
-            const Real* o = a.T + (((int64_t)n * 4 + (code & 3)) * 5 + v) * NQF;
             const int8_t* pm = sperm + (code >> 2) * NQF;
+            Real u[TR ? 1 : NQF];
+            const Real* o;
+            if constexpr (TR) {
+                o = a.T + (((int64_t)n * 4 + (code & 3)) * 5 + v) * NQF;
+            } else {
+                Real cn[NB];
+                load_row<NB>(a.U + ((int64_t)n * 5 + v) * NB, cn);
+                modal::face_trace<Real, P>(code & 3, cn, u);
+                o = u;
+            }
 #pragma unroll
             for (int q = 0; q < NQF; ++q) x[q] = Real(0.5) * (o[pm[q]] - x[q]);
         } else if (n == -1 - DG_BC_WALL) {
-            const Real* w = own + f * 5 * NQF;
+            Real wt[TR ? 1 : 4 * NQF];
+            const Real* w;
+            if constexpr (TR) {
+                w = own + f * 5 * NQF;
+            } else {
+                if (v == 4)   // density and momenta of the element
+                    for (int k = 0; k < 4; ++k) {
+                        Real ck[NB];
+                        load_row<NB>(a.U + ((e0 + e) * 5 + k) * NB, ck);
+                        modal::face_trace<Real, P, f>(ck, wt + k * NQF);
+                    }
+                else
+                    for (int k = 0; k < 4 * NQF; ++k) wt[k] = Real(1);   // unused
+                w = wt;
+            }
 #pragma unroll
             for (int q = 0; q < NQF; ++q) {
                 const Real m0 = w[NQF + q], m1 = w[2 * NQF + q], m2 = w[3 * NQF + q];
@@ -206,7 +231,7 @@ struct ViscPlan {
     static constexpr size_t BYTES = REALS * sizeof(Real);
 };
 
-template <typename Real, int P>
+template <typename Real, int P, bool TR>
 __global__ void __launch_bounds__(VT) k_ns_visc(NSArgs<Real> a) {
     using S = ViscPlan<Real, P>;
     constexpr int NB = nb_of(P), NQ = nq_of(P), NQF = nqf_of(P), NPF = S::NPF, NM = modal::Tables<P>::NM;
@@ -227,7 +252,13 @@ __global__ void __launch_bounds__(VT) k_ns_visc(NSArgs<Real> a) {
     Real c[NB];
     if (live) {
         Real* o = sP + t * S::SF;
-        if (r < 5) {
+        if (!TR) {
+            load_row<NB>(r < 5 ? a.U + ((e0 + e) * 5 + r) * NB : a.Z + ((e0 + e) * 15 + r - 5) * NB, c);
+            modal::traces<Real, P>(c, [&](int f, const Real* u) {
+#pragma unroll
+                for (int q = 0; q < NQF; ++q) o[f * NQF + q] = u[q];
+            });
+        } else if (r < 5) {
             load_row<NB>(a.U + ((e0 + e) * 5 + r) * NB, c);
 #pragma unroll
             for (int f = 0; f < 4; ++f) {
@@ -362,10 +393,10 @@ __global__ void __launch_bounds__(4 * EL) k_ns_lift(NSArgs<Real> a) {
     store_row<NB>(R, x);
 }
 
-template <typename Real, int P>
+template <typename Real, int P, bool TR>
 cudaError_t ns_launch(const NSArgs<Real>& a, cudaStream_t s) {
     constexpr size_t bytes = ViscPlan<Real, P>::BYTES;
-    auto visc = k_ns_visc<Real, P>;
+    auto visc = k_ns_visc<Real, P, TR>;
     static bool init = false;
     if (!init) {
         cudaError_t e = cudaFuncSetAttribute(visc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -373,7 +404,7 @@ cudaError_t ns_launch(const NSArgs<Real>& a, cudaStream_t s) {
         init = true;
     }
     // one warp per tile: a row holds three gradients' modes in registers
-    k_ns_grad<Real, P, 6><<<(unsigned)((a.ne + 5) / 6), threads_of(6), 0, s>>>(a);
+    k_ns_grad<Real, P, 6, TR><<<(unsigned)((a.ne + 5) / 6), threads_of(6), 0, s>>>(a);
     visc<<<(unsigned)((a.ne + EV - 1) / EV), VT, bytes, s>>>(a);
     if (small_tiles(a.ne)) k_ns_lift<Real, P, 8><<<(unsigned)((a.ne + 7) / 8), 32, 0, s>>>(a);
     else k_ns_lift<Real, P, 32><<<(unsigned)((a.ne + 31) / 32), 128, 0, s>>>(a);
@@ -418,7 +449,10 @@ __global__ void __launch_bounds__(256) k_rk_axpy_ff(const float* __restrict__ U,
 template <typename Real>
 cudaError_t ns_dispatch(dg_mesh* m, const void* U, void* T, void* Z, void* HB, void* R, double mu, double prandtl,
                         cudaStream_t s) {
-    cudaError_t e = launch_traces2(m, U, T, nullptr, nullptr, s);
+    // FP32 P1 below 6,000 elements: us per residual without | with the launch of the traces, 1,296 elements
+    // 40 | 42, 4,374 with boundary faces 40 | 44, 6,000 44 | 44
+    const bool rows_only = sizeof(Real) == 4 && m->p == 1 && m->host.ne < 6000;
+    cudaError_t e = rows_only ? cudaSuccess : launch_traces2(m, U, T, nullptr, nullptr, s);
     if (e != cudaSuccess) return e;
     NSArgs<Real> a;
     a.U = static_cast<const Real*>(U);
@@ -434,10 +468,12 @@ cudaError_t ns_dispatch(dg_mesh* m, const void* U, void* T, void* Z, void* HB, v
     a.mu = (Real)mu;
     a.gamma = (Real)m->gamma;
     a.kappa = (Real)(mu * m->gamma / ((m->gamma - 1.0) * prandtl));
+    if constexpr (sizeof(Real) == 4)
+        if (rows_only) return ns_launch<Real, 1, false>(a, s);
     switch (m->p) {
-        case 1: return ns_launch<Real, 1>(a, s);
-        case 2: return ns_launch<Real, 2>(a, s);
-        default: return ns_launch<Real, 3>(a, s);
+        case 1: return ns_launch<Real, 1, true>(a, s);
+        case 2: return ns_launch<Real, 2, true>(a, s);
+        default: return ns_launch<Real, 3, true>(a, s);
     }
 }
 }  // namespace

@@ -4,9 +4,8 @@
 // own viscous terms and face fluxes (k_ns_visc), the neighbour's half of the central flux (k_ns_lift);
 // the equations and boundary states are those of kernels_ns.cu.  The float-float state shows the
 // rounding of an FP32 viscous residual (two FP32 evaluations in different orders move a step's state by
-// 3e-9), so these meshes keep the order of summation, and the values, they have always had; FP64
-// meshes take the factored passes of kernels_ns.cu, and so do FP32 meshes but small P1 ones, where three
-// launches are faster than four (capi.cpp has the rule).
+// 3e-9), so these meshes keep the order of summation, and the values, they have always had; FP64 and
+// FP32 meshes take the factored passes of kernels_ns.cu (FP32 without room for their trace buffer: these).
 #include <algorithm>
 
 #include "dg_internal.h"

@@ -408,6 +408,34 @@ __device__ __forceinline__ void traces(const Real* c, Store store) {
     }
 }
 
+// the trace at the points of face F alone, with the sums of traces()
+template <typename Real, int P, int F>
+__device__ __forceinline__ void face_trace(const Real* c, Real* u) {
+    constexpr auto& T = kT<P>;
+    Real a[T.NF];
+#pragma unroll
+    for (int m = 0; m < T.NF; ++m) {
+        if constexpr (F < 2) {
+            Real e = 0, o = 0;
+#pragma unroll
+            for (int j = T.NB - 1; j >= 0; --j) axpy(T.odd[j] ? o : e, T.E[1][m][j], c[j]);
+            a[m] = F == 0 ? e - o : e + o;
+        } else {
+            a[m] = 0;
+#pragma unroll
+            for (int j = T.NB - 1; j >= 0; --j) axpy(a[m], T.E[F][m][j], c[j]);
+        }
+    }
+    face_values<Real, P>(a, u);
+}
+template <typename Real, int P>
+__device__ __forceinline__ void face_trace(int f, const Real* c, Real* u) {
+    if (f == 0) face_trace<Real, P, 0>(c, u);
+    else if (f == 1) face_trace<Real, P, 1>(c, u);
+    else if (f == 2) face_trace<Real, P, 2>(c, u);
+    else face_trace<Real, P, 3>(c, u);
+}
+
 // r[j] += sum_f sum_q wf_q h_f(q) phi_j on face f; load(f, h) fills a face's NQF values and returns
 // a factor of the face, which multiplies its moments
 template <typename Real, int P, typename Load>
