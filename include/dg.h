@@ -257,8 +257,7 @@ dg_status dg_boundary_flux(dg_mesh* mesh, const double* U, int stage, double out
  * derivative of the branch taken, ties to the interior side).  U, lambda,
  * out: device FP64 [ne][5][Nb] in caller order.  The first call allocates the
  * adjoint's work buffers, owned by the mesh: six of the state's size, and two of
- * 20 Nqf values per element in FP64 and, with room to spare, on larger FP32
- * meshes.  An FP64 mesh without room for the second of these works in the one
+ * 20 Nqf values per element (FP32: with room to spare).  An FP64 mesh without room for the second of these works in the one
  * of its RK steps: the call then waits for the device before it begins and for
  * the stream before it returns. */
 dg_status dg_residual_vjp(dg_mesh* mesh, const double* U, const double* lambda, double* out, void* stream);
